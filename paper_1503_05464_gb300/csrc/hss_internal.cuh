@@ -205,7 +205,6 @@ Err launch_sample(const T* A, int64_t n, int64_t lda, const T* R, int64_t ldr,
                   int64_t c0, int64_t c1, T* Sr, T* Sc, int64_t lds,
                   const int32_t* leaf_of, int mode, SampleScratch* scratch,
                   cudaStream_t s, float* ms_out);
-size_t sample_scratch_bytes(int64_t n, int64_t ncols, int mode, bool f64);
 // Scratch bytes launch_sample needs for this call (the kernel it picks
 // depends on the mode, A's alignment and lda; the tensor-core kernel's need
 // on the device's cluster count).

@@ -1,0 +1,54 @@
+"""GPU kernels at the sizes where their splits can go wrong, against plain
+FP64 arithmetic (numpy / torch)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.fixture(scope="module")
+def P():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1503_05464_gb300 as P
+    return P
+
+
+# one row; less than a tile; one past a panel and a tile, rows not 16-byte
+# aligned; 96 columns (32-column chunks) at an odd offset; many chunks (more
+# column chunks than the even split over the SMs handles in one wave); an
+# uneven leaf that crosses tile boundaries
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("n,pad,c0,c1,starts", [
+    (1, 0, 0, 1, None),
+    (31, 5, 0, 3, [0, 31]),
+    (129, 0, 0, 64, [0, 64, 129]),
+    (193, 1, 0, 33, [0, 1, 100, 193]),
+    (641, 3, 5, 101, [0, 320, 321, 641]),
+    (400, 0, 0, 700, [0, 130, 390, 400]),
+    (2100, 0, 0, 40, [0, 700, 1400, 2100]),
+])
+def test_simt_sampling_at_tile_edges(P, dtype, n, pad, c0, c1, starts):
+    g = torch.Generator(device=DEV)
+    g.manual_seed(n)
+    A = torch.randn((n, n + pad), generator=g, device=DEV, dtype=torch.float64).to(dtype)[:, :n]
+    R = torch.randn((n, c1), generator=g, device=DEV, dtype=torch.float64).to(dtype)
+    Sr = torch.full((n, c1), 7.0, dtype=dtype, device=DEV)
+    Sc = torch.full((n, c1), 7.0, dtype=dtype, device=DEV)
+    P.hss_sample(A, R, c0, c1, Sr, Sc, leaf_starts=starts)
+    only = torch.full((n, c1), 7.0, dtype=dtype, device=DEV)
+    P.hss_sample(A, R, c0, c1, only, None, leaf_starts=starts)
+    A64 = A.double().clone()
+    for a, b in zip(starts or [], (starts or [])[1:]):
+        A64[a:b, a:b] = 0.0
+    X = R[:, c0:c1].double()
+    # a length-n dot product: n roundings of |A||R|; 4 covers the compensation
+    u = 2.0 ** -24 if dtype == torch.float32 else 2.0 ** -53
+    for got, M in ((Sr, A64), (Sc, A64.T)):
+        bound = 4 * n * u * (M.abs() @ X.abs())
+        assert torch.all((got[:, c0:c1].double() - M @ X).abs() <= bound)
+        assert torch.all(got[:, :c0] == 7.0)
+    assert torch.equal(only, Sr)
