@@ -150,6 +150,53 @@ Err upload_async(void* dst, const void* src, size_t bytes, cudaStream_t s) {
   return ok();
 }
 
+Err upload_kept(void** dst, const std::vector<std::pair<const void*, size_t>>& parts) {
+  *dst = nullptr;
+  // a capture of the caller's may be under way on this thread: this work is
+  // not part of it
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  HSS_CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode));
+  static std::mutex mu;
+  static cudaStream_t streams[64] = {};
+  Err e;
+  int dev = 0;
+  cudaStream_t s = nullptr;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+    cudaGetLastError();
+    e = fail(HSS_ERR_CUDA, "upload_kept: device");
+  } else {
+    std::lock_guard<std::mutex> lock(mu);
+    if (!streams[dev] &&
+        cudaStreamCreateWithFlags(&streams[dev], cudaStreamNonBlocking) != cudaSuccess) {
+      cudaGetLastError();
+      e = fail(HSS_ERR_CUDA, "upload_kept: stream");
+    }
+    s = streams[dev];
+  }
+  if (e.st == HSS_OK) {
+    size_t bytes = 0, off = 0;
+    for (auto& p : parts) bytes += p.second;
+    e = dalloc(dst, std::max<size_t>(bytes, 1), s);
+    cudaError_t ce = cudaSuccess;
+    for (auto& p : parts) {
+      if (e.st != HSS_OK || ce != cudaSuccess) break;
+      if (p.second)
+        ce = cudaMemcpyAsync(static_cast<char*>(*dst) + off, p.first, p.second,
+                             cudaMemcpyHostToDevice, s);
+      off += p.second;
+    }
+    const cudaError_t cs = cudaStreamSynchronize(s);
+    if (e.st == HSS_OK && (ce != cudaSuccess || cs != cudaSuccess)) {
+      cudaGetLastError();
+      dfree(*dst, s);
+      *dst = nullptr;
+      e = fail(HSS_ERR_CUDA, "upload_kept: copy");
+    }
+  }
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  return e;
+}
+
 }  // namespace hss
 
 using namespace hss;

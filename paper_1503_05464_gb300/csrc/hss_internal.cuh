@@ -56,6 +56,11 @@ void dfree(void* p, cudaStream_t s);
 // pinned block of the calling thread, which the function returns at once.
 Err upload_async(void* dst, const void* src, size_t bytes, cudaStream_t s);
 
+// A device copy of host tables (one after the other) that outlives the call,
+// complete when the function returns (it uses a stream of its own, so the
+// caller's stream is neither waited for nor captured into).  Freed with dfree.
+Err upload_kept(void** dst, const std::vector<std::pair<const void*, size_t>>& parts);
+
 template <typename T>
 inline Err dalloc_t(T** p, size_t count, cudaStream_t s) {
   return dalloc(reinterpret_cast<void**>(p), count * sizeof(T), s);

@@ -129,9 +129,14 @@ void fill_info(hss_s* h) {
 }
 
 // ------------------------------------------------------------ Algorithm 2
+// (above it the task kernel would read each matrix entry once for 8 columns)
+constexpr int MATVEC_TASKS_MAX = 32;
 template <typename T>
 static Err matvec_impl(hss_s* h, const T* X, int64_t ldx, int nrhs, T* B, int64_t ldb,
                        cudaStream_t s) {
+  // few right-hand sides: one launch of small tasks; many: the level products
+  // on 64 x 64 tiles, which read a matrix entry once for 64 columns
+  if (nrhs <= MATVEC_TASKS_MAX) return matvec_tasks<T>(h, X, ldx, nrhs, B, ldb, s);
   const Tree& tr = h->tree;
   const int nn = (int)tr.nodes.size();
   if (nn == 1) {   // H = D

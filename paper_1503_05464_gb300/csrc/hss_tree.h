@@ -3,6 +3,8 @@
 
 #include "hss_internal.cuh"
 
+#include <mutex>
+
 struct hss_s;
 
 namespace hss {
@@ -132,6 +134,10 @@ struct DownBigWork {
 };
 void fill_info(hss_s* h);
 
+// H X for few right-hand sides in one launch (hss_matvec.cu)
+template <typename T>
+Err matvec_tasks(hss_s* h, const T* X, int64_t ldx, int nrhs, T* B, int64_t ldb, cudaStream_t s);
+
 }  // namespace hss
 
 // Handle behind hss_t: owns every device buffer of the compressed form.
@@ -148,12 +154,21 @@ struct hss_s {
   hss::UlvFactors ulv;
   hss::Arena store{(size_t)16 << 20};   // generators: D, B, E, permutations, skeletons
   cudaStream_t stream = nullptr;
+  // tables kept with the handle, built at their first use (plan_mu: calls on
+  // one handle may come from several threads); they hold pointers into
+  // `store` and sizes, never a caller's buffer
+  std::mutex plan_mu;
+  void* mv_tasks = nullptr;   // hss_matvec.cu: descriptions, then (at mv_off) the tasks
+  size_t mv_off = 0;
+  int mv_ntasks = 0;
+  int64_t mv_rows = 0;
   // The caller's stream may be gone by now: drain the device, then free on
   // the legacy stream.
   ~hss_s() {
     cudaDeviceSynchronize();
     ulv.release(nullptr);
     hss::dfree(tree.iota_dev, nullptr);
+    hss::dfree(mv_tasks, nullptr);
     store.release(nullptr);
     cudaDeviceSynchronize();
   }

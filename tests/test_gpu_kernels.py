@@ -52,3 +52,43 @@ def test_simt_sampling_at_tile_edges(P, dtype, n, pad, c0, c1, starts):
         assert torch.all((got[:, c0:c1].double() - M @ X).abs() <= bound)
         assert torch.all(got[:, :c0] == 7.0)
     assert torch.equal(only, Sr)
+
+
+# ranks on both sides of the 16-row tasks and of the 64-index stages, leaves
+# at several depths, 1 to 33 columns (33: the level products)
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("n,leaf,rank,comb", [(300, 64, 7, False), (1030, 100, 17, False),
+                                              (900, 150, 70, False), (500, 40, 16, True)])
+def test_matvec_tasks_match_dense(P, dtype, n, leaf, rank, comb):
+    import workloads as W
+    A = torch.tensor(W.random_hss(n, leaf, rank, seed=n, diag_shift=20.0)[0], device=DEV).to(dtype)
+    if comb:
+        A = torch.tensor(W.toeplitz_inv_distance(n).numpy(), device=DEV).to(dtype)
+    f64 = dtype == torch.float64
+    tree = W.comb_tree_splits(n, leaf) if comb else None
+    h = P.hss_compress(A, leaf_size=leaf, rtol=1e-11 if f64 else 1e-5, d0=rank + 20, d_step=32,
+                       seed=3, tree=tree)
+    g = torch.Generator(device=DEV).manual_seed(n)
+    X = torch.randn(n, 33, dtype=torch.float64, device=DEV, generator=g).to(dtype)
+    for k in (1, 3, 4, 9, 32, 33):
+        Xs = torch.empty((n, k + 2), dtype=dtype, device=DEV)[:, :k].copy_(X[:, :k])   # ldx > nrhs
+        Y = P.hss_matvec(h, Xs)
+        ref = A.double() @ X[:, :k].double()
+        err = float(torch.linalg.norm(Y.double() - ref) / torch.linalg.norm(ref))
+        assert err <= (1e-9 if f64 else 1e-4), (k, err)
+        assert torch.equal(P.hss_matvec(h, Xs), Y)
+
+
+def test_matvec_of_nan_finishes(P):
+    """An all-ones NaN (the work buffer's not-yet-written pattern) in x."""
+    import time
+    import workloads as W
+    A = torch.as_tensor(W.toeplitz_inv_distance(1000), device=DEV)
+    h = P.hss_compress(A, leaf_size=100)
+    x = torch.ones(1000, dtype=torch.float64, device=DEV)
+    x[::50] = torch.full((20,), -1, dtype=torch.int64, device=DEV).view(torch.float64)
+    t = time.perf_counter()
+    y = P.hss_matvec(h, x)
+    torch.cuda.synchronize()
+    assert time.perf_counter() - t < 1.0      # a poll gives up after about four seconds
+    assert bool(torch.isnan(y).all())
