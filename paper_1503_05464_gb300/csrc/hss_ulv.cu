@@ -21,7 +21,8 @@ using namespace hss;
 
 namespace hss {
 
-size_t ulv_big_min_m();
+size_t ulv_big_min_m();          // solve
+size_t ulv_factor_big_min_m();   // factorization
 Err ulv_factor_big_multi(const std::vector<std::pair<hss_s*, int>>& items,
                          const std::vector<int32_t*>& status, cudaStream_t s);
 Err ulv_solve_up_big_multi(const std::vector<UpBigWork>& work, cudaStream_t s);
@@ -773,7 +774,7 @@ void factor_many(int count, hss_t* hs, cudaStream_t s, hss_status* st) {
       const int depth = h->tree.maxdepth - r;
       if (depth < 0) continue;
       for (int id : h->tree.levels[depth]) {
-        if ((size_t)h->ulv.nodes[id].m >= ulv_big_min_m()) {
+        if ((size_t)h->ulv.nodes[id].m >= ulv_factor_big_min_m()) {
           big.push_back({h, id});
           big_status.push_back(status + q);
         } else {

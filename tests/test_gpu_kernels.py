@@ -92,3 +92,25 @@ def test_matvec_of_nan_finishes(P):
     torch.cuda.synchronize()
     assert time.perf_counter() - t < 1.0      # a poll gives up after about four seconds
     assert bool(torch.isnan(y).all())
+
+
+# node orders on both sides of the per-node / blocked line (64 rows) and of
+# the panels' cluster sizes (160, 320, 640 rows), partial last panels; the
+# root's LU has to pivot (no diagonal shift)
+@pytest.mark.parametrize("n,leaf,rank", [(260, 65, 31), (280, 70, 33), (640, 161, 75),
+                                         (1300, 325, 130), (1400, 350, 321)])
+def test_ulv_factor_solve_at_panel_edges(P, n, leaf, rank):
+    import workloads as W
+    A = W.random_hss(n, leaf, rank, seed=n)[0]
+    h = P.hss_compress(torch.tensor(A, device=DEV), leaf_size=leaf, rtol=1e-13, d0=rank + 20,
+                       d_step=32, seed=5)
+    P.hss_factor(h)
+    g = torch.Generator(device=DEV).manual_seed(n)
+    b = torch.randn(n, 5, dtype=torch.float64, device=DEV, generator=g)
+    x = P.hss_solve(h, b)
+    # normwise backward error against the compressed form itself: 50 n u covers
+    # the LQ and LU with a growth factor of order ten
+    res = float(torch.linalg.norm(P.hss_matvec(h, x) - b))
+    assert res <= 50 * n * 2.0 ** -53 * float(np.linalg.norm(A)) * float(torch.linalg.norm(x))
+    P.hss_factor(h)
+    assert torch.equal(P.hss_solve(h, b), x)
