@@ -78,8 +78,10 @@ struct UlvNode {
   double* Dtil = nullptr;   // k x k
   double* Vtt = nullptr;    // r x kc
   double* Vtb = nullptr;    // k x kc
-  double* T = nullptr;      // large nodes: compact WY factors, ceil(r/32) blocks of 32 x 32
-  double* D = nullptr;      // working D_tau (m x m), freed after factorization
+  // for the solve, ceil(r/32) blocks of 32 x 32 each: the compact WY factors
+  // of the reflectors' panels, and the inverses of L's diagonal blocks
+  double* T = nullptr;
+  double* Li = nullptr;
 };
 
 struct UlvFactors {
@@ -88,11 +90,28 @@ struct UlvFactors {
   double* root_lu = nullptr;   // m0 x m0
   int32_t* root_piv = nullptr; // m0
   int root_m = 0;
+  // for the solve: inverses of the LU's diagonal blocks (unit lower, upper;
+  // 32 x 32 each) and the interchanges as one permutation
+  double* root_li = nullptr;
+  double* root_ui = nullptr;
+  int32_t* root_perm = nullptr;
   void* block = nullptr;       // one allocation holding every factor
   size_t bytes = 0;
+  // the solve's task table (hss_solve.cu), built at the first solve: the
+  // descriptions and (at plan_off) the tasks on the device; the tasks and
+  // the phases they fall into; rows of a solve's work buffer
+  void* plan = nullptr;
+  size_t plan_off = 0;
+  std::vector<int2> plan_tasks;
+  std::vector<int> plan_phases;
+  int64_t plan_rows = 0;
   void release(cudaStream_t s) {
     dfree(block, s);
     block = nullptr;
+    dfree(plan, s);
+    plan = nullptr;
+    plan_tasks.clear();
+    plan_phases.clear();
     nodes.clear();
     root_lu = nullptr;
     root_piv = nullptr;
@@ -102,36 +121,6 @@ struct UlvFactors {
 
 Err finalize_generators(hss_s* h, cudaStream_t s);
 
-// per-node buffers of a solve (all FP64, nrhs columns): b (m), btb (k),
-// y (r), z (kc), x (m rows)
-struct UlvBufs {
-  double *b = nullptr, *btb = nullptr, *y = nullptr, *z = nullptr, *x = nullptr;
-};
-// one large child of the downward sweep and its part of the parent's x
-struct DownBig {
-  int child;
-  const double* xp;
-};
-// one handle's share of a level of the blocked (large-node) solve: the
-// upward sweep's nodes `ids`, or the downward sweep's large children `kids`
-struct UpBigWork {
-  hss_s* h;
-  std::vector<int> ids;
-  const std::vector<UlvBufs>* bufs;
-  const void* B;
-  int64_t ldb;
-  int nr;
-  hss_status* status;
-};
-struct DownBigWork {
-  hss_s* h;
-  std::vector<DownBig> kids;
-  const std::vector<UlvBufs>* bufs;
-  int nr;
-  void* X;
-  int64_t ldx;
-  hss_status* status;
-};
 void fill_info(hss_s* h);
 
 // H X for few right-hand sides in one launch (hss_matvec.cu)

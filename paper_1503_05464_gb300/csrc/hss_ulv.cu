@@ -1,16 +1,18 @@
-// ULV-like factorization (Algorithm 3) and solution (Algorithm 4, Appendix A)
-// of a compressed HSS form, in FP64 whatever the input precision.
+// ULV-like factorization (Algorithm 3) of a compressed HSS form, in FP64
+// whatever the input precision.
 //
-// Factorization, one CTA per node, level by level (deepest first):
+// One CTA per node, level by level (deepest first); nodes of 64 rows or more
+// go through hss_ulv_big.cu instead:
 //   D_tau  = A(I,I) at a leaf, [Dtil_1, B12 Vtb_2^T; B21 Vtb_1^T, Dtil_2] above;
 //   Vhat   = V at a leaf, diag(Vtb_1, Vtb_2) V above;
 //   W      = Omega D_tau with Omega = [-E I; I 0] Pi^T (Omega U = [0; I]);
 //   LQ of the top r = m - k rows of W by Householder reflectors applied from
 //   the right to every row of W, so W_t Q^T = [L 0] and W_b Q^T = [W_b Q_t^T,
 //   Dtil];  Vtilde = Q Vhat.   Root: LU with partial pivoting of D_0.
-// Solve: upward sweep b_tau -> btilde = Omega b -> y = L^{-1} btilde_t,
-// z = Vtt^T y (+ V^T [z_1; z_2]); root LU solve; downward sweep
-// x_child = Q_child^T [y_child; x_parent part].
+// At the end one launch forms what the solve (hss_solve.cu) multiplies by
+// instead of substituting: the inverses of the 32 x 32 diagonal blocks of L
+// and of the root's LU, the compact WY factors of the small nodes, and the
+// root's interchanges as a permutation.
 #include "hss_internal.cuh"
 #include "hss_tree.h"
 
@@ -21,12 +23,9 @@ using namespace hss;
 
 namespace hss {
 
-size_t ulv_big_min_m();          // solve
-size_t ulv_factor_big_min_m();   // factorization
+size_t ulv_factor_big_min_m();
 Err ulv_factor_big_multi(const std::vector<std::pair<hss_s*, int>>& items,
                          const std::vector<int32_t*>& status, cudaStream_t s);
-Err ulv_solve_up_big_multi(const std::vector<UpBigWork>& work, cudaStream_t s);
-Err ulv_solve_down_big_multi(const std::vector<DownBigWork>& work, cudaStream_t s);
 
 namespace {
 
@@ -52,107 +51,6 @@ __device__ double block_sum(double v, double* red) {
 
 __device__ __forceinline__ double ld_any(const void* p, int64_t i, int f64) {
   return f64 ? reinterpret_cast<const double*>(p)[i] : (double)reinterpret_cast<const float*>(p)[i];
-}
-
-// The solve kernels keep one right-hand side per warp in shared memory
-// (U_MAXM values: the small-node path takes nodes of fewer than 320 rows)
-// and stream the rows of their triangular factors or reflectors through
-// shared memory U_RB rows at a time, loaded by the whole block with
-// independent coalesced loads.  Each row's dot product is split over the
-// lanes (lane q takes the entries q mod 32) and summed by a butterfly, so the
-// result of a column depends neither on nrhs nor on what shares the launch.
-constexpr int U_MAXM = 320, U_RB = 8;
-
-struct SolveSmem {
-  double rows[U_RB][U_MAXM];   // rows [i0, i0 + U_RB) of the streamed matrix
-  double col[U_WARPS][U_MAXM]; // warp w's right-hand side
-};
-
-// rows[t][q] = A[(i0 + t) * ld + q] for t < i1 - i0, q0 <= q < q1; whole block
-__device__ __forceinline__ void stage_rows(SolveSmem& sm, const double* A, int64_t ld, int i0,
-                                           int i1, int q0, int q1) {
-  const int w = q1 - q0;
-  for (int e = threadIdx.x; e < (i1 - i0) * w; e += U_THREADS) {
-    const int t = e / w, q = q0 + (e - t * w);
-    sm.rows[t][q] = A[(int64_t)(i0 + t) * ld + q];
-  }
-}
-
-// Sums p[0..7] over the 32 lanes; lanes u and u + 8k return the sum of p[u].
-__device__ __forceinline__ double reduce_scatter8(double (&p)[U_RB]) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int h = U_RB / 2; h >= 1; h >>= 1) {
-    const bool hi = (lane & h) != 0;
-#pragma unroll
-    for (int k = 0; k < h; ++k) {
-      const double mine = hi ? p[h + k] : p[k];
-      const double oth = hi ? p[k] : p[h + k];
-      p[k] = mine + __shfl_xor_sync(0xffffffffu, oth, h);
-    }
-  }
-  p[0] += __shfl_xor_sync(0xffffffffu, p[0], 8);
-  p[0] += __shfl_xor_sync(0xffffffffu, p[0], 16);
-  return p[0];
-}
-
-// x = T^{-1} x on a warp's column x[0..m) with T triangular (row-major, ld):
-// lower (unit diagonal or not, rows in increasing order) or upper (rows in
-// decreasing order).  Chunks of U_RB rows: the terms of the rows already
-// solved are split over the lanes (U_RB sums per lane) and reduce-scattered,
-// so that lane u holds row u of the chunk; the chunk's diagonal block is then
-// solved by a column sweep (lane t's value is final at step t, times the
-// reciprocal of the diagonal, and is broadcast to the later rows).  Every
-// warp of the block calls it (the staging is block-wide); `active` says
-// whether this warp holds a column.
-__device__ void warp_tri_solve(SolveSmem& sm, double* x, const double* T, int64_t ld, int m,
-                               bool upper, bool unit, bool active) {
-  const int lane = threadIdx.x & 31;
-  const int nch = (m + U_RB - 1) / U_RB;
-  for (int ch = 0; ch < nch; ++ch) {
-    const int i0 = upper ? max(0, m - (ch + 1) * U_RB) : ch * U_RB;
-    const int i1 = upper ? m - ch * U_RB : min(m, i0 + U_RB);
-    const int nb = i1 - i0;
-    __syncthreads();
-    if (upper) stage_rows(sm, T, ld, i0, i1, i0, m);
-    else stage_rows(sm, T, ld, i0, i1, 0, i1);
-    __syncthreads();
-    if (!active) continue;
-    double p[U_RB];
-#pragma unroll
-    for (int t = 0; t < U_RB; ++t) p[t] = 0.0;
-    const int ja = upper ? i1 : 0, jb = upper ? m : i0;
-    for (int j = ja + lane; j < jb; j += 32) {
-      const double xj = x[j];
-#pragma unroll
-      for (int t = 0; t < U_RB; ++t)
-        if (t < nb) p[t] = fma(sm.rows[t][j], xj, p[t]);
-    }
-    const int u = lane & (U_RB - 1);
-    const double sum = reduce_scatter8(p);
-    double v = 0.0, rd = 1.0;
-    if (u < nb) {
-      v = x[i0 + u] - sum;
-      if (!unit) rd = 1.0 / sm.rows[u][i0 + u];
-    }
-    double xf = 0.0;
-    if (!upper) {
-      for (int t = 0; t < nb; ++t) {
-        const double xt = __shfl_sync(0xffffffffu, v * rd, t);
-        if (u == t) xf = xt;
-        if (u > t && u < nb) v = fma(-sm.rows[u][i0 + t], xt, v);
-      }
-    } else {
-      for (int t = nb - 1; t >= 0; --t) {
-        const double xt = __shfl_sync(0xffffffffu, v * rd, t);
-        if (u == t) xf = xt;
-        if (u < t) v = fma(-sm.rows[u][i0 + t], xt, v);
-      }
-    }
-    __syncwarp();
-    if (lane < nb) x[i0 + lane] = xf;
-    __syncwarp();
-  }
 }
 
 struct FacItem {
@@ -383,203 +281,92 @@ __global__ void __launch_bounds__(U_THREADS) ulv_factor_kernel(const FacItem* it
   }
 }
 
-// ---------------------------------------------------------------- solve
-struct SolItem {
-  int m, k, kc, mc, leaf, root, lo, nrhs;
-  const void* Bin;   // leaf rhs rows (input dtype), ld ldb
-  int64_t ldb;
-  // children data (non-leaf)
-  const double* btb1;
-  const double* btb2;
-  const double* y1;
-  const double* y2;
-  const double* z1;
-  const double* z2;
-  const double* WbQt1;
-  const double* WbQt2;
-  int k1, k2, kc1, kc2, r1, r2;
-  const void* B12;
-  const void* B21;
-  // this node
-  const int32_t* permr;
-  const double* Er;
-  const int32_t* permc;
-  const double* Ec;
-  const double* L;
-  const double* Vtt;
-  const double* lu;
-  const int32_t* piv;
-  double* b;     // m x nrhs scratch
-  double* btb;   // k x nrhs out
-  double* y;     // r x nrhs out
-  double* z;     // kc x nrhs out
-  double* x;     // root: m x nrhs out
+// What the solve needs of a factored node besides the factors, one CTA per
+// 32 x 32 block.
+enum { UB_LOWER = 0, UB_UNIT_LOWER = 1, UB_UPPER = 2, UB_WY = 3, UB_PERM = 4 };
+struct BlockItem {
+  const double* M;    // the diagonal block (ld), or (UB_WY) the panel's reflectors
+  int64_t ld;
+  double* out;        // 32 x 32
+  const double* tau;  // UB_WY
+  const int32_t* piv; // UB_PERM: n interchanges -> the permutation perm
+  int32_t* perm;
+  int n, wid, mode;   // order of the block; UB_WY: columns of the panel
 };
 
-__global__ void __launch_bounds__(U_THREADS) ulv_solve_up_kernel(const SolItem* items, int f64) {
-  const SolItem it = items[blockIdx.x];
-  const int m = it.m, k = it.k, r = m - k, kc = it.kc, nr = it.nrhs;
-  const int tid = threadIdx.x;
-  double* b = it.b;
-  for (int64_t e = tid; e < (int64_t)m * nr; e += U_THREADS) {
-    int i = (int)(e / nr), c = (int)(e - (int64_t)i * nr);
-    double v;
-    if (it.leaf) {
-      v = ld_any(it.Bin, (int64_t)(it.lo + i) * it.ldb + c, f64);
-    } else if (i < it.k1) {
-      v = it.btb1[(int64_t)i * nr + c];
-      for (int q = 0; q < it.r1; ++q) v = fma(-it.WbQt1[(int64_t)i * it.r1 + q], it.y1[(int64_t)q * nr + c], v);
-      for (int l = 0; l < it.kc2; ++l)
-        v = fma(-ld_any(it.B12, (int64_t)i * it.kc2 + l, f64), it.z2[(int64_t)l * nr + c], v);
-    } else {
-      int ii = i - it.k1;
-      v = it.btb2[(int64_t)ii * nr + c];
-      for (int l = 0; l < it.kc1; ++l)
-        v = fma(-ld_any(it.B21, (int64_t)ii * it.kc1 + l, f64), it.z1[(int64_t)l * nr + c], v);
-      for (int q = 0; q < it.r2; ++q) v = fma(-it.WbQt2[(int64_t)ii * it.r2 + q], it.y2[(int64_t)q * nr + c], v);
-    }
-    b[e] = v;
-  }
-  __syncthreads();
-  __shared__ SolveSmem sm;
-  const int w = tid >> 5, lane = tid & 31;
-  double* xw = sm.col[w];
-  if (it.root) {   // x = U^{-1} L^{-1} P b with the root's LU (m < U_MAXM)
-    if (m > U_MAXM) return;
-    for (int c0 = 0; c0 < nr; c0 += U_WARPS) {
-      const int c = c0 + w;
-      const bool active = c < nr;
-      if (active) {
-        for (int i = lane; i < m; i += 32) xw[i] = b[(int64_t)i * nr + c];
-        __syncwarp();
-        if (lane == 0)
-          for (int i = 0; i < m; ++i) {
-            const int p = it.piv[i];
-            if (p != i) {
-              const double t = xw[i];
-              xw[i] = xw[p];
-              xw[p] = t;
-            }
-          }
-        __syncwarp();
+constexpr int UBN = 32;
+
+__global__ void __launch_bounds__(U_THREADS) ulv_blocks_kernel(const BlockItem* items) {
+  __shared__ double M[UBN][UBN + 1];
+  __shared__ double xl[UBN][UBN + 1];
+  __shared__ double sd[UBN];
+  const BlockItem it = items[blockIdx.x];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, n = it.n;
+  if (it.mode == UB_PERM) {   // row i of the permuted system is row perm[i]
+    for (int i = tid; i < n; i += U_THREADS) it.perm[i] = i;
+    __syncthreads();
+    if (tid == 0)
+      for (int i = 0; i < n; ++i) {
+        const int p = it.piv[i];
+        if (p > i && p < n) {   // (a singular root's pivots are not all written)
+          const int t = it.perm[i];
+          it.perm[i] = it.perm[p];
+          it.perm[p] = t;
+        }
       }
-      warp_tri_solve(sm, xw, it.lu, m, m, false, true, active);
-      warp_tri_solve(sm, xw, it.lu, m, m, true, false, active);
-      if (active) {
-        __syncwarp();
-        for (int i = lane; i < m; i += 32) it.x[(int64_t)i * nr + c] = xw[i];
-      }
-    }
     return;
   }
-  // btilde = Omega b: top r rows -> y (before the solve), bottom k rows -> btb
-  for (int64_t e = tid; e < (int64_t)m * nr; e += U_THREADS) {
-    int i = (int)(e / nr), c = (int)(e - (int64_t)i * nr);
-    if (i < r) {
-      double v = b[(int64_t)it.permr[k + i] * nr + c];
-      for (int l = 0; l < k; ++l) v = fma(-it.Er[(int64_t)i * k + l], b[(int64_t)it.permr[l] * nr + c], v);
-      it.y[(int64_t)i * nr + c] = v;
-    } else {
-      it.btb[(int64_t)(i - r) * nr + c] = b[(int64_t)it.permr[i - r] * nr + c];
+  const bool upper = it.mode == UB_UPPER || it.mode == UB_WY;
+  if (it.mode == UB_WY) {   // I + U D with U the strict upper triangle of V V^T, D = diag(tau)
+    if (tid < UBN) sd[tid] = tid < n ? it.tau[tid] : 0.0;
+    __syncthreads();
+    for (int e = tid; e < n * n; e += U_THREADS) {
+      const int a = e / n, b = e - a * n;
+      if (a >= b) continue;
+      double s0 = 0.0, s1 = 0.0;
+      int c = 0;
+      for (; c + 1 < it.wid; c += 2) {
+        s0 = fma(it.M[a * it.ld + c], it.M[b * it.ld + c], s0);
+        s1 = fma(it.M[a * it.ld + c + 1], it.M[b * it.ld + c + 1], s1);
+      }
+      if (c < it.wid) s0 = fma(it.M[a * it.ld + c], it.M[b * it.ld + c], s0);
+      M[a][b] = (s0 + s1) * sd[b];
     }
+  } else {
+    for (int e = tid; e < n * n; e += U_THREADS) M[e / n][e % n] = it.M[(e / n) * it.ld + e % n];
+    __syncthreads();
+    if (tid < UBN) sd[tid] = (it.mode != UB_UNIT_LOWER && tid < n) ? 1.0 / M[tid][tid] : 1.0;
   }
   __syncthreads();
-  // y = L^{-1} btilde_t
-  if (r <= U_MAXM) {
-    for (int c0 = 0; c0 < nr; c0 += U_WARPS) {
-      const int c = c0 + w;
-      const bool active = c < nr;
-      if (active) {
-        for (int i = lane; i < r; i += 32) xw[i] = it.y[(int64_t)i * nr + c];
-        __syncwarp();
-      }
-      warp_tri_solve(sm, xw, it.L, r, r, false, false, active);
-      if (active) {
-        __syncwarp();
-        for (int i = lane; i < r; i += 32) it.y[(int64_t)i * nr + c] = xw[i];
-      }
+  // the inverse by substitution on the unit matrix: lane = column, warp w
+  // keeps rows w + 8 t; row l is final at its step
+  double x[4];
+#pragma unroll
+  for (int t = 0; t < 4; ++t) x[t] = (w + 8 * t == lane) ? 1.0 : 0.0;
+  for (int q = 0; q < n; ++q) {
+    const int l = upper ? n - 1 - q : q;
+    if (w == (l & 7)) {
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        if (t == (l >> 3)) {
+          if (it.mode != UB_WY) x[t] *= sd[l];
+          xl[l][lane] = x[t];
+        }
+    }
+    __syncthreads();
+    const double xv = xl[l][lane];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const int a = w + 8 * t;
+      if (upper ? a < l : (a > l && a < n)) x[t] = fma(-M[a][l], xv, x[t]);
     }
   }
-  __syncthreads();
-  // z = Vtt^T y (+ V^T [z1; z2])
-  for (int64_t e = tid; e < (int64_t)kc * nr; e += U_THREADS) {
-    int l = (int)(e / nr), c = (int)(e - (int64_t)l * nr);
-    double v = 0.0;
-    for (int q = 0; q < r; ++q) v = fma(it.Vtt[(int64_t)q * kc + l], it.y[(int64_t)q * nr + c], v);
-    if (!it.leaf) {
-      auto zrow = [&](int row) -> double {
-        return row < it.kc1 ? it.z1[(int64_t)row * nr + c] : it.z2[(int64_t)(row - it.kc1) * nr + c];
-      };
-      v += zrow(it.permc[l]);
-      for (int q = 0; q < it.mc - kc; ++q) v = fma(it.Ec[(int64_t)q * kc + l], zrow(it.permc[kc + q]), v);
-    }
-    it.z[e] = v;
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    const int a = w + 8 * t;
+    const double v = it.mode == UB_WY ? sd[a] * x[t] : x[t];
+    it.out[a * UBN + lane] = (a < n && lane < n) ? v : 0.0;
   }
-}
-
-struct DownItem {
-  int m, r, nrhs, leaf, lo;   // child: m rows, r reflectors
-  const double* y;            // r x nrhs
-  const double* xp;           // parent part: (m - r) x nrhs
-  const double* hv;
-  const double* tau;
-  double* x;                  // m x nrhs (non-leaf child) -- or
-  void* Xout;                 // leaf child: output rows
-  int64_t ldx;
-};
-
-__global__ void __launch_bounds__(U_THREADS) ulv_solve_down_kernel(const DownItem* items, int f64) {
-  const DownItem it = items[blockIdx.x];
-  const int m = it.m, r = it.r, nr = it.nrhs;
-  if (m > U_MAXM) return;
-  __shared__ SolveSmem sm;
-  __shared__ double taus[U_RB];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double* v = sm.col[w];
-  for (int c0 = 0; c0 < nr; c0 += U_WARPS) {
-    const int c = c0 + w;
-    const bool active = c < nr;
-    if (active)
-      for (int i = lane; i < m; i += 32)
-        v[i] = i < r ? it.y[(int64_t)i * nr + c] : it.xp[(int64_t)(i - r) * nr + c];
-    // Q^T = H_0 H_1 ... H_{r-1}: reflectors r-1 down to 0, U_RB at a time
-    for (int i1 = r; i1 > 0; i1 -= U_RB) {
-      const int i0 = max(0, i1 - U_RB);
-      __syncthreads();
-      stage_rows(sm, it.hv, m, i0, i1, i0, m);
-      if (threadIdx.x < i1 - i0) taus[threadIdx.x] = it.tau[i0 + threadIdx.x];
-      __syncthreads();
-      if (!active) continue;
-      for (int i = i1 - 1; i >= i0; --i) {
-        const double* h = sm.rows[i - i0];
-        double dot = 0.0;
-        for (int q = i + lane; q < m; q += 32) dot = fma(h[q], v[q], dot);
-        dot = wsum(dot) * taus[i - i0];
-        for (int q = i + lane; q < m; q += 32) v[q] = fma(-dot, h[q], v[q]);
-        __syncwarp();
-      }
-    }
-    if (!active) continue;
-    __syncwarp();
-    for (int i = lane; i < m; i += 32) {
-      const double val = v[i];
-      if (it.leaf) {
-        const int64_t o = (int64_t)(it.lo + i) * it.ldx + c;
-        if (f64) reinterpret_cast<double*>(it.Xout)[o] = val;
-        else reinterpret_cast<float*>(it.Xout)[o] = (float)val;
-      } else {
-        it.x[(int64_t)i * nr + c] = val;
-      }
-    }
-  }
-}
-
-__global__ void copy_out_kernel(const double* x, int m, int nr, void* X, int64_t ldx, int f64) {
-  int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e >= (int64_t)m * nr) return;
-  int i = (int)(e / nr), c = (int)(e - (int64_t)i * nr);
-  if (f64) reinterpret_cast<double*>(X)[(int64_t)i * ldx + c] = x[e];
-  else reinterpret_cast<float*>(X)[(int64_t)i * ldx + c] = (float)x[e];
 }
 
 template <typename TI>
@@ -615,7 +402,8 @@ Err ulv_prepare(hss_s* h, cudaStream_t s) {
     u.m = m_of(id);
     off[id] = tot;
     if (id == 0) {
-      tot += (size_t)u.m * u.m + (u.m + 1) / 2 + 1;   // LU + pivots (int32 packed)
+      // LU, its blocks' inverses, pivots and permutation (int32 packed)
+      tot += (size_t)u.m * u.m + 2 * (size_t)((u.m + UBN - 1) / UBN) * UBN * UBN + u.m + 2;
       continue;
     }
     const NodeGen& g = h->gen[id];
@@ -624,7 +412,7 @@ Err ulv_prepare(hss_s* h, cudaStream_t s) {
     int r = u.m - u.k;
     tot += (size_t)r * u.m + r + (size_t)r * r + (size_t)u.k * r + (size_t)u.k * u.k +
            (size_t)r * u.kc + (size_t)u.k * u.kc;
-    if ((size_t)u.m >= ulv_big_min_m()) tot += (size_t)((r + 31) / 32) * 32 * 32;
+    tot += 2 * (size_t)((r + UBN - 1) / UBN) * UBN * UBN;   // T, Li
   }
   double* blk = nullptr;
   HSS_TRY(dalloc_t(&blk, std::max<size_t>(tot, 1), s));
@@ -636,7 +424,12 @@ Err ulv_prepare(hss_s* h, cudaStream_t s) {
     if (id == 0) {
       F.root_m = u.m;
       F.root_lu = p;
-      F.root_piv = reinterpret_cast<int32_t*>(p + (size_t)u.m * u.m);
+      p += (size_t)u.m * u.m;
+      const size_t nb = (size_t)((u.m + UBN - 1) / UBN) * UBN * UBN;
+      F.root_li = p;
+      F.root_ui = p + nb;
+      F.root_piv = reinterpret_cast<int32_t*>(p + 2 * nb);
+      F.root_perm = F.root_piv + u.m;
       continue;
     }
     int r = u.m - u.k;
@@ -654,7 +447,8 @@ Err ulv_prepare(hss_s* h, cudaStream_t s) {
     p += (size_t)r * u.kc;
     u.Vtb = p;
     p += (size_t)u.k * u.kc;
-    if ((size_t)u.m >= ulv_big_min_m()) u.T = p;
+    u.T = p;
+    u.Li = p + (size_t)((r + UBN - 1) / UBN) * UBN * UBN;
   }
   return ok();
 }
@@ -814,6 +608,64 @@ void factor_many(int count, hss_t* hs, cudaStream_t s, hss_status* st) {
     dfree(dev, s);
     dfree(sc, s);
   }
+  // the blocks for the solve
+  if (e.st == HSS_OK) {
+    std::vector<BlockItem> items;
+    for (int q : live) {
+      if (st[q] != HSS_OK) continue;
+      const UlvFactors& F = hs[q]->ulv;
+      const int m0 = F.root_m;
+      BlockItem it{};
+      it.mode = UB_PERM;
+      it.n = m0;
+      it.piv = F.root_piv;
+      it.perm = F.root_perm;
+      items.push_back(it);
+      for (int i0 = 0; i0 < m0; i0 += UBN) {
+        BlockItem b{};
+        b.M = F.root_lu + (size_t)i0 * m0 + i0;
+        b.ld = m0;
+        b.n = std::min(UBN, m0 - i0);
+        b.mode = UB_UNIT_LOWER;
+        b.out = F.root_li + (size_t)(i0 / UBN) * UBN * UBN;
+        items.push_back(b);
+        b.mode = UB_UPPER;
+        b.out = F.root_ui + (size_t)(i0 / UBN) * UBN * UBN;
+        items.push_back(b);
+      }
+      for (size_t id = 1; id < F.nodes.size(); ++id) {
+        const UlvNode& u = F.nodes[id];
+        const int r = u.m - u.k;
+        for (int i0 = 0; i0 < r; i0 += UBN) {
+          const size_t o = (size_t)(i0 / UBN) * UBN * UBN;
+          BlockItem b{};
+          b.M = u.L + (size_t)i0 * r + i0;
+          b.ld = r;
+          b.n = std::min(UBN, r - i0);
+          b.mode = UB_LOWER;
+          b.out = u.Li + o;
+          items.push_back(b);
+          if ((size_t)u.m >= ulv_factor_big_min_m()) continue;   // T comes with its panels
+          b.M = u.hv + (size_t)i0 * u.m + i0;
+          b.ld = u.m;
+          b.wid = u.m - i0;
+          b.tau = u.tau + i0;
+          b.mode = UB_WY;
+          b.out = u.T + o;
+          items.push_back(b);
+        }
+      }
+    }
+    if (!items.empty()) {
+      BlockItem* dev = nullptr;
+      e = upload_and_launch(items, s, &dev);
+      if (e.st == HSS_OK) {
+        ulv_blocks_kernel<<<(unsigned)items.size(), U_THREADS, 0, s>>>(dev);
+        e = check_launch("ulv_blocks_kernel");
+      }
+      dfree(dev, s);
+    }
+  }
   if (e.st) fail_all(e);
   std::vector<int32_t> hst(std::max(count, 1), 0);
   if (status) {
@@ -860,305 +712,6 @@ extern "C" hss_status hss_factor_batched(int32_t count, hss_t* hs, void* stream,
     }
   std::vector<hss_status> st(std::max(count, 1), HSS_OK);
   factor_many(count, hs, (cudaStream_t)stream, st.data());
-  hss_status first = HSS_OK;
-  for (int32_t q = 0; q < count; ++q) {
-    if (status) status[q] = st[q];
-    if (st[q] != HSS_OK && first == HSS_OK) {
-      first = st[q];
-      if (hs[q]) set_thread_error(hs[q]->err);
-    }
-  }
-  return first;
-}
-
-// ----------------------------------------------------------------- solve
-namespace hss {
-namespace {
-
-// One solve of a batch: the handle, its right-hand sides and its buffers.
-struct SolveJob {
-  hss_s* h;
-  const void* B;
-  int64_t ldb;
-  int nr;
-  void* X;
-  int64_t ldx;
-  double* buf = nullptr;
-  std::vector<size_t> ob, obt, oy, oz, ox;
-  std::vector<UlvBufs> bufs;
-  hss_status* st;
-};
-
-// per node: b (m), btb (k), y (r), z (kc), x (m) -- all x nrhs
-Err solve_buffers(SolveJob& j, cudaStream_t s) {
-  const int nn = (int)j.h->tree.nodes.size();
-  const UlvFactors& F = j.h->ulv;
-  j.ob.resize(nn);
-  j.obt.resize(nn);
-  j.oy.resize(nn);
-  j.oz.resize(nn);
-  j.ox.resize(nn);
-  size_t tot = 0;
-  for (int id = 0; id < nn; ++id) {
-    const UlvNode& u = F.nodes[id];
-    const int r = u.m - u.k;
-    j.ob[id] = tot;
-    tot += (size_t)u.m * j.nr;
-    j.obt[id] = tot;
-    tot += (size_t)u.k * j.nr;
-    j.oy[id] = tot;
-    tot += (size_t)r * j.nr;
-    j.oz[id] = tot;
-    tot += (size_t)u.kc * j.nr;
-    j.ox[id] = tot;
-    tot += (size_t)u.m * j.nr;
-  }
-  HSS_TRY(dalloc_t(&j.buf, std::max<size_t>(tot, 1), s));
-  j.bufs.resize(nn);
-  for (int id = 0; id < nn; ++id)
-    j.bufs[id] = {j.buf + j.ob[id], j.buf + j.obt[id], j.buf + j.oy[id], j.buf + j.oz[id],
-                  j.buf + j.ox[id]};
-  return ok();
-}
-
-SolItem up_item(const SolveJob& j, int id) {
-  const hss_s* h = j.h;
-  const Tree& tr = h->tree;
-  const UlvFactors& F = h->ulv;
-  const TNode& nd = tr.nodes[id];
-  const UlvNode& u = F.nodes[id];
-  const NodeGen& g = h->gen[id];
-  double* buf = j.buf;
-  SolItem it{};
-  it.m = u.m;
-  it.k = u.k;
-  it.kc = u.kc;
-  it.mc = g.mc;
-  it.leaf = nd.c1 < 0;
-  it.root = id == 0;
-  it.lo = nd.lo;
-  it.nrhs = j.nr;
-  it.Bin = j.B;
-  it.ldb = j.ldb;
-  if (!it.leaf) {
-    const UlvNode& a = F.nodes[nd.c1];
-    const UlvNode& b = F.nodes[nd.c2];
-    it.btb1 = buf + j.obt[nd.c1];
-    it.btb2 = buf + j.obt[nd.c2];
-    it.y1 = buf + j.oy[nd.c1];
-    it.y2 = buf + j.oy[nd.c2];
-    it.z1 = buf + j.oz[nd.c1];
-    it.z2 = buf + j.oz[nd.c2];
-    it.WbQt1 = a.WbQt;
-    it.WbQt2 = b.WbQt;
-    it.k1 = a.k;
-    it.k2 = b.k;
-    it.kc1 = a.kc;
-    it.kc2 = b.kc;
-    it.r1 = a.m - a.k;
-    it.r2 = b.m - b.k;
-    it.B12 = g.B12;
-    it.B21 = g.B21;
-  }
-  it.permr = g.permr;
-  it.Er = g.Er;
-  it.permc = g.permc;
-  it.Ec = g.Ec;
-  it.L = u.L;
-  it.Vtt = u.Vtt;
-  it.lu = F.root_lu;
-  it.piv = F.root_piv;
-  it.b = buf + j.ob[id];
-  it.btb = buf + j.obt[id];
-  it.y = buf + j.oy[id];
-  it.z = buf + j.oz[id];
-  it.x = buf + j.ox[id];
-  return it;
-}
-
-// Solves every job: the upward sweep takes depth maxdepth - r of every
-// handle in round r, the downward sweep depth r; the small nodes of all
-// handles share one launch per round, the large ones the blocked path's
-// launches of that round.  Per node the arithmetic is that of a single solve.
-void solve_many(std::vector<SolveJob>& jobs, cudaStream_t s) {
-  int rounds = 0;
-  const int f64 = (!jobs.empty() && jobs[0].h->dtype == HSS_F64) ? 1 : 0;
-  for (SolveJob& j : jobs) {
-    Err e = solve_buffers(j, s);
-    if (e.st) {
-      j.h->err = e.msg;
-      *j.st = e.st;
-    }
-    rounds = std::max(rounds, j.h->tree.maxdepth + 1);
-  }
-  auto is_big = [](const hss_s* h, int id) {
-    return (size_t)h->ulv.nodes[id].m >= ulv_big_min_m();
-  };
-  auto fail_all = [&](const Err& e) {
-    for (SolveJob& j : jobs)
-      if (*j.st == HSS_OK) {
-        j.h->err = e.msg;
-        *j.st = e.st;
-      }
-  };
-  Err e;
-  // a failure of a shared big-path launch fails every handle that had work in it
-  auto fail_work = [](auto& work, const Err& eb) {
-    for (auto& w : work)
-      if (*w.status == HSS_OK) {
-        w.h->err = eb.msg;
-        *w.status = eb.st;
-      }
-  };
-  for (int r = 0; r < rounds && e.st == HSS_OK; ++r) {
-    std::vector<SolItem> items;
-    std::vector<UpBigWork> bigw;
-    for (SolveJob& j : jobs) {
-      if (*j.st != HSS_OK) continue;
-      const int depth = j.h->tree.maxdepth - r;
-      if (depth < 0) continue;
-      std::vector<int> big;
-      for (int id : j.h->tree.levels[depth]) {
-        if (is_big(j.h, id)) big.push_back(id);
-        else items.push_back(up_item(j, id));
-      }
-      if (!big.empty()) bigw.push_back({j.h, big, &j.bufs, j.B, j.ldb, j.nr, j.st});
-    }
-    Err eb = ulv_solve_up_big_multi(bigw, s);
-    if (eb.st) fail_work(bigw, eb);
-    if (items.empty()) continue;
-    SolItem* dev = nullptr;
-    e = upload_and_launch(items, s, &dev);
-    if (e.st == HSS_OK) {
-      ulv_solve_up_kernel<<<(unsigned)items.size(), U_THREADS, 0, s>>>(dev, f64);
-      e = check_launch("ulv_solve_up_kernel");
-    }
-    dfree(dev, s);
-  }
-  for (SolveJob& j : jobs) {
-    if (e.st || *j.st != HSS_OK || j.h->tree.nodes.size() != 1) continue;
-    const int m = j.h->ulv.nodes[0].m;
-    const int64_t total = (int64_t)m * j.nr;
-    copy_out_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(j.buf + j.ox[0], m, j.nr,
-                                                                     j.X, j.ldx, f64);
-    e = check_launch("copy_out_kernel");
-  }
-  for (int r = 0; r < rounds && e.st == HSS_OK; ++r) {
-    std::vector<DownItem> items;
-    std::vector<DownBigWork> bigw;
-    for (SolveJob& j : jobs) {
-      if (*j.st != HSS_OK) continue;
-      const hss_s* h = j.h;
-      const Tree& tr = h->tree;
-      const UlvFactors& F = h->ulv;
-      if (r >= tr.maxdepth) continue;
-      std::vector<DownBig> bigkids;
-      for (int id : tr.levels[r]) {
-        const TNode& nd = tr.nodes[id];
-        if (nd.c1 < 0) continue;
-        const int ka = F.nodes[nd.c1].k;
-        for (int side = 0; side < 2; ++side) {
-          const int c = side ? nd.c2 : nd.c1;
-          const double* xp = j.buf + j.ox[id] + (side ? (size_t)ka * j.nr : 0);
-          if (is_big(h, c)) {
-            bigkids.push_back({c, xp});
-            continue;
-          }
-          const UlvNode& u = F.nodes[c];
-          const TNode& cn = tr.nodes[c];
-          DownItem it{};
-          it.m = u.m;
-          it.r = u.m - u.k;
-          it.nrhs = j.nr;
-          it.leaf = cn.c1 < 0;
-          it.lo = cn.lo;
-          it.y = j.buf + j.oy[c];
-          it.xp = xp;
-          it.hv = u.hv;
-          it.tau = u.tau;
-          it.x = j.buf + j.ox[c];
-          it.Xout = j.X;
-          it.ldx = j.ldx;
-          items.push_back(it);
-        }
-      }
-      if (!bigkids.empty()) bigw.push_back({j.h, bigkids, &j.bufs, j.nr, j.X, j.ldx, j.st});
-    }
-    Err eb = ulv_solve_down_big_multi(bigw, s);
-    if (eb.st) fail_work(bigw, eb);
-    if (items.empty()) continue;
-    DownItem* dev = nullptr;
-    e = upload_and_launch(items, s, &dev);
-    if (e.st == HSS_OK) {
-      ulv_solve_down_kernel<<<(unsigned)items.size(), U_THREADS, 0, s>>>(dev, f64);
-      e = check_launch("ulv_solve_down_kernel");
-    }
-    dfree(dev, s);
-  }
-  if (e.st) fail_all(e);
-  for (SolveJob& j : jobs) dfree(j.buf, s);
-}
-
-// argument checks of one solve; INVALID / STATE with the handle's message
-hss_status check_solve(hss_s* h, const void* B, int64_t ldb, int64_t nrhs, const void* X,
-                       int64_t ldx) {
-  if (!h) return HSS_ERR_INVALID;
-  if (!h->ulv.done) {
-    h->err = "hss_solve: hss_factor has not run on this handle";
-    return HSS_ERR_STATE;
-  }
-  if (!B || !X || nrhs < 0 || ldb < nrhs || ldx < nrhs || nrhs > INT32_MAX) {
-    h->err = "hss_solve: bad B, X, nrhs or leading dimension";
-    return HSS_ERR_INVALID;
-  }
-  return HSS_OK;
-}
-
-}  // namespace
-}  // namespace hss
-
-extern "C" hss_status hss_solve(hss_t h, const void* B, int64_t ldb, int64_t nrhs, void* X,
-                                int64_t ldx, void* stream) {
-  hss_status st = check_solve(h, B, ldb, nrhs, X, ldx);
-  if (st != HSS_OK || nrhs == 0) return st;
-  std::vector<SolveJob> jobs(1);
-  jobs[0].h = h;
-  jobs[0].B = B;
-  jobs[0].ldb = ldb;
-  jobs[0].nr = (int)nrhs;
-  jobs[0].X = X;
-  jobs[0].ldx = ldx;
-  jobs[0].st = &st;
-  solve_many(jobs, (cudaStream_t)stream);
-  return st;
-}
-
-extern "C" hss_status hss_solve_batched(int32_t count, hss_t* hs, const void* const* B,
-                                        const int64_t* ldb, const int64_t* nrhs,
-                                        void* const* X, const int64_t* ldx, void* stream,
-                                        hss_status* status) {
-  if (count < 0 || (count > 0 && (!hs || !B || !ldb || !nrhs || !X || !ldx)))
-    return HSS_ERR_INVALID;
-  std::vector<hss_status> st(std::max(count, 1), HSS_OK);
-  std::vector<SolveJob> jobs;
-  for (int32_t q = 0; q < count; ++q) {
-    st[q] = check_solve(hs[q], B[q], ldb[q], nrhs[q], X[q], ldx[q]);
-    if (st[q] == HSS_OK && hs[0] && hs[q]->dtype != hs[0]->dtype) {
-      hs[q]->err = "hss_solve_batched: handles of different dtypes";
-      st[q] = HSS_ERR_INVALID;
-    }
-    if (st[q] != HSS_OK || nrhs[q] == 0) continue;
-    SolveJob j;
-    j.h = hs[q];
-    j.B = B[q];
-    j.ldb = ldb[q];
-    j.nr = (int)nrhs[q];
-    j.X = X[q];
-    j.ldx = ldx[q];
-    j.st = &st[q];
-    jobs.push_back(std::move(j));
-  }
-  solve_many(jobs, (cudaStream_t)stream);
   hss_status first = HSS_OK;
   for (int32_t q = 0; q < count; ++q) {
     if (status) status[q] = st[q];

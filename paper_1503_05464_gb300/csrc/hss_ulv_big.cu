@@ -19,7 +19,7 @@
 //   root    right-looking blocked LU with partial pivoting: the panel by a
 //           cluster that splits its rows (lu_panel_kernel), the block row by
 //           the inverse of the panel's unit triangle, GEMM update of the rest.
-// The factors have the per-node kernel's layout, so the solve is unchanged.
+// The factors have the per-node kernel's layout.
 // Every launch shape that a node's sums depend on follows from the node's own
 // order, so factors do not depend on what shares the launch.
 #include "hss_internal.cuh"
@@ -732,205 +732,6 @@ __global__ void __launch_bounds__(B_THREADS) lu_u12_kernel(const LuPanel* items)
   }
 }
 
-// ------------------------------------------------------------ solve parts
-// Diagonal block of a blocked triangular solve: rows [i0, i0 + nbb) of X
-// (ld nr) against the block of the triangular matrix (ld ldl) at (i0, i0).
-struct TriItem {
-  const double* Lm;
-  int64_t ldl;
-  double* X;
-  int nr, i0, nbb, upper, unit;
-};
-
-__global__ void tri_block_kernel(const TriItem* items) {
-  __shared__ double Lb[NB * NB];
-  const TriItem it = items[blockIdx.x];
-  for (int e = threadIdx.x; e < it.nbb * it.nbb; e += blockDim.x) {
-    const int a = e / it.nbb, b = e % it.nbb;
-    Lb[a * NB + b] = it.Lm[static_cast<int64_t>(it.i0 + a) * it.ldl + it.i0 + b];
-  }
-  __syncthreads();
-  for (int c = threadIdx.x; c < it.nr; c += blockDim.x) {
-    double x[NB];
-#pragma unroll
-    for (int a = 0; a < NB; ++a)
-      x[a] = a < it.nbb ? it.X[static_cast<int64_t>(it.i0 + a) * it.nr + c] : 0.0;
-    if (!it.upper) {
-#pragma unroll
-      for (int a = 0; a < NB; ++a) {
-        if (a >= it.nbb) break;
-        double v = x[a];
-#pragma unroll
-        for (int b = 0; b < NB; ++b)
-          if (b < a) v = fma(-Lb[a * NB + b], x[b], v);
-        x[a] = it.unit ? v : v / Lb[a * NB + a];
-      }
-    } else {
-#pragma unroll
-      for (int a = NB - 1; a >= 0; --a) {
-        if (a >= it.nbb) continue;
-        double v = x[a];
-#pragma unroll
-        for (int b = 0; b < NB; ++b)
-          if (b > a && b < it.nbb) v = fma(-Lb[a * NB + b], x[b], v);
-        x[a] = it.unit ? v : v / Lb[a * NB + a];
-      }
-    }
-#pragma unroll
-    for (int a = 0; a < NB; ++a)
-      if (a < it.nbb) it.X[static_cast<int64_t>(it.i0 + a) * it.nr + c] = x[a];
-  }
-}
-
-// the root's row interchanges, in factorization order, one thread per column
-__global__ void apply_piv_kernel(double* x, const int32_t* piv, int m, int nr) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= nr) return;
-  for (int i = 0; i < m; ++i) {
-    const int p = piv[i];
-    if (p != i) {
-      const double t = x[static_cast<int64_t>(i) * nr + c];
-      x[static_cast<int64_t>(i) * nr + c] = x[static_cast<int64_t>(p) * nr + c];
-      x[static_cast<int64_t>(p) * nr + c] = t;
-    }
-  }
-}
-
-// One-launch triangular solves for few right-hand sides.  The blocked solve
-// takes two launches per NB rows and runs each diagonal block on one thread
-// per column; FP64 dependence chains on one lane are slow on this GPU.  Here
-// a block of T_THREADS takes one (matrix, column) pair, keeps the column in
-// shared memory and walks it in chunks of T_RB rows:
-//   1. the terms of the rows already solved: thread q takes the entries
-//      q mod T_THREADS of the chunk's T_RB rows (independent coalesced loads
-//      from global memory, T_RB sums per thread);
-//   2. a reduce-scatter butterfly leaves lane u of every warp with its warp's
-//      sum for row u, and warp 0 adds the warps' sums in warp order;
-//   3. warp 0 solves the chunk's diagonal block by a column sweep: lane u
-//      holds row u; at step t lane t's value is final (times the reciprocal
-//      of the diagonal), is broadcast, and the later rows subtract their
-//      multiple of it.
-// Optionally: row interchanges first (factorization order), and an upper
-// solve after the lower one with the same matrix (the root's LU).  A
-// column's arithmetic depends only on its matrix, never on nr or on what
-// shares the launch.
-constexpr int T_RB = 32, T_THREADS = 128, T_WARPS = T_THREADS / 32;
-constexpr int W_MAXM = 4096;   // the column in shared memory: 32 KiB
-constexpr int W_MAXNR = 64;
-
-struct WTrsmItem {
-  const double* T;        // m x m (ld ldt): lower triangle, then (upper) its upper triangle
-  int64_t ldt;
-  double* X;              // m x nr, ld nr, in place
-  const int32_t* piv;     // null: no interchanges
-  int m, nr, lower_unit, upper;
-};
-
-// sums p[0..31] over the 32 lanes; lane u returns the sum of p[u]
-__device__ __forceinline__ double reduce_scatter32(double (&p)[T_RB]) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int h = 16; h >= 1; h >>= 1) {
-    const bool hi = (lane & h) != 0;
-#pragma unroll
-    for (int k = 0; k < h; ++k) {
-      const double mine = hi ? p[h + k] : p[k];
-      const double oth = hi ? p[k] : p[h + k];
-      p[k] = mine + __shfl_xor_sync(0xffffffffu, oth, h);
-    }
-  }
-  return p[0];
-}
-
-__global__ void __launch_bounds__(T_THREADS)
-block_trsm_kernel(const WTrsmItem* __restrict__ items, const int2* __restrict__ map) {
-  __shared__ double x[W_MAXM];
-  __shared__ double tb[T_RB][T_RB + 1];
-  __shared__ double red[T_WARPS][T_RB];
-  const int2 tm = map[blockIdx.x];
-  const WTrsmItem it = items[tm.x];
-  const int m = it.m, nr = it.nr, c = tm.y;
-  if (m > W_MAXM) return;
-  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-  for (int i = tid; i < m; i += T_THREADS) x[i] = it.X[(int64_t)i * nr + c];
-  __syncthreads();
-  if (it.piv && tid == 0)
-    for (int i = 0; i < m; ++i) {
-      const int p = it.piv[i];
-      if (p != i) {
-        const double t = x[i];
-        x[i] = x[p];
-        x[p] = t;
-      }
-    }
-  __syncthreads();
-  for (int pass = 0; pass < (it.upper ? 2 : 1); ++pass) {
-    const bool up = pass == 1, unit = !up && it.lower_unit;
-    const int nch = (m + T_RB - 1) / T_RB;
-    for (int ch = 0; ch < nch; ++ch) {
-      // lower: chunks from the top; upper: from the bottom
-      const int i0 = up ? max(0, m - (ch + 1) * T_RB) : ch * T_RB;
-      const int i1 = up ? m - ch * T_RB : min(m, i0 + T_RB);
-      const int nb = i1 - i0;
-      for (int e = tid; e < nb * nb; e += T_THREADS) {
-        const int u = e / nb, t = e - u * nb;
-        tb[u][t] = it.T[(int64_t)(i0 + u) * it.ldt + i0 + t];
-      }
-      double p[T_RB];
-#pragma unroll
-      for (int u = 0; u < T_RB; ++u) p[u] = 0.0;
-      const int ja = up ? i1 : 0, jb = up ? m : i0;
-      for (int j = ja + tid; j < jb; j += T_THREADS) {
-        const double xj = x[j];
-        const double* col = it.T + (int64_t)i0 * it.ldt + j;
-#pragma unroll
-        for (int u = 0; u < T_RB; ++u)
-          if (u < nb) p[u] = fma(col[(int64_t)u * it.ldt], xj, p[u]);
-      }
-      red[w][lane] = reduce_scatter32(p);
-      __syncthreads();
-      if (w == 0) {
-        double v = 0.0, rd = 1.0;
-        if (lane < nb) {
-          double sum = red[0][lane];
-#pragma unroll
-          for (int q = 1; q < T_WARPS; ++q) sum += red[q][lane];
-          v = x[i0 + lane] - sum;
-          if (!unit) rd = 1.0 / tb[lane][lane];
-        }
-        double xf = 0.0;
-        if (!up) {
-          for (int t = 0; t < nb; ++t) {
-            const double xt = __shfl_sync(0xffffffffu, v * rd, t);
-            if (lane == t) xf = xt;
-            if (lane > t && lane < nb) v = fma(-tb[lane][t], xt, v);
-          }
-        } else {
-          for (int t = nb - 1; t >= 0; --t) {
-            const double xt = __shfl_sync(0xffffffffu, v * rd, t);
-            if (lane == t) xf = xt;
-            if (lane < t) v = fma(-tb[lane][t], xt, v);
-          }
-        }
-        if (lane < nb) x[i0 + lane] = xf;
-      }
-      __syncthreads();
-    }
-  }
-  for (int i = tid; i < m; i += T_THREADS) it.X[(int64_t)i * nr + c] = x[i];
-}
-
-// X[lo + i][c] = v[i][c] in the output dtype
-__global__ void store_rows_kernel(const double* v, int m, int nr, void* X, int64_t ldx, int lo,
-                                  int f64) {
-  const int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (e >= static_cast<int64_t>(m) * nr) return;
-  const int i = static_cast<int>(e / nr), c = static_cast<int>(e % nr);
-  const int64_t o = static_cast<int64_t>(lo + i) * ldx + c;
-  if (f64) reinterpret_cast<double*>(X)[o] = v[e];
-  else reinterpret_cast<float*>(X)[o] = static_cast<float>(v[e]);
-}
-
 template <typename TI>
 Err upload(const std::vector<TI>& v, cudaStream_t s, Arena& ar, TI** out) {
   HSS_TRY(ar.alloc_t(out, std::max<size_t>(v.size(), 1), s));
@@ -992,15 +793,12 @@ Err run_gemms(const std::vector<GemmItem<double>>& v, cudaStream_t s, Arena& ar)
 
 }  // namespace
 
-// Solves take the blocked path from this order on (their kernels for smaller
-// nodes keep a column in shared memory); factorizations much earlier: one CTA
-// per node spends its time on dependent FP64 operations and on one SM's two
-// multiply-adds a clock.  Factor times in ms with the line at 32 / 64 / 96 /
-// 160 rows: Toeplitz n = 2000 2.11 / 1.70 / 1.71 / 3.28, n = 80,000 12.2 /
-// 12.2 / 13.4 / 14.9, Gaussian kernel n = 20,000 13.9 / 14.0 / 14.9 / 20.3
-// (3.3, 29.3 and 48.0 with one CTA per node below 320 and the panels on one
-// CTA).
-size_t ulv_big_min_m() { return 320; }
+// Nodes of this order or more are factored here: one CTA per node spends its
+// time on dependent FP64 operations and on one SM's two multiply-adds a clock.
+// Factor times in ms with the line at 32 / 64 / 96 / 160 rows: Toeplitz
+// n = 2000 2.11 / 1.70 / 1.71 / 3.28, n = 80,000 12.2 / 12.2 / 13.4 / 14.9,
+// Gaussian kernel n = 20,000 13.9 / 14.0 / 14.9 / 20.3 (3.3, 29.3 and 48.0
+// with one CTA per node below 320 and the panels on one CTA).
 size_t ulv_factor_big_min_m() { return 64; }
 
 namespace {
@@ -1131,7 +929,6 @@ Err ulv_factor_big_multi(const std::vector<std::pair<hss_s*, int>>& items,
     x.kc = x.root ? 0 : u.kc;
     x.mc = x.root ? 0 : g.mc;
     const size_t mm = static_cast<size_t>(x.m) * x.m;
-    const int npan = (x.r + NB - 1) / NB;
     if (x.root) {
       x.Dw = F.root_lu;
       HSS_TRY(ar.alloc_t(&x.Linv, NB * NB, s));
@@ -1141,8 +938,7 @@ Err ulv_factor_big_multi(const std::vector<std::pair<hss_s*, int>>& items,
       HSS_TRY(ar.alloc_t(&x.VhT, static_cast<size_t>(x.m) * std::max(x.kc, 1), s));
       if (!x.leaf)
         HSS_TRY(ar.alloc_t(&x.Vd, static_cast<size_t>(std::max(x.mc, 1)) * std::max(x.kc, 1), s));
-      x.Tall = F.nodes[id].T;   // kept for the solve's Q^T
-      if (!x.Tall) HSS_TRY(ar.alloc_t(&x.Tall, static_cast<size_t>(std::max(npan, 1)) * NB * NB, s));
+      x.Tall = F.nodes[id].T;
     }
     N.push_back(x);
   }
@@ -1303,297 +1099,6 @@ Err ulv_factor_big_multi(const std::vector<std::pair<hss_s*, int>>& items,
       cp.push_back({x.VhT + x.r, x.m, 1, u.Vtb, x.kc, x.k, x.kc, nullptr, 0, 1});
     }
     HSS_TRY(launch_copies(cp, s, ar));
-  }
-  ar.release(s);
-  return ok();
-}
-
-namespace {
-
-// X <- tri^{-1} X for a batch of (matrix, X) pairs of order ord[i], blocked:
-// NB-row diagonal blocks, then one GEMM per block for the rest
-Err blocked_trsm(const std::vector<TriItem>& base, const std::vector<int>& ord, bool upper,
-                 cudaStream_t s, Arena& ar) {
-  int maxo = 0;
-  for (int o : ord) maxo = std::max(maxo, o);
-  const int nblk = (maxo + NB - 1) / NB;
-  for (int q = 0; q < nblk; ++q) {
-    std::vector<TriItem> tri;
-    std::vector<GemmItem<double>> gm;
-    for (size_t t = 0; t < base.size(); ++t) {
-      const int o = ord[t];
-      const int nbl = (o + NB - 1) / NB;
-      if (q >= nbl) continue;
-      const int blk = upper ? nbl - 1 - q : q;
-      const int i0 = blk * NB, nbb = std::min(NB, o - i0);
-      TriItem ti = base[t];
-      ti.i0 = i0;
-      ti.nbb = nbb;
-      tri.push_back(ti);
-      const int nr = ti.nr;
-      if (!upper && i0 + nbb < o) {
-        double* out = ti.X + static_cast<size_t>(i0 + nbb) * nr;
-        gm.push_back(gemm(out, nr, o - i0 - nbb, nr, nbb,
-                          ti.Lm + static_cast<size_t>(i0 + nbb) * ti.ldl + i0, ti.ldl, 0,
-                          ti.X + static_cast<size_t>(i0) * nr, nr, 0, out, nr, -1.0));
-      }
-      if (upper && i0 > 0) {
-        gm.push_back(gemm(ti.X, nr, i0, nr, nbb, ti.Lm + i0, ti.ldl, 0,
-                          ti.X + static_cast<size_t>(i0) * nr, nr, 0, ti.X, nr, -1.0));
-      }
-    }
-    if (tri.empty()) continue;
-    TriItem* dt = nullptr;
-    HSS_TRY(upload(tri, s, ar, &dt));
-    tri_block_kernel<<<static_cast<unsigned>(tri.size()), 64, 0, s>>>(dt);
-    HSS_TRY(check_launch("tri_block_kernel"));
-    HSS_TRY(run_gemms(gm, s, ar));
-  }
-  return ok();
-}
-
-bool warp_trsm_fits(int m, int nr) { return m <= W_MAXM && nr <= W_MAXNR; }
-
-// one launch for every item (all of them warp_trsm_fits): a block per
-// (item, column)
-Err warp_trsm(const std::vector<WTrsmItem>& items, cudaStream_t s, Arena& ar) {
-  std::vector<int2> map;
-  for (size_t q = 0; q < items.size(); ++q)
-    for (int c = 0; c < items[q].nr; ++c) map.push_back(make_int2((int)q, c));
-  if (map.empty()) return ok();
-  WTrsmItem* di = nullptr;
-  int2* dm = nullptr;
-  HSS_TRY(upload(items, s, ar, &di));
-  HSS_TRY(upload(map, s, ar, &dm));
-  block_trsm_kernel<<<(unsigned)map.size(), T_THREADS, 0, s>>>(di, dm);
-  return check_launch("block_trsm_kernel");
-}
-
-}  // namespace
-
-// Upward sweep of the solve (Algorithm 4) for the large nodes of one level of
-// every handle in `work` (each entry: one handle's nodes and buffers), all
-// handles sharing each launch; per node the operations are those of a
-// single solve.
-Err ulv_solve_up_big_multi(const std::vector<UpBigWork>& work, cudaStream_t s) {
-  bool any = false;
-  for (const UpBigWork& w : work) any = any || !w.ids.empty();
-  if (!any) return ok();
-  Arena ar{(size_t)4 << 20};
-  // b: leaf rows of B, or the children's contributions
-  {
-    std::vector<CopyItem> cp;
-    std::vector<GemmItem<double>> g1, g2;
-    for (const UpBigWork& w : work) {
-      const hss_s* h = w.h;
-      const Tree& tr = h->tree;
-      const UlvFactors& F = h->ulv;
-      const std::vector<UlvBufs>& bufs = *w.bufs;
-      const int f64 = h->dtype == HSS_F64;
-      const size_t esz = f64 ? 8 : 4;
-      const int nr = w.nr;
-      for (int id : w.ids) {
-        const TNode& nd = tr.nodes[id];
-        const UlvNode& u = F.nodes[id];
-        const UlvBufs& me = bufs[id];
-        if (nd.c1 < 0) {
-          cp.push_back({static_cast<const char*>(w.B) + static_cast<size_t>(nd.lo) * w.ldb * esz,
-                        w.ldb, f64, me.b, nr, u.m, nr, nullptr, 0, 0});
-          continue;
-        }
-        const NodeGen& g = h->gen[id];
-        const UlvNode& a = F.nodes[nd.c1];
-        const UlvNode& b = F.nodes[nd.c2];
-        const UlvBufs& ba = bufs[nd.c1];
-        const UlvBufs& bb = bufs[nd.c2];
-        const int ra = a.m - a.k, rb = b.m - b.k;
-        double* top = me.b;
-        double* bot = me.b + static_cast<size_t>(a.k) * nr;
-        g1.push_back(gemm(top, nr, a.k, nr, ra, a.WbQt, ra, 0, ba.y, nr, 0, ba.btb, nr, -1.0));
-        GemmItem<double> b21 =
-            gemm(bot, nr, b.k, nr, a.kc, nullptr, a.kc, 0, ba.z, nr, 0, bb.btb, nr, -1.0);
-        b21.M = g.B21;
-        b21.m_is_f64 = f64 ? 1 : 2;
-        g1.push_back(b21);
-        GemmItem<double> b12 =
-            gemm(top, nr, a.k, nr, b.kc, nullptr, b.kc, 0, bb.z, nr, 0, top, nr, -1.0);
-        b12.M = g.B12;
-        b12.m_is_f64 = f64 ? 1 : 2;
-        g2.push_back(b12);
-        g2.push_back(gemm(bot, nr, b.k, nr, rb, b.WbQt, rb, 0, bb.y, nr, 0, bot, nr, -1.0));
-      }
-    }
-    HSS_TRY(launch_copies(cp, s, ar));
-    HSS_TRY(run_gemms(g1, s, ar));
-    HSS_TRY(run_gemms(g2, s, ar));
-  }
-  // roots: x = U^{-1} L^{-1} P b, every root in shared launches (one launch
-  // for all roots with few columns, the blocked solve for the others)
-  {
-    std::vector<TriItem> base;
-    std::vector<int> ord;
-    std::vector<WTrsmItem> wt;
-    for (const UpBigWork& w : work) {
-      if (!(w.ids.size() == 1 && w.ids[0] == 0)) continue;
-      const UlvFactors& F = w.h->ulv;
-      const UlvBufs& me = (*w.bufs)[0];
-      const int m = F.root_m, nr = w.nr;
-      HSS_CUDA_TRY(cudaMemcpyAsync(me.x, me.b, sizeof(double) * m * nr, cudaMemcpyDeviceToDevice, s));
-      if (warp_trsm_fits(m, nr)) {
-        wt.push_back({F.root_lu, m, me.x, F.root_piv, m, nr, 1, 1});
-        continue;
-      }
-      apply_piv_kernel<<<(nr + 127) / 128, 128, 0, s>>>(me.x, F.root_piv, m, nr);
-      HSS_TRY(check_launch("apply_piv_kernel"));
-      base.push_back({F.root_lu, m, me.x, nr, 0, 0, 0, 1});
-      ord.push_back(m);
-    }
-    HSS_TRY(warp_trsm(wt, s, ar));
-    if (!base.empty()) {
-      HSS_TRY(blocked_trsm(base, ord, false, s, ar));
-      for (TriItem& t : base) {
-        t.upper = 1;
-        t.unit = 0;
-      }
-      HSS_TRY(blocked_trsm(base, ord, true, s, ar));
-    }
-  }
-  // btilde = Omega b; y = L^{-1} btilde_t; z = Vtt^T y (+ V^T [z1; z2])
-  {
-    std::vector<GemmItem<double>> gm;
-    std::vector<TriItem> base;
-    std::vector<int> ord;
-    std::vector<WTrsmItem> wt;
-    for (const UpBigWork& w : work) {
-      if (w.ids.size() == 1 && w.ids[0] == 0) continue;
-      const UlvFactors& F = w.h->ulv;
-      const int nr = w.nr;
-      for (int id : w.ids) {
-        const UlvNode& u = F.nodes[id];
-        const NodeGen& g = w.h->gen[id];
-        const UlvBufs& me = (*w.bufs)[id];
-        const int r = u.m - u.k;
-        GemmItem<double> top = gemm(me.y, nr, r, nr, u.k, g.Er, u.k, 0, me.b, nr, 0, me.b, nr, -1.0);
-        top.Z.map = g.permr;
-        top.X.map = g.permr + u.k;
-        gm.push_back(top);
-        GemmItem<double> bot = gemm(me.btb, nr, u.k, nr, 0, nullptr, 1, 0, nullptr, 1, 0, me.b, nr, 1.0);
-        bot.X.map = g.permr;
-        gm.push_back(bot);
-        if (r > 0 && warp_trsm_fits(r, nr)) {
-          wt.push_back({u.L, r, me.y, nullptr, r, nr, 0, 0});
-        } else if (r > 0) {
-          base.push_back({u.L, r, me.y, nr, 0, 0, 0, 0});
-          ord.push_back(r);
-        }
-      }
-    }
-    HSS_TRY(run_gemms(gm, s, ar));
-    HSS_TRY(warp_trsm(wt, s, ar));
-    HSS_TRY(blocked_trsm(base, ord, false, s, ar));
-  }
-  {
-    std::vector<GemmItem<double>> g1, g2;
-    for (const UpBigWork& w : work) {
-      if (w.ids.size() == 1 && w.ids[0] == 0) continue;
-      const Tree& tr = w.h->tree;
-      const UlvFactors& F = w.h->ulv;
-      const std::vector<UlvBufs>& bufs = *w.bufs;
-      const int nr = w.nr;
-      for (int id : w.ids) {
-        const TNode& nd = tr.nodes[id];
-        const UlvNode& u = F.nodes[id];
-        const NodeGen& g = w.h->gen[id];
-        const UlvBufs& me = bufs[id];
-        const int r = u.m - u.k;
-        if (u.kc == 0) continue;
-        GemmItem<double> z = gemm(me.z, nr, u.kc, nr, r, u.Vtt, u.kc, 1, me.y, nr, 0, nullptr, 0, 1.0);
-        if (nd.c1 >= 0) {
-          const UlvNode& a = F.nodes[nd.c1];
-          z.X.p0 = bufs[nd.c1].z;
-          z.X.ld0 = nr;
-          z.X.p1 = bufs[nd.c2].z;
-          z.X.ld1 = nr;
-          z.X.split = a.kc;
-          z.X.map = g.permc;
-          GemmItem<double> ez = gemm(me.z, nr, u.kc, nr, g.mc - u.kc, g.Ec, u.kc, 1, nullptr, nr,
-                                     0, me.z, nr, 1.0);
-          ez.Z.p0 = bufs[nd.c1].z;
-          ez.Z.ld0 = nr;
-          ez.Z.p1 = bufs[nd.c2].z;
-          ez.Z.ld1 = nr;
-          ez.Z.split = a.kc;
-          ez.Z.map = g.permc + u.kc;
-          g2.push_back(ez);
-        }
-        g1.push_back(z);
-      }
-    }
-    HSS_TRY(run_gemms(g1, s, ar));
-    HSS_TRY(run_gemms(g2, s, ar));
-  }
-  ar.release(s);
-  return ok();
-}
-
-// Downward sweep for the large children of one level of every handle in
-// `work`: v = [y; x_parent part], v <- Q^T v with Q^T = H_0 H_1 ... H_{r-1}
-// applied panel by panel from the last, then the leaves' rows of X.
-Err ulv_solve_down_big_multi(const std::vector<DownBigWork>& work, cudaStream_t s) {
-  struct Kid {
-    const DownBigWork* w;
-    const DownBig* d;
-    double *z1, *z2;
-  };
-  std::vector<Kid> kids;
-  for (const DownBigWork& w : work)
-    for (const DownBig& d : w.kids) kids.push_back({&w, &d, nullptr, nullptr});
-  if (kids.empty()) return ok();
-  Arena ar{(size_t)4 << 20};
-  int maxr = 0;
-  for (Kid& k : kids) {
-    const UlvNode& u = k.w->h->ulv.nodes[k.d->child];
-    const UlvBufs& me = (*k.w->bufs)[k.d->child];
-    const int r = u.m - u.k, nr = k.w->nr;
-    maxr = std::max(maxr, r);
-    HSS_CUDA_TRY(cudaMemcpyAsync(me.x, me.y, sizeof(double) * r * nr, cudaMemcpyDeviceToDevice, s));
-    HSS_CUDA_TRY(cudaMemcpyAsync(me.x + static_cast<size_t>(r) * nr, k.d->xp,
-                                 sizeof(double) * u.k * nr, cudaMemcpyDeviceToDevice, s));
-    HSS_TRY(ar.alloc_t(&k.z1, static_cast<size_t>(NB) * nr, s));
-    HSS_TRY(ar.alloc_t(&k.z2, static_cast<size_t>(NB) * nr, s));
-  }
-  const int npmax = (maxr + NB - 1) / NB;
-  for (int q = 0; q < npmax; ++q) {
-    std::vector<GemmItem<double>> g1, g2, g3;
-    for (Kid& k : kids) {
-      const UlvNode& u = k.w->h->ulv.nodes[k.d->child];
-      const UlvBufs& me = (*k.w->bufs)[k.d->child];
-      const int r = u.m - u.k, m = u.m, nr = k.w->nr;
-      const int np = (r + NB - 1) / NB;
-      if (q >= np) continue;
-      const int p = np - 1 - q;
-      const int i0 = p * NB, nbb = std::min(NB, r - i0);
-      const double* vp = u.hv + static_cast<size_t>(i0) * m + i0;
-      const double* T = u.T + static_cast<size_t>(p) * NB * NB;
-      double* v = me.x + static_cast<size_t>(i0) * nr;
-      g1.push_back(gemm(k.z1, nr, nbb, nr, m - i0, vp, m, 0, v, nr, 0, nullptr, 0, 1.0));
-      g2.push_back(gemm(k.z2, nr, nbb, nr, nbb, T, NB, 0, k.z1, nr, 0, nullptr, 0, 1.0));
-      g3.push_back(gemm(v, nr, m - i0, nr, nbb, vp, m, 1, k.z2, nr, 0, v, nr, -1.0));
-    }
-    HSS_TRY(run_gemms(g1, s, ar));
-    HSS_TRY(run_gemms(g2, s, ar));
-    HSS_TRY(run_gemms(g3, s, ar));
-  }
-  for (Kid& k : kids) {
-    const TNode& cn = k.w->h->tree.nodes[k.d->child];
-    if (cn.c1 >= 0) continue;
-    const UlvNode& u = k.w->h->ulv.nodes[k.d->child];
-    const int nr = k.w->nr;
-    const int64_t total = static_cast<int64_t>(u.m) * nr;
-    store_rows_kernel<<<static_cast<unsigned>((total + 255) / 256), 256, 0, s>>>(
-        (*k.w->bufs)[k.d->child].x, u.m, nr, k.w->X, k.w->ldx, cn.lo,
-        k.w->h->dtype == HSS_F64 ? 1 : 0);
-    HSS_TRY(check_launch("store_rows_kernel"));
   }
   ar.release(s);
   return ok();

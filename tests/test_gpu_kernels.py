@@ -114,3 +114,42 @@ def test_ulv_factor_solve_at_panel_edges(P, n, leaf, rank):
     assert res <= 50 * n * 2.0 ** -53 * float(np.linalg.norm(A)) * float(torch.linalg.norm(x))
     P.hss_factor(h)
     assert torch.equal(P.hss_solve(h, b), x)
+
+
+# one column to more than a launch's 64 (two slabs), in place, on handles with
+# 8-row tasks (nodes above 160 rows), partial blocks, rank-zero nodes and a
+# single-node tree; several handles of different widths together
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+def test_ulv_solve_tasks(P, dtype):
+    import scipy.linalg as sla
+    import workloads as W
+    mats = [(W.random_hss(900, 225, 90, seed=1, diag_shift=60.0)[0], 225, 110),
+            (W.random_hss(130, 64, 33, seed=2, diag_shift=30.0)[0], 64, 45),
+            (sla.block_diag(*[np.eye(40) * (i + 2) for i in range(5)]), 40, 16),
+            (np.random.default_rng(3).standard_normal((70, 70)) + 20 * np.eye(70), 128, 16)]
+    f64 = dtype == torch.float64
+    hs, norms = [], []
+    for A, leaf, d0 in mats:
+        At = torch.tensor(A, device=DEV).to(dtype)
+        norms.append(float(np.linalg.norm(A)))
+        hs.append(P.hss_compress(At, leaf_size=leaf, rtol=1e-12 if f64 else 1e-6, d0=d0, d_step=16, seed=4))
+        P.hss_factor(hs[-1])
+    g = torch.Generator(device=DEV).manual_seed(9)
+    Bs = []
+    for h, nA, k in zip(hs, norms, (70, 3, 1, 9)):
+        B = torch.randn(h.n, k, dtype=torch.float64, device=DEV, generator=g).to(dtype)
+        X = P.hss_solve(h, B)
+        # normwise backward error against the compressed form: FP64 as in the
+        # test above; FP32 the product's own bound (length-n FP32 sums)
+        bound = (50 * 2.0 ** -53 if f64 else 4 * 2.0 ** -24) * h.n * nA * float(torch.linalg.norm(X.double()))
+        Y = torch.cat([P.hss_matvec(h, X[:, c:c + 32].contiguous()) for c in range(0, k, 32)], 1)
+        assert float(torch.linalg.norm(Y.double() - B.double())) <= bound
+        for c in {0, k - 1}:         # a column's bits do not depend on the others
+            assert torch.equal(P.hss_solve(h, B[:, c].contiguous()), X[:, c])
+        Y = B.clone()
+        assert torch.equal(P.hss_solve(h, Y, X=Y), X)
+        Bs.append(B)
+    Xs, st = P.hss_solve_batched(hs, Bs)
+    assert st == [0] * 4
+    for h, B, X in zip(hs, Bs, Xs):
+        assert torch.equal(P.hss_solve(h, B), X)
