@@ -10,15 +10,14 @@
 // elimination step:
 //   1. before the barrier every CTA pushes its candidate (largest residual
 //      norm among its active columns, lowest index on ties) into every CTA's
-//      shared memory, with that column's exact residual: the entry at the
-//      next pivot row and the sum of squares below it (one warp, fixed
-//      summation tree);
+//      shared memory, with the Householder reflector that the candidate
+//      column would give: sigma, tau and the scale of v, from the column's
+//      exact residual (the entry at the next pivot row and the sum of squares
+//      below it in a fixed order);
 //   2. after the barrier every CTA picks the same pivot from the C local
-//      candidates and derives from the owner's pushed residual, with the same
-//      arithmetic, |R_ii|, the stopping decision against max(rtol |R_11|,
-//      atol) and the Householder reflector, while its other warps copy the
-//      pivot column from the owner -- so no CTA waits for the owner, and all
-//      agree bitwise;
+//      candidates, reads |R_ii| = sigma, takes the stopping decision against
+//      max(rtol |R_11|, atol), and copies and scales the pivot column from the
+//      owner -- so no CTA waits for the owner, and all agree bitwise;
 //   3. every CTA applies the reflector to its active columns (a team of
 //      threads per column: dot product, fixed-order reduction, update), then
 //      downdates their norms with one lane per column -- recomputing a norm
@@ -31,7 +30,7 @@
 // perm[0..k) records the pivot order, the remaining columns follow in
 // increasing index order.  The pivot columns' R entries go to a global k x k
 // buffer, and each CTA solves T = R1^{-1} R2 for the remaining columns it owns
-// (column-oriented back substitution, all threads of the CTA), writing E = T^T
+// (column-oriented back substitution by blocks of 16 rows), writing E = T^T
 // so that the generator is Pi [I; E].
 //
 // Group mode: when a launch holds a few large items (a CTA's share of one
@@ -41,7 +40,18 @@
 // bounded barrier in global memory (a counter per item); each column's
 // arithmetic is that of the cluster mode, so the bits do not depend on the
 // number of CTAs.
+//
+// What bounds it: the chain of one step.  At 16 columns or so per CTA a step
+// takes 12600 cycles (n = 20000, m 150-340): the barrier 800, the pick and the
+// pivot column 1000-1500, the columns' pass 4000-5000, the downdates 1700 and
+// the candidate with its reflector 3800 -- forming the reflector before the
+// barrier (once, not in every CTA after it), integer arg-max reductions and
+// the integer root and quotient took the IDs of that compression from 11.4 to
+// 10.2 ms; large items (n = 60000, m to 4700) are bound by the FP64 pipe in
+// the pass: the registers kept under 128, so that two CTAs fit an SM, took
+// that compression from 1451 to 1299 ms.
 #include "hss_internal.cuh"
+#include "hss_fp.cuh"
 
 #include <cooperative_groups.h>
 
@@ -71,19 +81,45 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// Doubles of a reflector buffer (it also holds 128 partial sums) and of the
+// candidate's column (later a block of the back substitution: 16 x 17 entries
+// of R1 and 4 x 32 of T)
+constexpr int ID_BS = 16;
+__host__ __device__ inline int id_vec(int d) { return d < 128 ? 128 : d; }
+__host__ __device__ inline int id_cbuf(int d) {
+  return d < ID_BS * (ID_BS + 1) + 128 ? ID_BS * (ID_BS + 1) + 128 : d;
+}
+
 // Residual norms are >= 0 and inactive columns carry -1: as 64-bit integers
 // their bit patterns order the same way (the sign bit makes -1 negative), so
 // the arg-max runs on the integer pipes instead of the narrow FP64 one.
+// Three integer reductions (high word, low word, index) take a third of the
+// time of five shuffle rounds.
 __device__ __forceinline__ void warp_argmax_bits(long long& v, int& j) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const long long ov = __shfl_xor_sync(0xffffffffu, v, o);
-    const int oj = __shfl_xor_sync(0xffffffffu, j, o);
-    if (ov > v || (ov == v && oj < j)) {
-      v = ov;
-      j = oj;
-    }
-  }
+  const int hi = static_cast<int>(v >> 32);
+  const unsigned lo = static_cast<unsigned>(v);
+  const int mh = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+  j = __reduce_min_sync(0xffffffffu, (hi == mh && lo == ml) ? j : INT_MAX);
+  v = (static_cast<long long>(mh) << 32) | ml;
+}
+
+// a / b, correctly rounded, from y = 1 / b (itself correctly rounded): two
+// residual corrections of a y (P. Markstein, "Computation of elementary
+// functions on the IBM RISC System/6000 processor", IBM J. Res. Dev. 34,
+// 1990: the second gives the rounded quotient when the first is within an
+// ulp).  Five dependent FP64 operations instead of a division's ten or so;
+// operands whose quotient or residuals could leave the normal range, and a b
+// whose significand is all ones, take the division.
+__device__ __forceinline__ double div_by(double a, double b, double y) {
+  const int ea = (__double2hiint(a) >> 20) & 0x7ff, eb = (__double2hiint(b) >> 20) & 0x7ff;
+  const bool ones = (__double_as_longlong(b) & 0xfffffffffffffll) == 0xfffffffffffffll;
+  const bool zero = (__double_as_longlong(a) & LLONG_MAX) == 0;   // a y is the quotient
+  if (!zero && (ea < 600 || ea > 1400 || eb < 700 || eb > 1300 || ones)) return a / b;
+  double q = a * y;
+  if (zero) return q;
+  q = fma(fma(-q, b, a), y, q);
+  return fma(fma(-q, b, a), y, q);
 }
 
 // Sum over the column entries c >= i of f(c) with a summation order that does
@@ -122,61 +158,82 @@ __device__ __forceinline__ double team_sum(int i, int d, int member, F f) {
 // team_sum's order.  Each entry gets the same operations, in the same order,
 // as an update pass followed by a dot-product pass, so the bits are those of
 // the two passes; the column is read and written once instead of read twice
-// and written once.
-template <int TS>
+// and written once.  Chunks of 32 rows; the inner ones carry no bounds, and a
+// column in global memory (WS false) has its next chunk on the way.
+template <int TS, bool WS>
 __device__ __forceinline__ double team_update_dot(int i, int d, int member, bool pending, double a,
                                                   const double* __restrict__ up,
                                                   const double* __restrict__ u, double* w) {
-  constexpr int NP = 32 / TS;                      // partial sums per thread
-  constexpr bool PF = TS >= 4;                     // columns in global memory: pipelined
-  // rows per chunk 32 G (G = 1: deeper chunks for large teams, 8 loads in
-  // flight per thread, measured slower)
-  constexpr int G = 1;
-  constexpr int NQ = NP * G;
+  constexpr int NP = 32 / TS;              // partial sums per thread
+  constexpr int NG = NP < 8 ? NP : 8;      // rows of a chunk in flight per thread
+  constexpr bool PF = !WS && TS >= 4;      // next chunk loaded ahead
   double acc[NP];
 #pragma unroll
   for (int q = 0; q < NP; ++q) acc[q] = 0.0;
   const int lo = pending ? i - 1 : i;
   int base = (lo / 32) * 32;
-  double x[NQ];
+  double x[PF ? NP : 1];
+  auto load = [&](int b, int q) -> double {
+    const int c = b + member + q * TS;
+    return (c >= lo && c < d) ? w[c] : 0.0;
+  };
   if constexpr (PF) {
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-      const int c = base + member + q * TS;
-      x[q] = (c >= lo && c < d) ? w[c] : 0.0;
-    }
+    for (int q = 0; q < NP; ++q) x[q] = load(base, q);
   }
-  for (; base < d; base += 32 * G) {
-    double nx[NQ];
+  for (; base < d; base += 32) {
+    double nx[PF ? NP : 1];
     if constexpr (PF) {
+      if (base + 64 <= d) {
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) {
-        const int c = base + 32 * G + member + q * TS;
-        nx[q] = c < d ? w[c] : 0.0;
+        for (int q = 0; q < NP; ++q) nx[q] = w[base + 32 + member + q * TS];
+      } else {
+#pragma unroll
+        for (int q = 0; q < NP; ++q) nx[q] = load(base + 32, q);
+      }
+    }
+    if (base >= i && base + 32 <= d) {
+#pragma unroll
+      for (int g = 0; g < NP; g += NG) {
+        double pp[NG], uu[NG], xx[NG];
+#pragma unroll
+        for (int q = 0; q < NG; ++q) {
+          const int c = base + member + (g + q) * TS;
+          pp[q] = up[c - lo];
+          uu[q] = u[c - i];
+          if constexpr (PF) xx[q] = x[g + q];
+          else xx[q] = w[c];
+        }
+#pragma unroll
+        for (int q = 0; q < NG; ++q) {
+          const int c = base + member + (g + q) * TS;
+          const double t = fma(a, pp[q], xx[q]);
+          if (pending) {
+            xx[q] = t;
+            w[c] = t;
+          }
+          acc[g + q] = fma(uu[q], xx[q], acc[g + q]);
+        }
       }
     } else {
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) {
+      for (int q = 0; q < NP; ++q) {
         const int c = base + member + q * TS;
-        x[q] = (c >= lo && c < d) ? w[c] : 0.0;
-      }
-    }
-    // entry c = base + member + q TS goes to partial q mod NP (= c mod 32
-    // within the team's rows), in increasing c
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-      const int c = base + member + q * TS;
-      if (c >= lo && c < d) {
-        if (pending) {
-          x[q] = fma(a, up[c - lo], x[q]);
-          w[c] = x[q];
+        if (c >= lo && c < d) {
+          double xq;
+          if constexpr (PF) xq = x[q];
+          else xq = w[c];
+          if (pending) {
+            xq = fma(a, up[c - lo], xq);
+            w[c] = xq;
+          }
+          if (c >= i) acc[q] = fma(u[c - i], xq, acc[q]);
         }
-        if (c >= i) acc[q % NP] = fma(u[c - i], x[q], acc[q % NP]);
       }
     }
     if constexpr (PF) {
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) x[q] = nx[q];
+      for (int q = 0; q < NP; ++q) x[q] = nx[q];
     }
   }
 #pragma unroll
@@ -190,19 +247,20 @@ __device__ __forceinline__ double team_update_dot(int i, int d, int member, bool
   return r;
 }
 
-// A CTA's pivot candidate as its peers receive it: with the column's exact
-// residual (entry alpha at the next pivot row, sum st of the squares below
-// it) every CTA can form the reflector without waiting for the column.
+// A CTA's pivot candidate as its peers receive it, with the reflector it
+// would give.
 struct alignas(16) Cand {
   long long v;    // bit pattern of its largest active residual norm (LLONG_MIN: none)
   int j;          // its global column index
   int pad;
-  double st;      // sum of x_c^2 below the next pivot row
-  double alpha;   // x at the next pivot row
+  double sigma;   // |R_ii| if it is the pivot
+  double tau;
+  double scal;    // v = x scal below the pivot row
+  double pad2;
 };
-// (v, j) and (st, alpha) are read as two 16-byte loads
-static_assert(offsetof(Cand, j) == 8 && offsetof(Cand, st) == 16 &&
-                  offsetof(Cand, alpha) == 24 && sizeof(Cand) == 32,
+// (v, j), (sigma, tau) and scal are read as 16-byte loads
+static_assert(offsetof(Cand, j) == 8 && offsetof(Cand, sigma) == 16 && offsetof(Cand, scal) == 32 &&
+                  sizeof(Cand) == 48,
               "Cand layout");
 
 // A node side spread over more CTAs than a cluster holds (a "group"): the
@@ -229,17 +287,17 @@ __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
   return v;
 }
 
-template <int TS, bool GRP, int MINB = 1>
+// WS: the columns are in shared memory, else in the global work copy
+template <int TS, bool GRP, int MINB = 1, bool WS = false>
 __global__ void __launch_bounds__(ID_THREADS, MINB)
 id_cpqr_cluster_kernel(const IdItem* __restrict__ items, int f64in,
-                       int w_in_smem, double* __restrict__ r1buf_base,
+                       double* __restrict__ r1buf_base,
                        const int64_t* __restrict__ r1off, GroupArgs ga) {
   extern __shared__ __align__(16) double smem[];
   __shared__ Cand cands[2][16];
   __shared__ long long redb[ID_WARPS];
   __shared__ int redi[ID_WARPS];
-  __shared__ double hh[4];   // this step's sigma, tau, (unused), scale
-  __shared__ int hstop;
+  __shared__ double cbeta;   // R_ii of this CTA's last candidate
   __shared__ int nrest;
   __shared__ int nact;
   __shared__ int gstop;
@@ -305,12 +363,16 @@ id_cpqr_cluster_kernel(const IdItem* __restrict__ items, int f64in,
   }
   const int mloc = (m - crank + C - 1) / C;       // columns crank, crank+C, ...
   const int mloc_max = (m + C - 1) / C;
-  // reflectors of steps i (vbuf + (i & 1) d) and i - 1: the update of a step
-  // is applied in the same pass as the next step's dot product; after the
-  // elimination the same 3 d doubles hold R1's diagonal (d) and two staged
-  // R1 columns of the back substitution (colbuf, 2 d)
-  double* vbuf = smem;                            // 3 d
-  double* nrm = vbuf + 3 * d;                     // mloc_max
+  // reflectors of steps i (vbuf + (i & 1) dv) and i - 1: the update of a step
+  // is applied in the same pass as the next step's dot product; then the
+  // candidate's column (cbuf).  The buffer of u_{i-1} also takes the partial
+  // sums of a candidate's residual, at the end of step i.  After the
+  // elimination: R1's diagonal, its reciprocals, and a block of the back
+  // substitution
+  const int dv = id_vec(d);
+  double* vbuf = smem;                            // 2 dv
+  double* cbuf = vbuf + 2 * dv;                   // id_cbuf(d)
+  double* nrm = cbuf + id_cbuf(d);                // mloc_max
   double* lim = nrm + mloc_max;                   // mloc_max: tol3z * (norm at last recompute)^2
   double* rdiag = lim + mloc_max;                 // mloc_max: R_ii of the pivot columns
   double* dprev = rdiag + mloc_max;               // mloc_max: tau (u_i . w), update pending
@@ -324,13 +386,20 @@ id_cpqr_cluster_kernel(const IdItem* __restrict__ items, int f64in,
   int* alist = pstep + ((mloc_max + 1) & ~1);
   int* apos = alist + ((mloc_max + 1) & ~1);
   int* pend = apos + ((mloc_max + 1) & ~1);       // 1: the column's update by dprev is pending
-  double* colbuf = vbuf + d;                      // 2 d, after the elimination only
   double* Wsm = reinterpret_cast<double*>(pend + ((mloc_max + 1) & ~1));
   // odd column stride in shared memory: a thread per column reads without
   // bank conflicts
   const int ldw = d | 1;
+  // (telling the compiler the address space: generic loads and stores could
+  // alias the reflectors in shared memory and wait for each other)
   auto col = [&](int jl) -> double* {
-    return w_in_smem ? Wsm + (size_t)jl * ldw : it.work + (size_t)(jl * C + crank) * d;
+    if constexpr (WS) {
+      return Wsm + (size_t)jl * ldw;
+    } else {
+      double* q = it.work + (size_t)(jl * C + crank) * d;
+      __builtin_assume(__isGlobal(q));
+      return q;
+    }
   };
   // team of TS threads per column (power of two, chosen by the launcher):
   // all 256 threads stay busy whether a CTA owns 8 columns or 500
@@ -375,64 +444,100 @@ id_cpqr_cluster_kernel(const IdItem* __restrict__ items, int f64in,
   if (!sync_all()) return;
   // each CTA's candidate (largest residual norm of its active columns, as the
   // norm's bit pattern; lowest index on ties) goes into slot s of every CTA's
-  // cands[s][crank], so the reads after the next cluster barrier are local
-  // (one warp) push the candidate (v, j) for pivot row r: its residual is
-  // computed here with the fixed summation tree, so every CTA gets the same bits
-  auto push_candidate = [&](int s, long long v, int j, int r) {
-    double st = 0.0, alpha = 0.0;
-    if (v != LLONG_MIN) {
-      const int jl = (j - crank) / C;
+  // cands[s][crank], so the reads after the next cluster barrier are local.
+  // The whole CTA brings the candidate's column up to date (its update by
+  // u = u_{r-1} may be pending) and leaves it in cbuf as well; four warps on
+  // four schedulers sum its squares below the pivot row r, and warp 0 forms
+  // the reflector (lanes 0 and 1 the two quotients in one division) and
+  // pushes.  The sum: entry c goes to partial (c / 32) mod 4 of lane c mod 32,
+  // in increasing c, then ((p0 + p1) + (p2 + p3)) and a butterfly over the
+  // lanes: a fixed order, computed by the owner alone.
+  auto push_candidate = [&](int s, long long v, int j, int r, const double* u, double* psum) {
+    const bool have = v != LLONG_MIN;
+    const int jl = have ? (j - crank) / C : 0;
+    if (have) {
       double* w = col(jl);
-      // its pending update, if any, has been applied by the whole CTA;
-      // sum of squares below row r: entry c goes to partial (c / 32) mod 4
-      // of lane c mod 32, in increasing c (four independent chains, loads
-      // four chunks ahead), then ((p0 + p1) + (p2 + p3)) and a butterfly
-      // over the lanes: a fixed order, computed by the owner alone
-      double pa[4] = {0.0, 0.0, 0.0, 0.0};
-      for (int base = ((r + 1) / 128) * 128; base < d; base += 128) {
-        double x[4];
+      const bool pd = pend[jl] != 0;
+      const double a = -dprev[jl];
+      constexpr int U = 4;
+      for (int c0 = (pd ? r - 1 : r) + tid; c0 < d; c0 += U * ID_THREADS) {
+        double x[U];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int c = base + 32 * u + lane;
-          x[u] = (c >= r + 1 && c < d) ? w[c] : 0.0;
+        for (int q = 0; q < U; ++q) x[q] = c0 + q * ID_THREADS < d ? w[c0 + q * ID_THREADS] : 0.0;
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+          const int c = c0 + q * ID_THREADS;
+          if (c >= d) continue;
+          if (pd) {
+            x[q] = fma(a, u[c - (r - 1)], x[q]);
+            w[c] = x[q];
+          }
+          cbuf[c] = x[q];
         }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) pa[u] = fma(x[u], x[u], pa[u]);
       }
-      st = (pa[0] + pa[1]) + (pa[2] + pa[3]);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) st = st + __shfl_xor_sync(0xffffffffu, st, o);
-      alpha = r < d ? w[r] : 0.0;
     }
-    if constexpr (GRP) {
-      if (lane == 0) {
-        Cand* dst = ga.cand + (static_cast<size_t>(item) * 2 + s) * C + crank;
-        dst->v = v;
-        dst->j = j;
-        dst->st = st;
-        dst->alpha = alpha;
+    __syncthreads();
+    if (warp >= 4) return;
+    if (have && tid == 0) pend[jl] = 0;
+    double pa = 0.0;
+    if (have)
+      for (int base = ((r + 1) / 128) * 128; base < d; base += 128) {
+        const int c = base + 32 * warp + lane;
+        const double x = (c >= r + 1 && c < d) ? cbuf[c] : 0.0;
+        pa = fma(x, x, pa);
       }
+    psum[32 * warp + lane] = pa;
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    if (warp != 0) return;
+    double st = (psum[lane] + psum[32 + lane]) + (psum[64 + lane] + psum[96 + lane]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) st = st + __shfl_xor_sync(0xffffffffu, st, o);
+    const double alpha = have && r < d ? cbuf[r] : 0.0;
+    const double sigma = fp_sqrt(fma(alpha, alpha, st));
+    const bool refl = st != 0.0;
+    const double beta = refl ? -copysign(sigma, alpha) : alpha;
+    double q = 0.0;
+    if (refl && lane < 2) {
+      const double num = lane == 0 ? beta - alpha : 1.0;
+      const double den = lane == 0 ? beta : alpha - beta;
+      q = fp_div(num, den);
+    }
+    const double tau = __shfl_sync(0xffffffffu, q, 0), scal = __shfl_sync(0xffffffffu, q, 1);
+    if (lane == 0) cbeta = beta;
+    Cand* dst = nullptr;
+    if constexpr (GRP) {
+      if (lane == 0) dst = ga.cand + (static_cast<size_t>(item) * 2 + s) * C + crank;
     } else if (lane < C) {
-      Cand* dst = cg::this_cluster().map_shared_rank(&cands[s][crank], lane);
+      dst = cg::this_cluster().map_shared_rank(&cands[s][crank], lane);
+    }
+    if (dst != nullptr) {
       dst->v = v;
       dst->j = j;
-      dst->st = st;
-      dst->alpha = alpha;
+      dst->sigma = sigma;
+      dst->tau = tau;
+      dst->scal = scal;
     }
   };
-  if (warp == 0) {
+  {
     long long bv = LLONG_MIN;
     int bj = INT_MAX;
-    for (int jl = lane; jl < mloc; jl += 32) {
-      const long long x = __double_as_longlong(nrm[jl]);
-      const int j = jl * C + crank;
-      if (x > bv || (x == bv && j < bj)) {
-        bv = x;
-        bj = j;
+    if (warp == 0) {
+      for (int jl = lane; jl < mloc; jl += 32) {
+        const long long x = __double_as_longlong(nrm[jl]);
+        const int j = jl * C + crank;
+        if (x > bv || (x == bv && j < bj)) {
+          bv = x;
+          bj = j;
+        }
+      }
+      warp_argmax_bits(bv, bj);
+      if (lane == 0) {
+        redb[0] = bv;
+        redi[0] = bj;
       }
     }
-    warp_argmax_bits(bv, bj);
-    push_candidate(0, bv, bj, 0);
+    __syncthreads();
+    push_candidate(0, redb[0], redi[0], 0, vbuf, vbuf + dv);
   }
 
   const int kmax = min(m, d);
@@ -440,132 +545,98 @@ id_cpqr_cluster_kernel(const IdItem* __restrict__ items, int f64in,
   // costs the same however few lanes are active)
   const int nwd = min(ID_WARPS, (mloc_max + 31) / 32);
   int k = kmax;
-  double r11 = 0.0;
+  long long thr = 0;   // bit pattern of max(rtol |R_11|, atol)
   for (int i = 0; i < kmax; ++i) {
     if (!sync_all()) return;   // candidates of step i pushed, dot products of step i-1 done
     const int slot = i & 1;
-    double* vloc = vbuf + (i & 1) * d;          // pivot column, then reflector u_i
-    const double* vprev = vbuf + ((i + 1) & 1) * d;   // u_{i-1}
+    double* vloc = vbuf + (i & 1) * dv;         // reflector u_i
+    const double* vprev = vbuf + ((i + 1) & 1) * dv;  // u_{i-1}
     // every warp reduces the C candidates (lane r <- CTA r): all threads agree
     // on the pivot without a block barrier
     long long bv = LLONG_MIN;
     int p = INT_MAX;
-    double wst = 0.0, wal = 0.0;   // the best candidate's residual (group mode)
     const Cand* gc = nullptr;
     if constexpr (GRP) {
       gc = ga.cand + (static_cast<size_t>(item) * 2 + slot) * C;
-      // every candidate (v, j and its residual st, alpha) is loaded before
-      // any is compared: one round trip to L2 for up to 320 CTAs instead of
-      // one per 32, and none more for the winner's residual
+      // every candidate (v, j) is loaded before any is compared: one round
+      // trip to L2 for up to 320 CTAs instead of one per 32
       constexpr int U = 10;
       for (int r0 = lane; r0 < C; r0 += 32 * U) {
-        long long vv[U];
-        int jj[U];
-        double ss[U], aa[U];
+        longlong2 x[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           const int r = r0 + 32 * u;
-          vv[u] = LLONG_MIN;
-          jj[u] = INT_MAX;
-          ss[u] = aa[u] = 0.0;
-          if (r < C) {
-            const longlong2 x = __ldcg(reinterpret_cast<const longlong2*>(&gc[r]));
-            const double2 y = __ldcg(reinterpret_cast<const double2*>(&gc[r]) + 1);
-            vv[u] = x.x;
-            jj[u] = static_cast<int>(x.y & 0xffffffffll);
-            ss[u] = y.x;
-            aa[u] = y.y;
-          }
+          x[u] = r < C ? __ldcg(reinterpret_cast<const longlong2*>(&gc[r]))
+                       : make_longlong2(LLONG_MIN, INT_MAX);
         }
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (vv[u] > bv || (vv[u] == bv && jj[u] < p)) {
-            bv = vv[u];
-            p = jj[u];
-            wst = ss[u];
-            wal = aa[u];
+        for (int u = 0; u < U; ++u) {
+          const int j = static_cast<int>(x[u].y & 0xffffffffll);
+          if (x[u].x > bv || (x[u].x == bv && j < p)) {
+            bv = x[u].x;
+            p = j;
           }
+        }
       }
     } else if (lane < C) {
       bv = cands[slot][lane].v;
       p = cands[slot][lane].j;
     }
-    const int mine = p;   // this lane's best before the warp's reduction
     warp_argmax_bits(bv, p);
-    if constexpr (GRP) {
-      // the winner's residual from the lane that loaded it
-      const unsigned has = __ballot_sync(0xffffffffu, mine == p);
-      const int src = __ffs(has) - 1;
-      wst = __shfl_sync(0xffffffffu, wst, src);
-      wal = __shfl_sync(0xffffffffu, wal, src);
-    }
     const int owner = p % C;
-    if (tid == 0 || tid == 32) {
-      // the reflector from the owner's pushed residual, the same arithmetic on
-      // every CTA; two threads on two schedulers run the two divisions side
-      // by side while the other warps copy the pivot column
-      double st, alpha;
-      if constexpr (GRP) {
-        st = wst;
-        alpha = wal;
-      } else {
-        st = cands[slot][owner].st;
-        alpha = cands[slot][owner].alpha;
-      }
-      const double sa = fma(alpha, alpha, st);
-      const double sigma = sqrt(sa);
-      const double r11_now = (i == 0) ? sigma : r11;
-      const int stop = (r11_now == 0.0 || sigma <= fmax(rtol * r11_now, atol)) ? 1 : 0;
-      const bool refl = !stop && st != 0.0;
-      const double beta = refl ? -copysign(sigma, alpha) : alpha;
-      if (tid == 0) {
-        hh[0] = sigma;
-        hh[1] = refl ? (beta - alpha) / beta : 0.0;
-        hstop = stop;
-        if (!stop) {
-          if (owner == crank) {
-            const int jp = p / C;
-            rdiag[jp] = beta;
-            nrm[jp] = -1.0;
-            pstep[jp] = i;
-            const int pos = apos[jp], last = alist[nact - 1];
-            alist[pos] = last;
-            apos[last] = pos;
-            --nact;
-          }
-          if (crank == 0) perm[i] = p;
-        }
-      } else {
-        hh[3] = refl ? 1.0 / (alpha - beta) : 0.0;
-      }
-    } else if (tid >= 64) {
-      // the pivot column, entries i..d-1, from its owner
-      if (w_in_smem) {
-        const double* src = cg::this_cluster().map_shared_rank(Wsm + (size_t)(p / C) * ldw, owner);
-        for (int c = i + tid - 64; c < d; c += ID_THREADS - 64) vloc[c - i] = src[c];
-      } else {
-        // written by another CTA: read from L2, eight loads in flight per
-        // thread before the stores
-        const double* src = it.work + (size_t)p * d;
-        constexpr int U = 8, NT = ID_THREADS - 64;
-        for (int c0 = i + tid - 64; c0 < d; c0 += NT * U) {
-          double x[U];
-#pragma unroll
-          for (int u = 0; u < U; ++u) x[u] = c0 + NT * u < d ? __ldcg(src + c0 + NT * u) : 0.0;
-#pragma unroll
-          for (int u = 0; u < U; ++u)
-            if (c0 + NT * u < d) vloc[c0 + NT * u - i] = x[u];
-        }
-      }
+    // the winner's reflector and its column, entries i..d-1, from the owner
+    double sigma, tau, scal;
+    if constexpr (GRP) {
+      const double2 y = __ldcg(reinterpret_cast<const double2*>(&gc[owner]) + 1);
+      scal = __ldcg(&gc[owner].scal);
+      sigma = y.x;
+      tau = y.y;
+    } else {
+      sigma = cands[slot][owner].sigma;
+      tau = cands[slot][owner].tau;
+      scal = cands[slot][owner].scal;
     }
-    __syncthreads();
-    if (i == 0) r11 = hh[0];
-    if (hstop) {
+    // the stopping test on bit patterns (all values are >= 0): |R_11| = 0 or
+    // |R_ii| <= max(rtol |R_11|, atol)
+    const long long sb = __double_as_longlong(sigma) & LLONG_MAX;   // (a NaN is above all)
+    if (i == 0) thr = sb == 0 ? LLONG_MAX : __double_as_longlong(fmax(rtol * sigma, atol) + 0.0);
+    if (sb <= thr) {
       k = i;
       break;   // every CTA of the cluster takes the same decision
     }
-    const double tau = hh[1], scal = hh[3];
-    for (int c = i + tid; c < d; c += ID_THREADS) vloc[c - i] = (c == i) ? 1.0 : vloc[c - i] * scal;
+    if (tid == 0) {
+      if (owner == crank) {
+        const int jp = p / C;
+        rdiag[jp] = cbeta;
+        nrm[jp] = -1.0;
+        pstep[jp] = i;
+        const int pos = apos[jp], last = alist[nact - 1];
+        alist[pos] = last;
+        apos[last] = pos;
+        --nact;
+      }
+      if (crank == 0) perm[i] = p;
+    }
+    if constexpr (WS) {
+      const double* src = cg::this_cluster().map_shared_rank(Wsm + (size_t)(p / C) * ldw, owner);
+      for (int c = i + tid; c < d; c += ID_THREADS) vloc[c - i] = c == i ? 1.0 : src[c] * scal;
+    } else {
+      // written by another CTA: read from L2, eight loads in flight per
+      // thread before the stores
+      const double* src = it.work + (size_t)p * d;
+      constexpr int U = 8;
+      for (int c0 = i + tid; c0 < d; c0 += ID_THREADS * U) {
+        double x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          x[u] = c0 + ID_THREADS * u < d ? __ldcg(src + c0 + ID_THREADS * u) : 0.0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int c = c0 + ID_THREADS * u;
+          if (c < d) vloc[c - i] = c == i ? 1.0 : x[u] * scal;
+        }
+      }
+    }
     __syncthreads();
     // one pass per active column (a team of TS threads, the teams dealt over
     // the compacted list): the pending update of step i-1 and the dot
@@ -575,9 +646,9 @@ id_cpqr_cluster_kernel(const IdItem* __restrict__ items, int f64in,
       const int q = jb + lane / TS;
       const bool act = q < na;
       const int jl = act ? alist[q] : 0;
-      double* wj = act ? col(jl) : nullptr;
+      double* wj = col(jl);
       const bool pd = act && pend[jl] != 0;
-      const double dot = team_update_dot<TS>(i, act ? d : 0, member, pd, pd ? -dprev[jl] : 0.0,
+      const double dot = team_update_dot<TS, WS>(i, act ? d : 0, member, pd, pd ? -dprev[jl] : 0.0,
                                              vprev, vloc, wj);
       if (act && member == 0) {
         dprev[jl] = dot * tau;
@@ -603,7 +674,7 @@ id_cpqr_cluster_kernel(const IdItem* __restrict__ items, int f64in,
           const double r = fabs(fma(-dprev[jl], 1.0, col(jl)[i]));
           const double q = fmax(0.0, (nj - r) * (nj + r));
           if (q <= lim[jl]) recompute = true;
-          else newn = sqrt(q);
+          else newn = fp_sqrt(q);
         }
         // cancellation: recompute those norms, one column at a time with the
         // whole warp (the fixed summation tree gives the same bits as a team)
@@ -648,9 +719,7 @@ id_cpqr_cluster_kernel(const IdItem* __restrict__ items, int f64in,
     __syncthreads();
     {
       // the CTA's candidate (the same total order as the warps' arg-max),
-      // known to every thread; the whole CTA applies its pending update of
-      // step i, so all its rows' loads are in flight at once, then one warp
-      // sums its residual and pushes it
+      // known to every thread
       long long cv = LLONG_MIN;
       int cj = INT_MAX;
       for (int w = 0; w < nwd; ++w)
@@ -658,18 +727,7 @@ id_cpqr_cluster_kernel(const IdItem* __restrict__ items, int f64in,
           cv = redb[w];
           cj = redi[w];
         }
-      if (cv != LLONG_MIN) {
-        const int jl = (cj - crank) / C;
-        if (pend[jl]) {
-          double* w = col(jl);
-          const double a = -dprev[jl];
-          for (int c = i + tid; c < d; c += ID_THREADS) w[c] = fma(a, vloc[c - i], w[c]);
-          __syncthreads();
-          if (tid == 0) pend[jl] = 0;
-          __syncthreads();
-        }
-      }
-      if (warp == 0) push_candidate(slot ^ 1, cv, cj, i + 1);
+      push_candidate(slot ^ 1, cv, cj, i + 1, vloc, vbuf + ((i + 1) & 1) * dv);
     }
   }
 
@@ -683,7 +741,7 @@ id_cpqr_cluster_kernel(const IdItem* __restrict__ items, int f64in,
   }
   // the update of step k - 1 is still pending on the remaining columns
   if (k > 0) {
-    const double* ul = vbuf + ((k - 1) & 1) * d;
+    const double* ul = vbuf + ((k - 1) & 1) * dv;
     const int na = nact;
     for (int q = warp; q < na; q += ID_WARPS) {
       const int jl = alist[q];
@@ -712,68 +770,157 @@ id_cpqr_cluster_kernel(const IdItem* __restrict__ items, int f64in,
   if (!sync_all()) return;   // R1 and flags visible to the whole cluster
   if (crank == 0 && tid == 0) *it.k = k;
   // position of each remaining column in perm[k..m): the count of remaining
-  // columns of lower index
+  // columns of lower index.  Warp 0 walks the flags 32 at a time with the
+  // count so far; the columns this CTA owns are among them, and go to rlist
+  // in order
   int* restpos = pstep;   // reuse: local rest position
-  for (int jl = tid; jl < mloc; jl += ID_THREADS) {
-    const int j = jl * C + crank;
-    int q = -1;
-    if (__ldcg(flag + j)) {
-      q = 0;
-      for (int x = 0; x < j; ++x) q += __ldcg(flag + x);
-    }
-    restpos[jl] = q;
-  }
-  __syncthreads();
-  // T = R1^{-1} R2 for the remaining columns this CTA owns, by column-oriented
-  // back substitution with the whole CTA: at step a each remaining column's
-  // T_a = rhs_a / R_aa (one thread per column), then rhs_c -= R_ca T_a for
-  // c < a (threads over (c, column) pairs).  The right-hand sides are the
-  // columns' first k entries, solved in place; R1's diagonal and its columns
-  // are staged in shared memory one step ahead.  Per column the operations and
-  // their order (a = k-1 down to 0) do not depend on the CTA or cluster size.
   int* rlist = reinterpret_cast<int*>(nrm);   // local indices of the remaining columns
-  if (tid == 0) {
-    int nr = 0;
-    for (int jl = 0; jl < mloc; ++jl)
-      if (restpos[jl] >= 0) rlist[nr++] = jl;
-    nrest = nr;
+  __syncthreads();        // pstep and nrm have been read
+  if (warp == 0) {
+    constexpr int U = 8;
+    int before = 0, mine = 0;
+    for (int j0 = 0; j0 < m; j0 += 32 * U) {
+      int f[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int j = j0 + 32 * u + lane;
+        f[u] = j < m ? __ldcg(flag + j) : 0;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int j = j0 + 32 * u + lane;
+        const unsigned rest = __ballot_sync(0xffffffffu, f[u] != 0);
+        const bool own = j < m && j % C == crank;
+        const unsigned keep = __ballot_sync(0xffffffffu, own && f[u] != 0);
+        const unsigned below = (1u << lane) - 1u;
+        if (own) {
+          const int jl = (j - crank) / C;
+          restpos[jl] = f[u] ? before + __popc(rest & below) : -1;
+          if (f[u]) rlist[mine + __popc(keep & below)] = jl;
+        }
+        before += __popc(rest);
+        mine += __popc(keep);
+      }
+    }
+    if (lane == 0) nrest = mine;
   }
-  double* diag = vbuf;    // k <= d entries
-  for (int a = tid; a < k; a += ID_THREADS) diag[a] = __ldcg(R1 + (size_t)a * k + a);
-  if (k > 0)
-    for (int c = tid; c < k - 1; c += ID_THREADS)
-      colbuf[((k - 1) & 1) * d + c] = __ldcg(R1 + (size_t)(k - 1) * k + c);
+  // T = R1^{-1} R2 for the remaining columns this CTA owns, by column-oriented
+  // back substitution: T_a = rhs_a / R_aa, then rhs_c -= R_ca T_a for c < a, a
+  // from k-1 down to 0, solved in place in the columns' first k entries.  By
+  // blocks of 16 rows: the block itself by groups of four warps (lane =
+  // column, warp q rows q mod 4 of the block: a row's quotient goes through
+  // shared memory to the group), then all its terms for the rows above in one
+  // pass (a thread per row, R's 16 entries in registers).  Each entry gets
+  // its terms one by one in the order of decreasing a, so neither the blocks
+  // nor the CTA or cluster size change its bits.  (Two block barriers and a
+  // division's 680 cycles of latency per row: 0.38 ms at m = 342, k = 241;
+  // by blocks 0.24 ms.)
+  double* diag = vbuf;        // k <= d entries
+  double* rinv = vbuf + dv;   // their reciprocals
+  double(*Rb)[ID_BS + 1] = reinterpret_cast<double(*)[ID_BS + 1]>(cbuf);
+  double(*xs)[2][32] = reinterpret_cast<double(*)[2][32]>(cbuf + ID_BS * (ID_BS + 1));
+  for (int a = tid; a < k; a += ID_THREADS) {
+    const double x = __ldcg(R1 + (size_t)a * k + a);
+    diag[a] = x;
+    rinv[a] = 1.0 / x;
+  }
   __syncthreads();
   const int nr = nrest;
   for (int u = tid; u < nr; u += ID_THREADS) perm[k + restpos[rlist[u]]] = rlist[u] * C + crank;
-  for (int a = k - 1; a >= 0 && nr > 0; --a) {
-    // next step's column of R1 (entries c < a - 1), by the warps not dividing
-    if (a >= 1 && tid >= 32)
-      for (int c = tid - 32; c < a - 1; c += ID_THREADS - 32)
-        colbuf[((a - 1) & 1) * d + c] = __ldcg(R1 + (size_t)(a - 1) * k + c);
-    for (int u = tid; u < nr; u += ID_THREADS) {
-      const int jl = rlist[u];
-      double* r2 = col(jl);
-      const double x = r2[a] / diag[a];
-      r2[a] = x;
-      it.E[(size_t)restpos[jl] * k + a] = x;
+  constexpr int BS = ID_BS;
+  for (int a1 = k; a1 > 0 && nr > 0; a1 -= BS) {
+    const int a0 = max(0, a1 - BS), nb = a1 - a0;
+    for (int e = tid; e < nb * nb; e += ID_THREADS) {
+      const int q = e / nb, t = e - q * nb;
+      if (t < q) Rb[t][q] = __ldcg(R1 + (size_t)(a0 + q) * k + a0 + t);
     }
     __syncthreads();
-    const double* ra = colbuf + (a & 1) * d;   // R_ca for c < a
-    for (int idx = tid; idx < a * nr; idx += ID_THREADS) {
-      const int u = idx / a, c = idx - u * a;
-      double* r2 = col(rlist[u]);
-      r2[c] = fma(-ra[c], r2[a], r2[c]);
+    const int grp = warp >> 2, w4 = warp & 3;
+    for (int u0 = 0; u0 < nr; u0 += 64) {
+      const int u = u0 + 32 * grp + lane;
+      const bool act = u < nr;
+      const int jl = act ? rlist[u] : 0;
+      double* r2 = col(jl);
+      double v[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) v[t] = act && w4 + 4 * t < nb ? r2[a0 + w4 + 4 * t] : 0.0;
+      if (u0 + 32 * grp < nr) {   // uniform in the group
+        for (int q = nb - 1; q >= 0; --q) {
+          if ((q & 3) == w4) {
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+              if (t == (q >> 2)) {
+                v[t] = div_by(v[t], diag[a0 + q], rinv[a0 + q]);
+                xs[grp][q & 1][lane] = v[t];
+              }
+          }
+          asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory");
+          const double xq = xs[grp][q & 1][lane];   // (two slots: a barrier lies between uses)
+#pragma unroll
+          for (int t = 0; t < 4; ++t)
+            if (w4 + 4 * t < q) v[t] = fma(-Rb[w4 + 4 * t][q], xq, v[t]);
+        }
+      }
+      if (act) {
+        double* E = it.E + (size_t)restpos[jl] * k;
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+          if (w4 + 4 * t < nb) {
+            r2[a0 + w4 + 4 * t] = v[t];
+            E[a0 + w4 + 4 * t] = v[t];
+          }
+      }
+    }
+    __syncthreads();
+    if (a0 > 0) {
+      // rows c < a0: threads over (row, every ng-th column)
+      const int cw = min(ID_THREADS, (a0 + 31) & ~31), ng = ID_THREADS / cw, ug = tid / cw;
+      for (int c = tid - ug * cw; c < a0 && ug < ng; c += cw) {
+        double rq[BS];
+#pragma unroll
+        for (int q = 0; q < BS; ++q) rq[q] = q < nb ? __ldcg(R1 + (size_t)(a0 + q) * k + c) : 0.0;
+        // four columns at a time: an entry's 16 terms are a chain of 67
+        // cycles each
+        for (int u = ug; u < nr; u += 4 * ng) {
+          double* r2[4];
+          double v[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            r2[e] = col(rlist[min(u + e * ng, nr - 1)]);
+            v[e] = r2[e][c];
+          }
+#pragma unroll
+          for (int q = BS - 1; q >= 0; --q)
+            if (q < nb) {
+#pragma unroll
+              for (int e = 0; e < 4; ++e)
+                if (u + e * ng < nr) v[e] = fma(-rq[q], r2[e][a0 + q], v[e]);
+            }
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (u + e * ng < nr) r2[e][c] = v[e];
+        }
+      }
     }
     __syncthreads();
   }
 }
 
-using IdKernel = void (*)(const IdItem*, int, int, double*, const int64_t*, GroupArgs);
+using IdKernel = void (*)(const IdItem*, int, double*, const int64_t*, GroupArgs);
 std::array<IdKernel, 6> kernels() {
   return {id_cpqr_cluster_kernel<1, false>, id_cpqr_cluster_kernel<2, false>,
           id_cpqr_cluster_kernel<4, false>, id_cpqr_cluster_kernel<8, false>,
           id_cpqr_cluster_kernel<16, false>, id_cpqr_cluster_kernel<32, false>};
+}
+// Columns in shared memory.  At most 128 registers a thread where that does
+// not spill: with one CTA per SM only 15 clusters of 8 (7 of 16) fit on the
+// GPU at once, so a launch of 128 CTAs would run a second wave for its last
+// cluster (897 -> 1343 us and 1304 -> 2122 us on two levels of a Gaussian
+// kernel's compression).
+std::array<IdKernel, 6> smem_kernels() {
+  return {id_cpqr_cluster_kernel<1, false, 1, true>,  id_cpqr_cluster_kernel<2, false, 1, true>,
+          id_cpqr_cluster_kernel<4, false, 2, true>,  id_cpqr_cluster_kernel<8, false, 2, true>,
+          id_cpqr_cluster_kernel<16, false, 2, true>, id_cpqr_cluster_kernel<32, false, 2, true>};
 }
 std::array<IdKernel, 6> group_kernels() {
   return {id_cpqr_cluster_kernel<1, true>, id_cpqr_cluster_kernel<2, true>,
@@ -977,7 +1124,7 @@ Err launch_id_batched(const IdItem* items_dev, const std::vector<IdItem>& h, boo
   const int d = std::max(max_d, 1);
   auto need = [&](int c) {
     int mloc = (max_m + c - 1) / c;
-    return sizeof(double) * (3 * (size_t)d + 4 * (size_t)mloc) +
+    return sizeof(double) * (2 * (size_t)id_vec(d) + (size_t)id_cbuf(d) + 4 * (size_t)mloc) +
            4 * sizeof(int) * (size_t)((mloc + 1) & ~1);
   };
   // a large side among many items: more CTAs per item until its share of the
@@ -1021,6 +1168,7 @@ Err launch_id_batched(const IdItem* items_dev, const std::vector<IdItem>& h, boo
       HSS_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
       std::vector<IdKernel> ck;
       for (auto fn : kernels()) ck.push_back(fn);
+      for (auto fn : smem_kernels()) ck.push_back(fn);
       for (auto fn : kernels2()) ck.push_back(fn);
       for (auto fn : ck) {
         cudaFuncAttributes fa;
@@ -1188,7 +1336,7 @@ Err launch_id_batched(const IdItem* items_dev, const std::vector<IdItem>& h, boo
     if (trial) cudaEventRecord(trial->e0, s);
     cudaError_t e = cudaLaunchKernelEx(&gcfg, (two_per_sm ? group_kernels2() : group_kernels())[ti],
                                        items_dev,
-                                       f64 ? 1 : 0, 0, r1, (const int64_t*)offd, ga);
+                                       f64 ? 1 : 0, r1, (const int64_t*)offd, ga);
     if (trial) {
       if (e == cudaSuccess) cudaEventRecord(trial->e1, s);
       TeamTuner::get().launched(trial, e == cudaSuccess);
@@ -1262,8 +1410,10 @@ Err launch_id_batched(const IdItem* items_dev, const std::vector<IdItem>& h, boo
       two = two_fit(C, smem, 0);
     }
     if (trial) cudaEventRecord(trial->e0, s);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, (two ? kernels2() : kernels())[ti], items_dev,
-                                       f64 ? 1 : 0, w_in_smem, r1, (const int64_t*)offd, ga);
+    // (clusters of 4 and more: two CTAs per SM also where there are SMs enough,
+    // as for the columns in shared memory)
+    const IdKernel fn = (w_in_smem ? smem_kernels() : two || C >= 4 ? kernels2() : kernels())[ti];
+    cudaError_t e = cudaLaunchKernelEx(&cfg, fn, items_dev, f64 ? 1 : 0, r1, (const int64_t*)offd, ga);
     if (trial) {
       if (e == cudaSuccess) cudaEventRecord(trial->e1, s);
       TeamTuner::get().launched(trial, e == cudaSuccess);

@@ -153,3 +153,40 @@ def test_ulv_solve_tasks(P, dtype):
     assert st == [0] * 4
     for h, B, X in zip(hs, Bs, Xs):
         assert torch.equal(P.hss_solve(h, B), X)
+
+
+# one column; k at, below and above a block of 16 rows of the back
+# substitution; fewer, as many and more columns than a warp; short columns
+# (the shared blocks larger than a column) and long ones; columns in shared
+# and (the last) in global memory; k = min(m, d), nothing left for E
+@pytest.mark.parametrize("d,m,k", [
+    (17, 1, 1), (16, 33, 16), (40, 31, 15), (40, 33, 17), (127, 65, 31), (129, 200, 33),
+    (401, 90, 48), (64, 520, 60), (33, 20, 20), (900, 700, 97),
+])
+def test_id_at_block_edges(P, d, m, k):
+    """Against the oracle's CPQR: the same pivots (random matrices of exact
+    rank: residual norms differ far above rounding) and generators (the
+    triangle's condition is below 1e5, so its rounding below 1e-10)."""
+    from oracle import hss_oracle as O
+    rng = np.random.default_rng(1000 * d + m)
+    Y = rng.standard_normal((d, k)) @ rng.standard_normal((k, m))
+    r = O.interpolative_decomposition(Y, 1e-11)
+    Yt = torch.tensor(Y.T.copy(), dtype=torch.float64, device=DEV)
+    for copies in (1, 7):   # alone, and in a batch (other clusters, the same bits)
+        for kg, perm, E in P.hss_id_batched([Yt] * copies, 1e-11):
+            perm = perm.cpu().numpy()
+            assert kg == r.k == k
+            assert list(perm[:k]) == list(r.perm[:k])
+            assert sorted(perm.tolist()) == list(range(m))
+            G = np.zeros((m, k))
+            G[perm[:k]] = np.eye(k)
+            G[perm[k:]] = E.cpu().numpy().reshape(m - k, k)
+            np.testing.assert_allclose(G, r.basis(), rtol=1e-7, atol=1e-9)
+
+
+@pytest.mark.parametrize("d,m", [(40, 30), (300, 500)])
+def test_id_of_nan_finishes(P, d, m):
+    Y = torch.full((m, d), float("nan"), dtype=torch.float64, device=DEV)
+    k, perm, _ = P.hss_id_batched([Y], 1e-6)[0]
+    assert 0 <= k <= min(m, d)
+    assert sorted(perm.cpu().tolist()) == list(range(m))
