@@ -46,8 +46,8 @@
 // pivot column 1000-1500, the columns' pass 4000-5000, the downdates 1700 and
 // the candidate with its reflector 3800 -- forming the reflector before the
 // barrier (once, not in every CTA after it), integer arg-max reductions and
-// the integer root and quotient took the IDs of that compression from 11.4 to
-// 10.2 ms; large items (n = 60000, m to 4700) are bound by the FP64 pipe in
+// the integer root and quotient took that compression (all of it) from 17.2 to
+// 16.0 ms; large items (n = 60000, m to 4700) are bound by the FP64 pipe in
 // the pass: the registers kept under 128, so that two CTAs fit an SM, took
 // that compression from 1451 to 1299 ms.
 #include "hss_internal.cuh"
