@@ -26,10 +26,12 @@
 // converters write.  R_p^T goes to TMEM from the transposed copy of R in
 // global memory (no shared-memory stage).
 //
-// Pipeline (warp-specialised, mbarrier hand-offs, 576 threads):
+// Pipeline (warp-specialised, mbarrier hand-offs, 640 threads):
 //   warp 0       TMA producer: FP32 half-tiles of A (128 x 32, 128-byte
-//                swizzle), one stage per converter group; R_J (64 rows) per tile and
-//                R_p (128 rows) per panel segment, bfloat16;
+//                swizzle), one stage per converter group, asked into L2 one
+//                tile ahead;
+//   warp 19      TMA producer: R_J (64 rows) per tile and R_p (128 rows) per
+//                panel segment, bfloat16;
 //   warps 2-9    converters: two threads per row, one per half-tile; apply
 //                the leaf mask (the index range of the row's leaf), split into
 //                the bfloat16 planes or round to TF32 (double-buffered,
@@ -38,18 +40,26 @@
 //   warp 1       MMA issuer (one thread): tcgen05.mma into TMEM;
 //   warps 10-13  column drain: the column product of each tile (TMEM, three
 //                buffers) is summed over the panel pair through distributed
-//                shared memory (each CTA sends its partner the half of the 64
-//                columns the partner owns and adds the half it receives,
-//                pipelined by one tile) and written to a partial slab
-//                Sc_part[pg][j][c] (c contiguous): half the slab of one
-//                partial per panel;
-//   warps 14-17  row fold: the row accumulator (TMEM) holds a chain of at
-//                most g.chain tiles; the fold adds it to the flush group's
-//                running sum (TMEM) and gives it back to the MMA, and writes
-//                the sum of a flush group (at most 16 tiles) to the group's
-//                slot of a row slab.  The MMA issues a tile's column product
-//                before its row product, so the tensor core stays busy while
-//                the fold reads the previous chain.
+//                shared memory: each CTA sends its partner the half of the 64
+//                columns the partner owns (one bulk copy; TF32: st.async);
+//   warps 14-17  row fold and column sum: the row accumulator (TMEM) holds a
+//                chain of at most g.chain tiles; the fold adds it to the flush
+//                group's running sum (TMEM) and gives it back to the MMA, and
+//                writes the sum of a flush group (at most 16 tiles) to the
+//                group's slot of a row slab.  The MMA issues a tile's column
+//                product, and commits it, before its row product, so the
+//                tensor core and the drain stay busy while the fold reads the
+//                previous chain.  Then the half received from the partner is
+//                added to this CTA's own half, in the exchange slot;
+//   warp 18      copies the sums to a partial slab Sc_part[pg][j][c] (c
+//                contiguous): half the slab of one partial per panel; and
+//                gives the slot back to the partner.
+// What bounds it: the hand-offs.  At n = 20000 and 128 columns a tile takes
+// 3800 cycles, of which the tensor pipe is busy 1540, shared memory about 2400
+// (operands, planes, stages, exchange) and HBM 2300 (A, and 1 GB of slabs).
+// The call took 1.33 ms and takes 0.88: an issuing warp with uniform operands
+// (1.24 -> 1.00), places stepped instead of divided out (1.30 -> 1.19), the
+// slab and the exchange by bulk copies, the reduction's rows (0.96 -> 0.88).
 // TMEM columns: [0,128) the row accumulator, [128,256) the running row sum,
 // [256,448) three column accumulators, [448,512) R_p^T, the column
 // product's A operand (TF32: two column accumulators in [256,384) and R_p^T,
@@ -108,7 +118,7 @@ constexpr int FLUSH_MAX = 16;    // tiles per flush group of the running row sum
 // about linearly with the chain (measured: 16 tiles gave 4.6x the row-sample
 // error of 2 tiles), so the fold warps add the chains of a flush group in
 // FP32 on the CUDA cores.
-constexpr int THREADS = 576;
+constexpr int THREADS = 640;
 constexpr long long WAIT_LIMIT = 1ll << 32;   // clock cycles (about 2 s)
 
 constexpr uint32_t A_HALF_BYTES = BM * 32 * 4;   // 16 KB
@@ -155,7 +165,7 @@ enum {
   B_RIEMPTY = B_RIFULL + 1, B_CFULL = B_RIEMPTY + 1, B_CEMPTY = B_CFULL + CBUF,
   B_RFULL = B_CEMPTY + CBUF, B_REMPTY = B_RFULL + 1, B_DRAIN = B_REMPTY + 1, B_XFULL = B_DRAIN + 1,
   B_XEMPTY = B_XFULL + XSLOTS, B_RTFULL = B_XEMPTY + XSLOTS, B_RSEMPTY = B_RTFULL + 1,
-  B_COUNT = B_RSEMPTY + 1
+  B_XREAD = B_RSEMPTY + 1, B_COUNT = B_XREAD + XSLOTS
 };
 
 struct TcArgs {
@@ -191,6 +201,33 @@ __host__ __device__ __forceinline__ long long tile_owner(long long t, long long 
   return ((t + 1) * P - 1) / T;
 }
 
+// A position in a cluster's range: panel pair, column tile, the tile's flush
+// group, its place in the group and in its chain.  Stepped, not recomputed:
+// the divisions of t by the tiles per panel took 1000-1900 cycles per tile in
+// every role, of 6000 in all (n = 20000, 128 columns: 1.30 -> 1.19 ms).
+struct Walk {
+  int pg, J, grp, g, h;
+  __device__ __forceinline__ Walk(long long t, int ntc, int gs, int chain) {
+    pg = static_cast<int>(t / ntc);
+    J = static_cast<int>(t - static_cast<long long>(pg) * ntc);
+    grp = J / gs;
+    g = J - grp * gs;
+    h = g % chain;
+  }
+  __device__ __forceinline__ void next(int ntc, int gs, int chain) {
+    ++g;
+    if (++h == chain) h = 0;
+    if (g == gs) {
+      g = h = 0;
+      ++grp;
+    }
+    if (++J == ntc) {
+      J = grp = g = h = 0;
+      ++pg;
+    }
+  }
+};
+
 template <int NT>
 __global__ void __launch_bounds__(THREADS, 1)
     sample_tc_kernel(const __grid_constant__ CUtensorMap tmA,
@@ -210,8 +247,10 @@ __global__ void __launch_bounds__(THREADS, 1)
   // saw it (one flag per wait: each is written once per tile, between the
   // group's named barriers)
   volatile int* dstop = abort_flag + 1;   // [0], [1]: per tile; [2]: R_p copy
-  volatile int* fstop = abort_flag + 4;   // the row fold warps: [0], [1] by chain parity; [2] per tile
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  volatile int* rstop = abort_flag + 4;   // row fold, by chain parity
+  volatile int* fstop = abort_flag + 6;   // column sum, by tile parity
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (warp-uniform for the compiler)
   auto bar = [&](int i) { return su32(&bars[i]); };
 
   if (tid == 0) {
@@ -230,7 +269,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     mbar_init(bar(B_REMPTY), BM);
     for (int i = 0; i < CBUF; ++i) {
       mbar_init(bar(B_CFULL + i), 1);
-      mbar_init(bar(B_CEMPTY + i), 2 * BM);   // the drain's and the fold's reads
+      mbar_init(bar(B_CEMPTY + i), 2 * BM);   // the drain's and the column sum's reads
     }
     mbar_init(bar(B_RIFULL), 1);
     mbar_init(bar(B_RIEMPTY), 1);
@@ -240,6 +279,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     for (int i = 0; i < XSLOTS; ++i) {
       mbar_init(bar(B_XFULL + i), 1);
       mbar_init(bar(B_XEMPTY + i), 1);
+      mbar_init(bar(B_XREAD + i), BM);
     }
     *abort_flag = 0;
     fence_mbar_init();
@@ -267,33 +307,48 @@ __global__ void __launch_bounds__(THREADS, 1)
   const int ntc = g.ntc, gs = g.gs, chain = g.chain;
 
   if (warp == 0) {
-    // ------------------------------------------------------ TMA producer
+    // -------------------------------------------------- TMA producer of A
     if (lane == 0) {
-      int a_cnt = 0, tl = 0, ri_cnt = 0;
-      for (long long t = tb; t < te; ++t) {
-        const int p = KC * static_cast<int>(t / ntc) + crank, J = static_cast<int>(t % ntc);
-        const bool first = (t == tb) || J == 0;
-        if (!is_tf32<NT>() && !g.rows_only && first) {
-          // the previous segment's R_p has been copied to TMEM
-          if (!mbar_wait(bar(B_RSEMPTY), (ri_cnt & 1) ^ 1, abort_flag, g.err, 1, WAIT_LIMIT))
-            break;
-          mbar_expect_tx(bar(B_RIFULL), g.ncb * (RI_BYTES / 2));
-          for (int cb = 0; cb < g.ncb; ++cb)
-            tma_load_2d(su32(sm + L::ri + cb * (RI_BYTES / 2)), &tmRI, cb * 64, p * BM,
-                        bar(B_RIFULL));
-          ++ri_cnt;
-        }
+      int a_cnt = 0;
+      Walk w(tb, ntc, gs, chain), f = w;
+      for (long long t = tb; t < te; ++t, w = f) {
+        // the next tile into L2 (one ahead: 0.908 -> 0.880 ms at n = 20000 and
+        // 128 columns; two the same, three and six slower)
+        f.next(ntc, gs, chain);
+        if (t + 1 < te)
+          for (int h = 0; h < 2; ++h)
+            tma_prefetch_2d(&tmA, f.J * BN + h * 32, (KC * f.pg + crank) * BM);
         bool ok = true;
         for (int h = 0; h < 2 && ok; ++h) {
           const int s = a_cnt % AS, u = a_cnt / AS;
           ok = mbar_wait(bar(B_AEMPTY + s), (u & 1) ^ 1, abort_flag, g.err, 2, WAIT_LIMIT);
           if (!ok) break;
           mbar_expect_tx(bar(B_AFULL + s), A_HALF_BYTES);
-          tma_load_2d(su32(sm + L::a + s * A_HALF_BYTES), &tmA, J * BN + h * 32, p * BM,
-                      bar(B_AFULL + s));
+          tma_load_2d(su32(sm + L::a + s * A_HALF_BYTES), &tmA, w.J * BN + h * 32,
+                      (KC * w.pg + crank) * BM, bar(B_AFULL + s));
           ++a_cnt;
         }
         if (!ok) break;
+      }
+      if (*abort_flag) {
+        // let every copy this thread issued land before the CTA exits
+        volatile int never = 0;
+        for (int s = 0; s < AS; ++s) {
+          const int uses = (a_cnt - s + AS - 1) / AS;
+          if (uses > 0) mbar_wait(bar(B_AFULL + s), (uses - 1) & 1, &never, g.err, 9, WAIT_LIMIT);
+        }
+      }
+    }
+  } else if (warp == 19) {
+    // ------------------------------------- TMA producer of R_J and R_p
+    // (a thread of its own: R_J waits for the MMAs two tiles back, A only for
+    // the converters)
+    if (lane == 0) {
+      int tl = 0, ri_cnt = 0;
+      Walk w(tb, ntc, gs, chain);
+      for (long long t = tb; t < te; ++t, w.next(ntc, gs, chain)) {
+        const int p = KC * w.pg + crank, J = w.J;
+        const bool first = (t == tb) || J == 0;
         const int r = tl & 1, u = tl >> 1;
         if (!mbar_wait(bar(B_RJEMPTY + r), (u & 1) ^ 1, abort_flag, g.err, 3, WAIT_LIMIT)) break;
         if constexpr (is_tf32<NT>()) {
@@ -309,14 +364,20 @@ __global__ void __launch_bounds__(THREADS, 1)
                         bar(B_RJFULL + r));
         }
         ++tl;
+        if (!is_tf32<NT>() && !g.rows_only && first) {
+          // the previous segment's exchange copies have left the buffer of R_p
+          if (!mbar_wait(bar(B_RSEMPTY), (ri_cnt & 1) ^ 1, abort_flag, g.err, 1, WAIT_LIMIT))
+            break;
+          mbar_expect_tx(bar(B_RIFULL), g.ncb * (RI_BYTES / 2));
+          for (int cb = 0; cb < g.ncb; ++cb)
+            tma_load_2d(su32(sm + L::ri + cb * (RI_BYTES / 2)), &tmRI, cb * 64, p * BM,
+                        bar(B_RIFULL));
+          ++ri_cnt;
+        }
       }
       if (*abort_flag) {
-        // let every copy this thread issued land before the CTA exits
+        // as above
         volatile int never = 0;
-        for (int s = 0; s < AS; ++s) {
-          const int uses = (a_cnt - s + AS - 1) / AS;
-          if (uses > 0) mbar_wait(bar(B_AFULL + s), (uses - 1) & 1, &never, g.err, 9, WAIT_LIMIT);
-        }
         for (int r = 0; r < 2; ++r) {
           const int uses = (tl - r + 1) / 2;
           if (uses > 0) mbar_wait(bar(B_RJFULL + r), (uses - 1) & 1, &never, g.err, 9, WAIT_LIMIT);
@@ -326,7 +387,16 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
   } else if (warp == 1) {
     // ------------------------------------------------------- MMA issuer
-    if (lane == 0) {
+    // The whole warp walks the tiles with warp-uniform values, and one elected
+    // lane issues: the operands then stand in uniform registers, and an MMA
+    // does not wait for moves into them (issued by a lone thread, each took 70
+    // cycles, twice what the column product's MMAs run for).
+    const uint32_t tb_u = __shfl_sync(0xffffffffu, tbase, 0);
+    auto wait = [&](int slot, uint32_t parity, int code) {
+      return __all_sync(0xffffffffu,
+                        mbar_wait(bar(slot), parity, abort_flag, g.err, code, WAIT_LIMIT)) != 0;
+    };
+    {
       // bfloat16: the planes K-major and R_J MN-major (row product), R_p^T
       // from TMEM and the planes MN-major (column product).  TF32: R_J^T and
       // the A stages, both K-major (the transposed row product, M = sample
@@ -344,34 +414,41 @@ __global__ void __launch_bounds__(THREADS, 1)
                                            : sdesc(su32(sm + L::rj), RJ_BOX, 1024);   // R_J, MN-major
       const uint64_t a_stg = sdesc(su32(sm + L::a), 16, 1024);   // TF32: A stages, K-major
       int tl = 0, seg = 0, ch = 0, since = 0;
-      for (long long t = tb; t < te; ++t) {
-        const int J = static_cast<int>(t % ntc);
+      Walk w(tb, ntc, gs, chain);
+      for (long long t = tb; t < te; ++t, w.next(ntc, gs, chain)) {
+        const int J = w.J;
         const bool first = (t == tb) || J == 0, last = (t == te - 1) || J == ntc - 1;
-        const bool gend = last || (J % gs) == gs - 1;
-        const bool cend = gend || ((J % gs) % chain) == chain - 1;
+        const bool gend = last || w.g == gs - 1;
+        const bool cend = gend || w.h == chain - 1;
         const bool col = !g.rows_only;
-        if (col && first && !mbar_wait(bar(B_RTFULL), seg & 1, abort_flag, g.err, 4, WAIT_LIMIT))
-          break;
+        if (col && first && !wait(B_RTFULL, seg & 1, 4)) break;
         const int ps = tl & 1, u = tl >> 1;
         const int cb = tl % CB, cu = tl / CB;
-        if (!mbar_wait(bar(B_PFULL + ps), u & 1, abort_flag, g.err, 5, WAIT_LIMIT)) break;
-        if (!mbar_wait(bar(B_RJFULL + ps), u & 1, abort_flag, g.err, 6, WAIT_LIMIT)) break;
-        if (col && !mbar_wait(bar(B_CEMPTY + cb), (cu & 1) ^ 1, abort_flag, g.err, 7, WAIT_LIMIT))
-          break;
+        // three barriers in one poll: lane 0 R_J, lane 1 the column buffer, the
+        // others the planes
+        {
+          const bool l0 = lane == 0, l1 = lane == 1 && col;
+          const uint32_t b = l0 ? bar(B_RJFULL + ps) : l1 ? bar(B_CEMPTY + cb) : bar(B_PFULL + ps);
+          const uint32_t par = l1 ? (cu & 1) ^ 1 : u & 1;
+          if (!__all_sync(0xffffffffu, mbar_wait(b, par, abort_flag, g.err, l0 ? 6 : l1 ? 7 : 5,
+                                                 WAIT_LIMIT)))
+            break;
+          __syncwarp();
+        }
         fence_after();
         const uint64_t poff = (ps * L::pstage) >> 4;
         const uint64_t roff = (ps * L::rjstage) >> 4;
         // the column product first: it keeps the tensor core busy while the
         // fold warps read the previous chain's row accumulator
-        const uint32_t dc = tbase + T_COL + 64 * cb;
-        if (!col) {
-          // row samples only
+        const uint32_t dc = tb_u + T_COL + 64 * cb;
+        if (!col || !elect_one()) {
+          // row samples only, or another lane
         } else if constexpr (is_tf32<NT>()) {
           // K = 8 panel rows per MMA: eight TMEM columns of R_p^T, 32 bytes
           // along the rows of one 8 KB chunk of the transposed tile
 #pragma unroll
           for (int k = 0; k < BM / 8; ++k)
-            mma_tf32_tmem_a(dc, tbase + T_RP + 8 * k,
+            mma_tf32_tmem_a(dc, tb_u + T_RP + 8 * k,
                             b_col + poff + (((k >> 2) * 8192 + 32 * (k & 3)) >> 4), idc,
                             k > 0 ? 1u : 0u);
         } else {
@@ -379,57 +456,61 @@ __global__ void __launch_bounds__(THREADS, 1)
           for (int term = 0; term < NT; ++term) {
 #pragma unroll
             for (int k = 0; k < BM / 16; ++k)
-              mma_bf16_tmem_a(dc, tbase + T_RP + 8 * k,
+              mma_bf16_tmem_a(dc, tb_u + T_RP + 8 * k,
                               b_col + poff + ((term * PLANE_BYTES + 2048 * k) >> 4), idc,
                               (term > 0 || k > 0) ? 1u : 0u);
           }
         }
+        __syncwarp();
+        if (col && elect_one()) mma_commit(bar(B_CFULL + cb));
         if (since == 0) {
-          if (!mbar_wait(bar(B_REMPTY), (ch & 1) ^ 1, abort_flag, g.err, 8, WAIT_LIMIT)) break;
+          if (!wait(B_REMPTY, (ch & 1) ^ 1, 8)) break;
           fence_after();
         }
-        const uint32_t dr = tbase + T_ROW;
-        if constexpr (is_tf32<NT>()) {
-          // K = 8 columns of the tile per MMA: 32 bytes along the rows of
-          // one half of R_J^T and of the tile's A stage of that half (the
-          // tile's two stages are adjacent: four stages, two per tile)
-          const uint64_t aoff = (((2 * tl) % AS) * A_HALF_BYTES) >> 4;
+        const uint32_t dr = tb_u + T_ROW;
+        __syncwarp();
+        if (elect_one()) {
+          if constexpr (is_tf32<NT>()) {
+            // K = 8 columns of the tile per MMA: 32 bytes along the rows of
+            // one half of R_J^T and of the tile's A stage of that half (the
+            // tile's two stages are adjacent: four stages, two per tile)
+            const uint64_t aoff = (((2 * tl) % AS) * A_HALF_BYTES) >> 4;
 #pragma unroll
-          for (int k = 0; k < BN / 8; ++k) {
-            const uint32_t koff = (k >> 2) * A_HALF_BYTES + 32 * (k & 3);
-            mma_tf32(dr, b_row + roff + (koff >> 4), a_stg + aoff + (koff >> 4), idr,
-                     (since > 0 || k > 0) ? 1u : 0u);
+            for (int k = 0; k < BN / 8; ++k) {
+              const uint32_t koff = (k >> 2) * A_HALF_BYTES + 32 * (k & 3);
+              mma_tf32(dr, b_row + roff + (koff >> 4), a_stg + aoff + (koff >> 4), idr,
+                       (since > 0 || k > 0) ? 1u : 0u);
+            }
+            // the tile's A stages go back to the producer when these MMAs are done
+            mma_commit(bar(B_AEMPTY + (2 * tl) % AS));
+            mma_commit(bar(B_AEMPTY + (2 * tl) % AS + 1));
+          } else {
+#pragma unroll
+            for (int term = 0; term < NT; ++term) {
+#pragma unroll
+              for (int k = 0; k < BN / 16; ++k)
+                mma_bf16(dr, a_row + poff + ((term * PLANE_BYTES + 32 * k) >> 4),
+                         b_row + roff + ((2048 * k) >> 4), idr,
+                         (since > 0 || term > 0 || k > 0) ? 1u : 0u);
+            }
           }
-          // the tile's A stages go back to the producer when these MMAs are done
-          mma_commit(bar(B_AEMPTY + (2 * tl) % AS));
-          mma_commit(bar(B_AEMPTY + (2 * tl) % AS + 1));
-        } else {
-#pragma unroll
-          for (int term = 0; term < NT; ++term) {
-#pragma unroll
-            for (int k = 0; k < BN / 16; ++k)
-              mma_bf16(dr, a_row + poff + ((term * PLANE_BYTES + 32 * k) >> 4),
-                       b_row + roff + ((2048 * k) >> 4), idr,
-                       (since > 0 || term > 0 || k > 0) ? 1u : 0u);
-          }
+          mma_commit(bar(B_PEMPTY + ps));
+          mma_commit(bar(B_RJEMPTY + ps));
+          if (cend) mma_commit(bar(B_RFULL));   // the row accumulator holds the chain's sum
+          if (col && last) mma_commit(bar(B_RIEMPTY));
         }
-        mma_commit(bar(B_PEMPTY + ps));
-        mma_commit(bar(B_RJEMPTY + ps));
-        if (col) mma_commit(bar(B_CFULL + cb));
+        __syncwarp();
         ++since;
-        if (cend) {   // the row accumulator holds the chain's sum
-          mma_commit(bar(B_RFULL));
+        if (cend) {
           ++ch;
           since = 0;
         }
-        if (col && last) {
-          mma_commit(bar(B_RIEMPTY));
-          ++seg;
-        }
+        if (col && last) ++seg;
         ++tl;
       }
       // every MMA issued has completed before TMEM is released
-      mma_commit(bar(B_DRAIN));
+      __syncwarp();
+      if (elect_one()) mma_commit(bar(B_DRAIN));
       volatile int never = 0;
       mbar_wait(bar(B_DRAIN), 0, &never, g.err, 10, WAIT_LIMIT);
     }
@@ -439,8 +520,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int row = ct & (BM - 1), h = ct >> 7;   // row of the tile, half-tile
     int tl = 0;
     int mlo = 0, mhi = 0;   // the leaf of this thread's row: columns [mlo, mhi) are masked
-    for (long long t = tb; t < te; ++t) {
-      const int p = KC * static_cast<int>(t / ntc) + crank, J = static_cast<int>(t % ntc);
+    Walk w(tb, ntc, gs, chain);
+    for (long long t = tb; t < te; ++t, w.next(ntc, gs, chain)) {
+      const int p = KC * w.pg + crank, J = w.J;
       const int ps = tl & 1, u = tl >> 1;
       const int n = g.n;
       if (t == tb || J == 0) {
@@ -543,10 +625,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     // Each tile's column product (c x 64, in one of three TMEM buffers) is
     // summed over the cluster's two panels before it reaches HBM: these warps
     // send the partner the half of the 64 columns that the partner owns
-    // (st.async into its shared memory, counted on its X_FULL); the row fold
-    // warps add the half received to this CTA's own half and store the sum.
-    // One thread does the waits and the group follows it through a named
-    // barrier, so its control flow stays uniform.
+    // (counted on its X_FULL); the column-sum warps add the half received to
+    // this CTA's own half.  One thread does the waits and the group follows it
+    // through a named barrier, so its control flow stays uniform.
     const int e = (warp & 3) * 32 + lane;       // TMEM lane: sample column
     const uint32_t loff = static_cast<uint32_t>((warp & 3) * 32) << 16;
     const int c = g.c;
@@ -560,16 +641,26 @@ __global__ void __launch_bounds__(THREADS, 1)
     // (no column product: nothing to drain)
     const int nt = g.rows_only ? 0 : static_cast<int>(te - tb);
     int rseg = 0;
-    for (int i = 0; i < nt; ++i) {
+    Walk wk(tb, ntc, gs, chain);
+    for (int i = 0; i < nt; ++i, wk.next(ntc, gs, chain)) {
+      const int p = KC * wk.pg + crank;
       const int cb = i % CB, cu = i / CB;
       const int xs = i % XSLOTS, xu = i / XSLOTS;
-      const int J = static_cast<int>((tb + i) % ntc);
-      if (i == 0 || J == 0) {
+      if (i == 0 || wk.J == 0) {
         // a panel segment starts: R_p (bfloat16, in shared memory from the
         // TMA) goes to TMEM transposed, as the column product's A operand,
         // once the previous segment's MMAs are done with TMEM
         if (elect) {
-          const bool ok =
+          bool ok = true;
+          if (!is_tf32<NT>() && i > 0) {
+            // the partner has received what was last sent from each half of
+            // the buffer of R_p: the producer may load the next
+            for (int x = i > 1 ? i - 2 : 0; x < i && ok; ++x)
+              ok = mbar_wait(bar(B_XEMPTY + x % XSLOTS), (x / XSLOTS) & 1, abort_flag, g.err, 15,
+                             WAIT_LIMIT);
+            if (ok) mbar_arrive(bar(B_RSEMPTY));
+          }
+          ok = ok &&
               (is_tf32<NT>() ||
                mbar_wait(bar(B_RIFULL), rseg & 1, abort_flag, g.err, 19, WAIT_LIMIT)) &&
               mbar_wait(bar(B_RIEMPTY), (rseg & 1) ^ 1, abort_flag, g.err, 20, WAIT_LIMIT);
@@ -582,7 +673,6 @@ __global__ void __launch_bounds__(THREADS, 1)
           // lane e: R^T[e][p 128 + r] for the 128 panel rows r, one per
           // column, from global memory (R^T is zero-padded to 2 ngp 128
           // columns, so the rows of a pair's phantom last panel exist)
-          const int p = KC * static_cast<int>((tb + i) / ntc) + crank;
           const float4* src = reinterpret_cast<const float4*>(
               g.rt + static_cast<size_t>(e) * g.ldrt + static_cast<size_t>(p) * BM);
 #pragma unroll
@@ -617,14 +707,10 @@ __global__ void __launch_bounds__(THREADS, 1)
           }
           tmem_wait_st();
         }
-        // the reads of R_p, before the next TMA copy into its buffer
-        fence_proxy_async();
+        // the reads of R_p, before the copies into its buffer
         fence_before();
         named_sync(1, 128);
-        if (elect) {
-          mbar_arrive(bar(B_RTFULL));    // the MMAs may read it
-          mbar_arrive(bar(B_RSEMPTY));   // the producer may load the next R_p
-        }
+        if (elect) mbar_arrive(bar(B_RTFULL));   // the MMAs may read it
         ++rseg;
       }
       // (one barrier per tile: the flag alternates, so it is written again
@@ -645,113 +731,62 @@ __global__ void __launch_bounds__(THREADS, 1)
       tmem_wait_ld();
       fence_before();
       mbar_arrive(bar(B_CEMPTY + cb));
-      if (e < c) {
-        // 16-byte chunks swizzled by row: conflict-free on both sides
+      // 16-byte chunks swizzled by row: conflict-free on both sides
+      if constexpr (is_tf32<NT>()) {
+        if (e < c) {
 #pragma unroll
-        for (int q4 = 0; q4 < HB / 4; ++q4)
-          st_async_v4(xpeer + xs * X_BYTES + xrow + ((q4 ^ (e & 7)) << 4), xfull_peer + 8 * xs,
-                      w[4 * q4], w[4 * q4 + 1], w[4 * q4 + 2], w[4 * q4 + 3]);
+          for (int q4 = 0; q4 < HB / 4; ++q4)
+            st_async_v4(xpeer + xs * X_BYTES + xrow + ((q4 ^ (e & 7)) << 4), xfull_peer + 8 * xs,
+                        w[4 * q4], w[4 * q4 + 1], w[4 * q4 + 2], w[4 * q4 + 3]);
+        }
+      } else {
+        // one bulk copy from the buffer of R_p, which is free between its
+        // copies to TMEM (1024 stores of 16 bytes into the other SM held
+        // these warps for 2000 cycles per tile)
+        uint8_t* stage = sm + L::ri + xs * X_BYTES;
+        if (e < c) {
+#pragma unroll
+          for (int q4 = 0; q4 < HB / 4; ++q4)
+            *reinterpret_cast<float4*>(stage + xrow + ((q4 ^ (e & 7)) << 4)) =
+                make_float4(w[4 * q4], w[4 * q4 + 1], w[4 * q4 + 2], w[4 * q4 + 3]);
+        }
+        fence_proxy_async();
+        named_sync(1, 128);
+        if (elect)
+          bulk_copy_cluster(xpeer + xs * X_BYTES, su32(stage), static_cast<uint32_t>(c) * (HB * 4),
+                            xfull_peer + 8 * xs);
       }
     }
-  } else if (warp >= 14) {
-    // --------------------------------------------------------- row fold
-    // Per tile: the half of the column product received from the partner
-    // (an exchange slot) plus this CTA's own half (TMEM) goes to the column
-    // slab, and the slot goes back to the partner.  At the end of a chain
-    // (at most g.chain tiles) the row accumulator is added to the flush group's
-    // running sum (TMEM, FP32 on the CUDA cores); at the end of a flush group
-    // (at most 16 tiles) the sum goes to the group's slot of the row slab.
-    // One thread does the waits and the group follows it through named
-    // barriers.
+  } else if (warp >= 14 && warp < 18) {
+    // -------------------------------------------- row fold and column sum
+    // Per tile, first the end of a chain, if it is one (the MMA waits for the
+    // accumulator), then the half of the column product received from the
+    // partner (an exchange slot) plus this CTA's own half (TMEM).  One thread
+    // does the waits and the group follows it through named barriers.
     const int e = (warp & 3) * 32 + lane;       // TMEM lane: sample column / panel row
     const uint32_t loff = static_cast<uint32_t>((warp & 3) * 32) << 16;
     const int c = g.c;
-    // 32-column chunks of the row accumulator: sample columns, or (TF32,
-    // the transposed row product: lane = sample column) panel rows
-    const int nch = is_tf32<NT>() ? BM / 32 : (c + 31) / 32;
     const bool elect = warp == 14 && lane == 0;
     constexpr int HB = BN / KC;
     const uint32_t own = static_cast<uint32_t>(crank * HB);
-    const uint32_t xempty_peer = mapa(bar(B_XEMPTY), static_cast<uint32_t>(crank ^ 1));
     const uint32_t xrow = static_cast<uint32_t>(e) * (HB * 4);
-    int ch = 0, jfirst = -1, i = 0;
-    bool gfirst = true;   // the next chain is the first of this CTA's part of a group
-    for (long long t = tb; t < te; ++t, ++i) {
-      const int pg = static_cast<int>(t / ntc);
-      const int p = KC * pg + crank, J = static_cast<int>(t % ntc);
-      const bool last = (t == te - 1) || J == ntc - 1;
-      const bool gend = last || (J % gs) == gs - 1;
-      const bool cend = gend || ((J % gs) % chain) == chain - 1;
-      if (jfirst < 0) jfirst = J;
-      // ---- tile i's column sums (none when only the row product runs)
-      if (!g.rows_only) {
-        const int cb = i % CB, cu = i / CB;
-        const int xs = i % XSLOTS, xu = i / XSLOTS;
-        if (elect) {
-          // this CTA's column product of the tile is in TMEM (the buffer cannot
-          // move on to a later tile before this group has read it), and the
-          // partner's half has arrived
-          mbar_expect_tx(bar(B_XFULL + xs), static_cast<uint32_t>(c) * (HB * 4));
-          const bool ok =
-              mbar_wait(bar(B_CFULL + cb), cu & 1, abort_flag, g.err, 18, WAIT_LIMIT) &&
-              mbar_wait(bar(B_XFULL + xs), xu & 1, abort_flag, g.err, 16, WAIT_LIMIT);
-          fstop[2] = ok ? 0 : 1;
-        }
-        named_sync(2, 128);
-        if (fstop[2]) break;
-        // the partner's half into registers, and the slot back to the partner
-        float r[HB];
-        {
-          const uint8_t* xslot = sm + L::xb + xs * X_BYTES + xrow;
-#pragma unroll
-          for (int q4 = 0; q4 < HB / 4; ++q4) {
-            const float4 x = *reinterpret_cast<const float4*>(xslot + ((q4 ^ (e & 7)) << 4));
-            r[4 * q4] = x.x;
-            r[4 * q4 + 1] = x.y;
-            r[4 * q4 + 2] = x.z;
-            r[4 * q4 + 3] = x.w;
-          }
-        }
-        named_sync(2, 128);
-        if (elect) mbar_arrive_remote(xempty_peer + 8 * xs);
-        fence_after();
-        {
-          float m[HB];
-          tmem_ld32(tbase + loff + T_COL + 64 * cb + own, m);
-          tmem_wait_ld();
-          fence_before();
-          mbar_arrive(bar(B_CEMPTY + cb));
-          if (e < c) {
-            // the pair's sum for columns j = J 64 + own .. + 31 and sample
-            // column e: Sc_part[pg][j][e], so that a warp stores one whole
-            // 128-byte row per instruction (rows are padded to whole tiles;
-            // past n the TMA fill is zero, so the pad holds zeros, which the
-            // reduction never reads)
-            float* dst = g.sc_part +
-                         (static_cast<size_t>(pg) * g.npad + static_cast<size_t>(J) * BN + own) * c + e;
-#pragma unroll
-            for (int x = 0; x < HB; ++x) dst[static_cast<size_t>(x) * c] = m[x] + r[x];
-          }
-        }
-      }
-      if (!cend) continue;
-      // ---- the end of a chain: into the running sum, or to the row slab at
-      // the end of a flush group
+    int ch = 0, gstart = -1;
+    bool gfirst = true;   // the chain is the first of this CTA's part of a group
+    // the end of a chain: the row accumulator goes into the flush group's
+    // running sum, and at the end of the group the sum to the row slab
+    auto fold_chain = [&](const Walk& w, bool gend) -> bool {
+      const int p = KC * w.pg + crank;
+      // 32-column chunks of the row accumulator: sample columns, or (TF32,
+      // the transposed row product: lane = sample column) panel rows
+      const int nch = is_tf32<NT>() ? BM / 32 : (c + 31) / 32;
       const int fb = ch & 1;
       // (the flag alternates with the chain: it is written again only after
       // the next chain's barrier, which every thread reaches after reading it)
       if (elect)
-        fstop[fb] = mbar_wait(bar(B_RFULL), ch & 1, abort_flag, g.err, 14, WAIT_LIMIT) ? 0 : 1;
+        rstop[fb] = mbar_wait(bar(B_RFULL), ch & 1, abort_flag, g.err, 14, WAIT_LIMIT) ? 0 : 1;
       named_sync(2, 128);
-      if (fstop[fb]) break;
+      if (rstop[fb]) return false;
       fence_after();
-      // slot (p, group, side), side 1 when the chunk starts inside the group
-      // (a cluster range began there); a panel past the last (the second of
-      // a pair when the panel count is odd) has none
-      const int grp = J / gs;
-      const int side = (jfirst % gs) != 0 ? 1 : 0;
-      float* dst = g.sr_part +
-                   ((((static_cast<size_t>(p) * g.ngroups + grp) * 2 + side) * c) * BM) + e;
       for (int q = 0; q < nch; ++q) {
         float a[32];
         tmem_ld32(tbase + loff + T_ROW + 32 * q, a);
@@ -776,34 +811,121 @@ __global__ void __launch_bounds__(THREADS, 1)
       mbar_arrive(bar(B_REMPTY));
       ++ch;
       gfirst = gend;
-      if (!gend) continue;
-      jfirst = -1;
-      if (p < g.npanel) {
-        for (int q = 0; q < nch; ++q) {
-          float a[32];
-          tmem_ld32(tbase + loff + T_RSUM + 32 * q, a);
-          tmem_wait_ld();
-          if constexpr (is_tf32<NT>()) {
-            // lane e holds sample column e of panel rows 32 q .. 32 q + 31
-            if (e < c) {
-              float* d = dst - e + static_cast<size_t>(e) * BM + 32 * q;
+      if (!gend) return true;
+      // slot (p, group, side), side 1 when the chunk starts inside the group
+      // (a cluster range began there); a panel past the last (the second of
+      // a pair when the panel count is odd) has none
+      const int side = gstart != 0 ? 1 : 0;
+      gstart = -1;
+      if (p >= g.npanel) return true;
+      float* dst = g.sr_part +
+                   ((((static_cast<size_t>(p) * g.ngroups + w.grp) * 2 + side) * c) * BM) + e;
+      for (int q = 0; q < nch; ++q) {
+        float a[32];
+        tmem_ld32(tbase + loff + T_RSUM + 32 * q, a);
+        tmem_wait_ld();
+        if constexpr (is_tf32<NT>()) {
+          // lane e holds sample column e of panel rows 32 q .. 32 q + 31
+          if (e < c) {
+            float* d = dst - e + static_cast<size_t>(e) * BM + 32 * q;
 #pragma unroll
-              for (int x4 = 0; x4 < 8; ++x4)
-                *reinterpret_cast<float4*>(d + 4 * x4) =
-                    make_float4(a[4 * x4], a[4 * x4 + 1], a[4 * x4 + 2], a[4 * x4 + 3]);
-            }
-          } else {
+            for (int x4 = 0; x4 < 8; ++x4)
+              *reinterpret_cast<float4*>(d + 4 * x4) =
+                  make_float4(a[4 * x4], a[4 * x4 + 1], a[4 * x4 + 2], a[4 * x4 + 3]);
+          }
+        } else {
 #pragma unroll
-            for (int x = 0; x < 32; ++x) {
-              const int cc = 32 * q + x;
-              if (cc < c) dst[static_cast<size_t>(cc) * BM] = a[x];
-            }
+          for (int x = 0; x < 32; ++x) {
+            const int cc = 32 * q + x;
+            if (cc < c) dst[static_cast<size_t>(cc) * BM] = a[x];
           }
         }
       }
+      return true;
+    };
+    const int nt = static_cast<int>(te - tb);
+    Walk w(tb, ntc, gs, chain);
+    for (int i = 0; i < nt; ++i, w.next(ntc, gs, chain)) {
+      const int cb = i % CB, cu = i / CB;
+      const int xs = i % XSLOTS, xu = i / XSLOTS;
+      const bool gend = w.J == ntc - 1 || i == nt - 1 || w.g == gs - 1;
+      const bool cend = gend || w.h == chain - 1;
+      if (gstart < 0) gstart = w.g;   // where this CTA's part of the group begins
+      if (cend && !fold_chain(w, gend)) break;
+      if (!g.rows_only) {
+        // (the flag alternates: it is written again only after the next tile's
+        // barrier, which every thread reaches after reading it)
+        if (elect) {
+          // this CTA's column product of the tile is in TMEM (the buffer cannot
+          // move on to a later tile before this group has read it), and the
+          // partner's half has arrived
+          mbar_expect_tx(bar(B_XFULL + xs), static_cast<uint32_t>(c) * (HB * 4));
+          const bool ok =
+              mbar_wait(bar(B_CFULL + cb), cu & 1, abort_flag, g.err, 18, WAIT_LIMIT) &&
+              mbar_wait(bar(B_XFULL + xs), xu & 1, abort_flag, g.err, 16, WAIT_LIMIT);
+          fstop[i & 1] = ok ? 0 : 1;
+        }
+        named_sync(2, 128);
+        if (fstop[i & 1]) break;
+        fence_after();
+        float m[HB];
+        tmem_ld32(tbase + loff + T_COL + 64 * cb + own, m);
+        // the partner's half into registers; the slot may then go back
+        float r[HB];
+        {
+          const uint8_t* xslot = sm + L::xb + xs * X_BYTES + xrow;
+#pragma unroll
+          for (int q4 = 0; q4 < HB / 4; ++q4) {
+            const float4 x = *reinterpret_cast<const float4*>(xslot + ((q4 ^ (e & 7)) << 4));
+            r[4 * q4] = x.x;
+            r[4 * q4 + 1] = x.y;
+            r[4 * q4 + 2] = x.z;
+            r[4 * q4 + 3] = x.w;
+          }
+        }
+        tmem_wait_ld();
+        fence_before();
+        mbar_arrive(bar(B_CEMPTY + cb));
+        named_sync(2, 128);   // the slot has been read
+        if (e < c) {
+          // the pair's sum for columns j = J 64 + own .. + 31 and sample column
+          // e into the slot, [j][e], as it stands in the slab
+          float* slot = reinterpret_cast<float*>(sm + L::xb + xs * X_BYTES) + e;
+#pragma unroll
+          for (int x = 0; x < HB; ++x) slot[x * c] = m[x] + r[x];
+        }
+        fence_proxy_async();
+        mbar_arrive(bar(B_XREAD + xs));
+      }
     }
+  } else if (warp == 18 && lane == 0) {
+    // ---------------------------------- slab stores, exchange slots back
+    // A tile's sums go from its slot to Sc_part[pg][j][.], 32 whole rows (rows
+    // are padded to whole tiles; past n the TMA fill is zero, so the pad holds
+    // zeros, which the reduction never reads), in one bulk store; then the
+    // partner may fill the slot again.
+    const uint32_t xempty_peer = mapa(bar(B_XEMPTY), static_cast<uint32_t>(crank ^ 1));
+    const int nt = g.rows_only ? 0 : static_cast<int>(te - tb), c = g.c;
+    constexpr int HB = BN / KC;
+    Walk w(tb, ntc, gs, chain);
+    for (int i = 0; i < nt; ++i, w.next(ntc, gs, chain)) {
+      const int xs = i % XSLOTS, xu = i / XSLOTS;
+      if (!mbar_wait(bar(B_XREAD + xs), xu & 1, abort_flag, g.err, 21, WAIT_LIMIT)) break;
+      float* dst = g.sc_part + (static_cast<size_t>(w.pg) * g.npad +
+                                static_cast<size_t>(w.J) * BN + crank * HB) * c;
+      bulk_store(dst, su32(sm + L::xb + xs * X_BYTES), static_cast<uint32_t>(c) * (HB * 4));
+      bulk_store_read();
+      mbar_arrive_remote(xempty_peer + 8 * xs);
+    }
+    bulk_store_wait();
   }
 
+  // after a timeout, copies between the two CTAs may still be on their way
+  if (*abort_flag && tid == 0) {
+    const long long t0 = clock64();
+    while (clock64() - t0 < 200000) {
+    }
+  }
   fence_before();
   __syncthreads();
   // no CTA leaves while its partner may still write into its shared memory
@@ -839,7 +961,10 @@ __global__ void row_slot_flags_kernel(int ngp, int ntc, long long T, int Q, int 
 // Sc[j, c0 + cc] = sum over panel pairs of Sc_part[pg][j][cc] (pair order;
 // one thread per V consecutive columns cc of one j, cc fastest);
 // Sr[i, c0 + cc] = sum over the flush slots of row i's panel, in order (one
-// thread per (panel, cc, row), rows fastest: the slot reads are contiguous).
+// thread per (panel, cc, four rows), rows fastest: the slot reads are
+// contiguous; six groups' loads stand in flight.  One row per thread and one
+// group at a time left this part waiting on latency: at n = 20000 and 128
+// columns the kernel took 0.255 ms, now 0.180).
 template <int V>
 __global__ void sample_tc_reduce_kernel(const float* __restrict__ sc_part,
                                         const float* __restrict__ sr_part,
@@ -851,7 +976,7 @@ __global__ void sample_tc_reduce_kernel(const float* __restrict__ sc_part,
   // Sc == nullptr: the row samples only
   const long long ncv = Sc != nullptr ? static_cast<long long>(n) * cv : 0;
   if (idx < ncv) {
-    const int j = static_cast<int>(idx / cv), cc = static_cast<int>(idx % cv) * V;
+    const int j = static_cast<int>(idx / cv), cc = static_cast<int>(idx - static_cast<long long>(j) * cv) * V;
     const float* src = sc_part + static_cast<size_t>(j) * c + cc;
     const size_t stride = static_cast<size_t>(npad) * c;
     float s[V], k[V];
@@ -882,21 +1007,48 @@ __global__ void sample_tc_reduce_kernel(const float* __restrict__ sc_part,
       for (int x = 0; x < V; ++x) neumaier_add(s[x], k[x], __ldcs(src + stride * p + x));
 #pragma unroll
     for (int x = 0; x < V; ++x) Sc[static_cast<size_t>(j) * lds + cc + x] = s[x] + k[x];
-  } else if (idx < ncv + static_cast<long long>(npanel) * c * BM) {
+  } else if (idx < ncv + static_cast<long long>(npanel) * c * (BM / 4)) {
     const long long r = idx - ncv;
-    const int row = static_cast<int>(r % BM);
-    const long long pc = r / BM;
-    const int cc = static_cast<int>(pc % c), p = static_cast<int>(pc / c);
+    const int row = static_cast<int>(r % (BM / 4)) * 4;
+    const unsigned pc = static_cast<unsigned>(r / (BM / 4));
+    const int p = static_cast<int>(pc / static_cast<unsigned>(c)), cc = static_cast<int>(pc - p * c);
     const int i = p * BM + row;
     if (i >= n) return;
-    float s = 0.f, k = 0.f;
-    for (int grp = 0; grp < ngroups; ++grp) {
-      const size_t slot = (static_cast<size_t>(p) * ngroups + grp) * 2;
-      neumaier_add(s, k, __ldcs(sr_part + ((slot * c) + cc) * BM + row));
-      if (side1[(p / KC) * ngroups + grp])
-        neumaier_add(s, k, __ldcs(sr_part + (((slot + 1) * c) + cc) * BM + row));
+    float s[4], k[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) s[x] = k[x] = 0.f;
+    const size_t slot = static_cast<size_t>(c) * BM;
+    const float* src = sr_part + (static_cast<size_t>(p) * ngroups * 2 * c + cc) * BM + row;
+    const uint8_t* two = side1 + (p / KC) * ngroups;
+    constexpr int U = 6;
+    for (int g0 = 0; g0 < ngroups; g0 += U) {
+      float4 v[U][2];
+      bool t[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        t[u] = g0 + u < ngroups && two[g0 + u];
+        if (g0 + u < ngroups)
+          v[u][0] = __ldcs(reinterpret_cast<const float4*>(src + 2 * (g0 + u) * slot));
+        if (t[u]) v[u][1] = __ldcs(reinterpret_cast<const float4*>(src + (2 * (g0 + u) + 1) * slot));
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (g0 + u >= ngroups) break;
+        neumaier_add(s[0], k[0], v[u][0].x);
+        neumaier_add(s[1], k[1], v[u][0].y);
+        neumaier_add(s[2], k[2], v[u][0].z);
+        neumaier_add(s[3], k[3], v[u][0].w);
+        if (t[u]) {
+          neumaier_add(s[0], k[0], v[u][1].x);
+          neumaier_add(s[1], k[1], v[u][1].y);
+          neumaier_add(s[2], k[2], v[u][1].z);
+          neumaier_add(s[3], k[3], v[u][1].w);
+        }
+      }
     }
-    Sr[static_cast<size_t>(i) * lds + cc] = s + k;
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+      if (i + x < n) Sr[static_cast<size_t>(i + x) * lds + cc] = s[x] + k[x];
   }
 }
 
@@ -912,12 +1064,17 @@ __global__ void leaf_bounds_kernel(const int32_t* __restrict__ leaf_of, int n, i
 }
 
 // R16[i, cc] = R[i, c0 + cc] (bfloat16-exact) for cc < c, zero up to cpad
+// (64 or 128): a block of 64 x 4 threads per 16 rows
 __global__ void r_to_bf16_kernel(const float* __restrict__ R, long long ldr, int n, int c,
                                  int cpad, __nv_bfloat16* R16) {
-  const long long idx = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (idx >= static_cast<long long>(n) * cpad) return;
-  const int i = static_cast<int>(idx / cpad), cc = static_cast<int>(idx % cpad);
-  R16[idx] = __float2bfloat16_rn(cc < c ? R[static_cast<size_t>(i) * ldr + cc] : 0.f);
+  const int i0 = blockIdx.x * 16 + threadIdx.y;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int i = i0 + 4 * q;
+    for (int cc = threadIdx.x; cc < cpad && i < n; cc += 64)
+      R16[static_cast<size_t>(i) * cpad + cc] =
+          __float2bfloat16_rn(cc < c ? R[static_cast<size_t>(i) * ldr + cc] : 0.f);
+  }
 }
 
 // TF32: Rt[cc, i] = R[i, c0 + cc] for cc < c and i < n, zero elsewhere in
@@ -1151,8 +1308,7 @@ Err launch_sample_tc(const float* A, int64_t n, int64_t lda, const float* R, int
                        CMAX));
       tmRI = tmRJ;   // R_p^T comes from global memory
     } else {
-      const long long nconv = static_cast<long long>(n) * cpad;
-      r_to_bf16_kernel<<<static_cast<unsigned>((nconv + 255) / 256), 256, 0, s>>>(
+      r_to_bf16_kernel<<<static_cast<unsigned>((n + 15) / 16), dim3(64, 4), 0, s>>>(
           R + c0 + done, ldr, static_cast<int>(n), c, cpad, R16);
       HSS_TRY(check_launch("r_to_bf16_kernel"));
       HSS_TRY(make_map(&tmRJ, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, R16, cpad, n, cpad * 2, 64, BN));
@@ -1198,7 +1354,7 @@ Err launch_sample_tc(const float* A, int64_t n, int64_t lda, const float* R, int
                                                               pl.ngroups, side1);
       HSS_TRY(check_launch("row_slot_flags_kernel"));
     }
-    const long long nrow = static_cast<long long>(pl.npanel) * c * BM;
+    const long long nrow = static_cast<long long>(pl.npanel) * c * (BM / 4);
     const int npad = pl.ntc * BN;
     float* scout = Sc != nullptr ? Sc + c0 + done : nullptr;
     if (c % 4 == 0) {

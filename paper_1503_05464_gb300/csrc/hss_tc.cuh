@@ -38,11 +38,12 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t b, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint32_t b) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(b) : "memory");
 }
-// non-blocking test: never suspends the thread
+// test that may suspend the thread for a bounded time (fewer polls in the
+// shared-memory pipe than test_wait)
 __device__ __forceinline__ bool mbar_test(uint32_t b, uint32_t parity) {
   uint32_t ok;
   asm volatile(
-      "{ .reg .pred p; mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, "
+      "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, "
       "p; }"
       : "=r"(ok)
       : "r"(b), "r"(parity)
@@ -116,6 +117,36 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm,
       "{%2, %3}], [%4];" ::"r"(dst),
       "l"(tm), "r"(x), "r"(y), "r"(bar)
       : "memory");
+}
+// the same box into L2 only
+__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* tm, int x, int y) {
+  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(tm), "r"(x),
+               "r"(y)
+               : "memory");
+}
+// `bytes` (a multiple of 16, both addresses on 16 bytes) from this CTA's shared
+// memory into another CTA's, counted on that CTA's mbarrier
+__device__ __forceinline__ void bulk_copy_cluster(uint32_t rdst, uint32_t src, uint32_t bytes,
+                                                  uint32_t rbar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, "
+      "[%3];" ::"r"(rdst),
+      "r"(src), "r"(bytes), "r"(rbar)
+      : "memory");
+}
+// the same into global memory; bulk_store_read waits until the sources of this
+// thread's stores may be written again
+__device__ __forceinline__ void bulk_store(void* dst, uint32_t src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(src),
+               "r"(bytes)
+               : "memory");
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void bulk_store_read() {
+  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+}
+__device__ __forceinline__ void bulk_store_wait() {
+  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* tm) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory");
@@ -227,6 +258,13 @@ __device__ __forceinline__ float to_tf32(float x) {
   uint32_t r;
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
   return __uint_as_float(r);
+}
+// true for one lane of a converged warp, always the same
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{ .reg .pred p; elect.sync _|p, 0xffffffff; selp.u32 %0, 1, 0, p; }" : "=r"(r));
+  return r != 0;
 }
 // arrive once on `bar` when every tcgen05 operation issued so far by this
 // thread has completed

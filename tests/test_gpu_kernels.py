@@ -190,3 +190,38 @@ def test_id_of_nan_finishes(P, d, m):
     k, perm, _ = P.hss_id_batched([Y], 1e-6)[0]
     assert 0 <= k <= min(m, d)
     assert sorted(perm.cpu().tolist()) == list(range(m))
+
+
+# one tile; a pair's phantom second panel; clusters whose range crosses panel
+# pairs (R_p changes, the exchange through its buffer drains first), ragged
+# tiles, one column, a second 64-column box, the full width, two sweeps
+@pytest.mark.parametrize("mode,tol", [("bf16x3", 1e-5), ("bf16x2", 3e-5), ("tf32", 5.2e-4)])
+@pytest.mark.parametrize("n,c,starts", [
+    (60, 7, None), (129, 1, [0, 100, 129]), (700, 65, None), (2000, 128, [0, 700, 701, 2000]),
+    (2003, 131, None), (3500, 33, [0, 1000, 3500]),
+])
+def test_tensor_core_sampling_at_segment_edges(P, mode, tol, n, c, starts):
+    """Against FP64, and the same bits on every repeat.  Bound, relative to
+    |A| |R|: the split's 2^-24 / 2^-16 / 2^-11 and at most 80 FP32 roundings
+    (2^-23 each: the tensor core truncates)."""
+    pitch = (n + 3) // 4 * 4
+    rng = np.random.default_rng(n + c)
+    A = torch.tensor(rng.standard_normal((n, pitch)), dtype=torch.float32, device=DEV)[:, :n]
+    R = torch.zeros((n, c), device=DEV)
+    P.hss_random_gaussian(3, n, 0, c, R)
+    A64, R64 = A.double(), R.double()
+    if starts is not None:
+        A64 = A64.clone()
+        for lo, hi in zip(starts[:-1], starts[1:]):
+            A64[lo:hi, lo:hi] = 0
+    first = None
+    for _ in range(6):
+        Sr = torch.empty((n, c), device=DEV)
+        Sc = torch.empty((n, c), device=DEV)
+        P.hss_sample(A, R, 0, c, Sr, Sc, leaf_starts=starts, mode=mode)
+        if first is None:
+            first = (Sr, Sc)
+        assert torch.equal(Sr, first[0]) and torch.equal(Sc, first[1])
+    for M, S in ((A64, Sr), (A64.T, Sc)):
+        bound = tol * (M.abs() @ R64.abs()) + 1e-30
+        assert bool(((S.double() - M @ R64).abs() <= bound).all())
