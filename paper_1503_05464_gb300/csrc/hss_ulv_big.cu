@@ -14,8 +14,8 @@
 //           (I - V^T T V = H_i0 ... H_i1) by a cluster of CTAs that split its
 //           columns (lq_panel_kernel), then the trailing rows of W and all of
 //           Vhat^T -- whose rows the reflectors turn into Vtilde^T =
-//           (Q Vhat)^T -- in one launch: R <- R - ((R V^T) T) V, a CTA per 32
-//           rows (lq_update_kernel);
+//           (Q Vhat)^T -- in one launch: R <- R - ((R V^T) T) V, a CTA per 8
+//           to 32 rows (lq_update_kernel);
 //   root    right-looking blocked LU with partial pivoting: the panel by a
 //           cluster that splits its rows (lu_panel_kernel), the block row by
 //           the inverse of the panel's unit triangle, GEMM update of the rest.
@@ -31,6 +31,7 @@
 
 #include <algorithm>
 #include <climits>
+#include <functional>
 
 namespace cg = cooperative_groups;
 
@@ -335,7 +336,7 @@ __global__ void __launch_bounds__(B_THREADS) lq_panel_kernel(const LqPanel* item
 }
 
 // Rows [0, rows) of R (ld ldr, wid columns) <- R - ((R V^T) T) V with V nbb x
-// wid (ld ldv), T NB x NB upper triangular: one CTA per 32 rows.
+// wid (ld ldv), T NB x NB upper triangular: one CTA per 8 NR rows.
 struct UpdItem {
   double* R;
   const double* V;
@@ -352,121 +353,149 @@ __device__ __forceinline__ void u_cp(void* dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(BYTES));
 }
 
-// Measured: 39 ms of 31 GFLOP of updates in the factorization of a Schur
-// complement of n = 10,000 (0.64 of the FP64 rate; the products they replace
-// took 95 ms).
 // Both products of a row block in one pass, so that the panel's update of W
 // and Vhat^T is one launch (it was six GEMM launches a panel, three of them
-// with a few CTAs: g = V Vhat has 32 rows).  Bound: FP64 FMAs; every thread
-// keeps 4 (first product) or 8 (second) independent sums, the next stage of R
-// and V is on its way while the current one is multiplied.
+// with a few CTAs: g = V Vhat has 32 rows).  Warp w keeps rows w, w + 8, ...;
+// a lane is a row of V in the first product, two columns of a stage in the
+// second, so that no lane of an FP64 instruction is idle whatever NR is.
+// The next stage of R and V is on its way while the current one is multiplied.
+// Bound: FP64 FMAs, and how evenly the row blocks fall on the SMs: 31 GFLOP of
+// updates in the factorization of a Schur complement of n = 10,000 took 95 ms
+// as GEMMs, 39 ms by blocks of 32 rows (200 blocks on 152 SMs take as long as
+// 304), and take 30 ms by blocks of 8 to 32 (see launch_updates).  A row's
+// sums run in the order of its columns, whatever its block.
+template <int NR>
 __global__ void __launch_bounds__(B_THREADS)
 lq_update_kernel(const UpdItem* __restrict__ items, const int2* __restrict__ map) {
+  constexpr int BR = 8 * NR;
   extern __shared__ double usm[];
-  double* Rs = usm;                    // [2][32][UP]
-  double* Vs = Rs + 2 * NB * UP;       // [2][32][UP]
-  __shared__ double Ys[NB][NB + 1];
-  __shared__ double Y2[NB][NB + 1];
+  double* Rs = usm;                    // [2][BR][UP]
+  double* Vs = Rs + 2 * BR * UP;       // [2][32][UP]
+  __shared__ double Ys[BR][NB + 1];
+  __shared__ double Y2[BR][NB + 1];
   __shared__ double Ts[NB][NB + 1];
   const int2 tm = map[blockIdx.x];
   const UpdItem it = items[tm.x];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int r0 = tm.y * NB, rows = min(NB, it.rows - r0), wid = it.wid, nbb = it.nbb;
+  const int r0 = tm.y * BR, rows = min(BR, it.rows - r0), wid = it.wid, nbb = it.nbb;
   double* R = it.R + static_cast<int64_t>(r0) * it.ldr;
   const int nst = (wid + UK - 1) / UK;
-  const bool hi = rows > 16;   // else the second half of the block has no work
-  auto load_rows = [&](double* dst, const double* src, int64_t ld, int nr, int c0) {
-    for (int e = tid; e < NB * UK; e += B_THREADS) {
+  const int na = (rows + 7) / 8;   // rows w + 8 a, a >= na, have no work in any warp
+  auto load_rows = [&](double* dst, const double* src, int64_t ld, int nr, int nall, int c0) {
+    for (int e = tid; e < nall * UK; e += B_THREADS) {
       const int r = e / UK, c = e - r * UK;
       if (r < nr && c0 + c < wid) u_cp<8>(dst + r * UP + c, src + r * ld + c0 + c);
       else dst[r * UP + c] = 0.0;
     }
   };
   for (int e = tid; e < NB * NB; e += B_THREADS) Ts[e / NB][e % NB] = it.T[e];
-  load_rows(Rs, R, it.ldr, rows, 0);
-  load_rows(Vs, it.V, it.ldv, nbb, 0);
+  load_rows(Rs, R, it.ldr, rows, BR, 0);
+  load_rows(Vs, it.V, it.ldv, nbb, NB, 0);
   asm volatile("cp.async.commit_group;");
-  const int tx = tid & 15, ty = tid >> 4;
-  double y[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+  double y[NR];
+#pragma unroll
+  for (int a = 0; a < NR; ++a) y[a] = 0.0;
   for (int k = 0; k < nst; ++k) {
     const int b = k & 1;
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
     if (k + 1 < nst) {
-      load_rows(Rs + (b ^ 1) * NB * UP, R, it.ldr, rows, (k + 1) * UK);
-      load_rows(Vs + (b ^ 1) * NB * UP, it.V, it.ldv, nbb, (k + 1) * UK);
+      load_rows(Rs + (b ^ 1) * BR * UP, R, it.ldr, rows, BR, (k + 1) * UK);
+      load_rows(Vs + (b ^ 1) * NB * UP, it.V, it.ldv, nbb, NB, (k + 1) * UK);
       asm volatile("cp.async.commit_group;");
     }
-    const double* rs = Rs + b * NB * UP;
-    const double* vs = Vs + b * NB * UP;
+    const double* rs = Rs + b * BR * UP + w * UP;
+    const double* vs = Vs + b * NB * UP + lane * UP;
     const int lim = min(UK, wid - k * UK);
+    if (na == NR) {
 #pragma unroll 4
-    for (int c = 0; c < lim; ++c) {
-      const double v_0 = vs[tx * UP + c], v_1 = vs[(tx + 16) * UP + c];
-      const double r_0 = rs[ty * UP + c];
-      y[0][0] = fma(r_0, v_0, y[0][0]);
-      y[0][1] = fma(r_0, v_1, y[0][1]);
-      if (hi) {
-        const double r_1 = rs[(ty + 16) * UP + c];
-        y[1][0] = fma(r_1, v_0, y[1][0]);
-        y[1][1] = fma(r_1, v_1, y[1][1]);
+      for (int c = 0; c < lim; ++c) {
+        const double v = vs[c];
+#pragma unroll
+        for (int a = 0; a < NR; ++a) y[a] = fma(rs[8 * a * UP + c], v, y[a]);
+      }
+    } else {
+#pragma unroll 4
+      for (int c = 0; c < lim; ++c) {
+        const double v = vs[c];
+#pragma unroll
+        for (int a = 0; a + 1 < NR; ++a)
+          if (a < na) y[a] = fma(rs[8 * a * UP + c], v, y[a]);
       }
     }
   }
   __syncthreads();
   // V's first stage again, for the second product
-  load_rows(Vs, it.V, it.ldv, nbb, 0);
+  load_rows(Vs, it.V, it.ldv, nbb, NB, 0);
   asm volatile("cp.async.commit_group;");
 #pragma unroll
-  for (int a = 0; a < 2; ++a)
-#pragma unroll
-    for (int b = 0; b < 2; ++b) Ys[ty + 16 * a][tx + 16 * b] = y[a][b];
+  for (int a = 0; a < NR; ++a) Ys[w + 8 * a][lane] = y[a];
   __syncthreads();
-  {   // Y T: lane = row, warp w columns 4 w .. 4 w + 3, whose T ends at row 4 w + 3
-    double z[4] = {0.0, 0.0, 0.0, 0.0};
+  {   // Y T: warp w has columns 4 w .. 4 w + 3, whose T ends at row 4 w + 3; the
+      // lanes are the block's rows, times two or four groups of columns when
+      // there are few
+    constexpr int G = NR == 1 ? 4 : NR == 2 ? 2 : 1, CG = 4 / G;
+    const int row = G == 1 ? min(lane, BR - 1) : lane & (BR - 1);
+    const int c0 = 4 * w + (G == 1 ? 0 : lane / BR * CG);
+    double z[CG];
+#pragma unroll
+    for (int q = 0; q < CG; ++q) z[q] = 0.0;
     for (int l = 0; l < 4 * w + 4; ++l) {
-      const double v = Ys[lane][l];
+      const double v = Ys[row][l];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) z[q] = fma(v, Ts[l][4 * w + q], z[q]);
+      for (int q = 0; q < CG; ++q) z[q] = fma(v, Ts[l][c0 + q], z[q]);
     }
+    if (G > 1 || lane < BR)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) Y2[lane][4 * w + q] = z[q];
+      for (int q = 0; q < CG; ++q) Y2[row][c0 + q] = z[q];
   }
   for (int k = 0; k < nst; ++k) {
     const int b = k & 1;
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
     if (k + 1 < nst) {
-      load_rows(Vs + (b ^ 1) * NB * UP, it.V, it.ldv, nbb, (k + 1) * UK);
+      load_rows(Vs + (b ^ 1) * NB * UP, it.V, it.ldv, nbb, NB, (k + 1) * UK);
       asm volatile("cp.async.commit_group;");
     }
-    const double* vs = Vs + b * NB * UP;
-    double o[2][4];
+    const double* vs = Vs + b * NB * UP + lane;
+    double o[NR][2];
 #pragma unroll
-    for (int a = 0; a < 2; ++a)
+    for (int a = 0; a < NR; ++a)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int r = ty + 16 * a, c = k * UK + tx + 16 * q;
+      for (int q = 0; q < 2; ++q) {
+        const int r = w + 8 * a, c = k * UK + lane + 32 * q;
         o[a][q] = (r < rows && c < wid) ? R[r * it.ldr + c] : 0.0;
       }
-    // (columns past wid add zeros; a block of 16 columns past it is skipped)
-    const int nq = (min(UK, wid - k * UK) + 15) / 16;
+    // (columns past wid add zeros; a block of 32 columns past it is skipped)
+    const bool two = wid - k * UK > 32;
+    if (two && na == NR) {
+#pragma unroll 4
+      for (int l = 0; l < nbb; ++l) {
+        const double v0 = vs[l * UP], v1 = vs[l * UP + 32];
+#pragma unroll
+        for (int a = 0; a < NR; ++a) {
+          const double f = -Y2[w + 8 * a][l];
+          o[a][0] = fma(f, v0, o[a][0]);
+          o[a][1] = fma(f, v1, o[a][1]);
+        }
+      }
+    } else
 #pragma unroll 4
     for (int l = 0; l < nbb; ++l) {
-      const double a0 = -Y2[ty][l], a1 = -Y2[ty + 16][l];
+      const double v0 = vs[l * UP], v1 = vs[l * UP + 32];
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (q < nq) {
-          const double v = vs[l * UP + tx + 16 * q];
-          o[0][q] = fma(a0, v, o[0][q]);
-          if (hi) o[1][q] = fma(a1, v, o[1][q]);
+      for (int a = 0; a < NR; ++a)
+        if (a < na) {
+          const double f = -Y2[w + 8 * a][l];
+          o[a][0] = fma(f, v0, o[a][0]);
+          if (two) o[a][1] = fma(f, v1, o[a][1]);
         }
     }
 #pragma unroll
-    for (int a = 0; a < 2; ++a)
+    for (int a = 0; a < NR; ++a)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int r = ty + 16 * a, c = k * UK + tx + 16 * q;
+      for (int q = 0; q < 2; ++q) {
+        const int r = w + 8 * a, c = k * UK + lane + 32 * q;
         if (r < rows && c < wid) R[r * it.ldr + c] = o[a][q];
       }
   }
@@ -857,23 +886,60 @@ Err launch_panels(const std::vector<Item>& all, void (*const kern[4])(const Item
   return ok();
 }
 
+// Rows per block: 8, 16, 24 or 32, whichever lets the launch end first with its
+// blocks handed to the SMs as they become free (longest first).  A block costs
+// its width times its rows, in eights, and 0.06 of its width for what does not
+// shrink with the rows (V's stages, barriers); if some SM gets a second block,
+// half of the longest on top (blocks resident together end together, so the
+// rounds are coarser than that).  With eight blocks of 32 rows or more per SM
+// the last round no longer matters.
 Err launch_updates(const std::vector<UpdItem>& items, cudaStream_t s, Arena& ar) {
   std::vector<UpdItem> live;
-  std::vector<int2> map;
-  for (const UpdItem& u : items) {
-    if (u.rows <= 0) continue;
-    for (int t = 0; t * NB < u.rows; ++t) map.push_back(make_int2((int)live.size(), t));
-    live.push_back(u);
+  for (const UpdItem& u : items)
+    if (u.rows > 0) live.push_back(u);
+  if (live.empty()) return ok();
+  std::stable_sort(live.begin(), live.end(),
+                   [](const UpdItem& a, const UpdItem& b) { return a.wid > b.wid; });
+  int dev = 0, sms = 0;
+  HSS_CUDA_TRY(cudaGetDevice(&dev));
+  HSS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  int64_t rows32 = 0;
+  for (const UpdItem& u : live) rows32 += (u.rows + 31) / 32;
+  int best = 4;
+  if (rows32 < 8 * sms) {
+    double best_t = 0.0;
+    std::vector<double> end;
+    for (int nr = 4; nr >= 1; --nr) {
+      end.assign(static_cast<size_t>(sms), 0.0);   // a heap: the SM free first on top
+      double t = 0.0;
+      int blocks = 0;
+      for (const UpdItem& u : live)
+        for (int r0 = 0; r0 < u.rows; r0 += 8 * nr, ++blocks) {
+          std::pop_heap(end.begin(), end.end(), std::greater<double>());
+          end.back() += u.wid * ((std::min(8 * nr, u.rows - r0) + 7) / 8 + 0.06);
+          t = std::max(t, end.back());
+          std::push_heap(end.begin(), end.end(), std::greater<double>());
+        }
+      if (blocks > sms) t += 0.5 * nr * live.front().wid;
+      if (nr == 4 || t < best_t) {
+        best = nr;
+        best_t = t;
+      }
+    }
   }
-  if (map.empty()) return ok();
+  std::vector<int2> map;
+  for (size_t q = 0; q < live.size(); ++q)
+    for (int t = 0; t * 8 * best < live[q].rows; ++t) map.push_back(make_int2((int)q, t));
   UpdItem* di = nullptr;
   int2* dm = nullptr;
   HSS_TRY(upload(live, s, ar, &di));
   HSS_TRY(upload(map, s, ar, &dm));
-  const size_t smem = sizeof(double) * 4 * NB * UP;
-  HSS_CUDA_TRY(cudaFuncSetAttribute(lq_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  static void (*const kern[4])(const UpdItem*, const int2*) = {lq_update_kernel<1>, lq_update_kernel<2>,
+                                                               lq_update_kernel<3>, lq_update_kernel<4>};
+  const size_t smem = sizeof(double) * 2 * (NB + 8 * best) * UP;
+  HSS_CUDA_TRY(cudaFuncSetAttribute(kern[best - 1], cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)smem));
-  lq_update_kernel<<<(unsigned)map.size(), B_THREADS, smem, s>>>(di, dm);
+  kern[best - 1]<<<(unsigned)map.size(), B_THREADS, smem, s>>>(di, dm);
   return check_launch("lq_update_kernel");
 }
 

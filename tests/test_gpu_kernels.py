@@ -116,6 +116,23 @@ def test_ulv_factor_solve_at_panel_edges(P, n, leaf, rank):
     assert torch.equal(P.hss_solve(h, b), x)
 
 
+# few to many row blocks per launch: the update takes blocks of 8, 16, 24 or 32
+# rows, and a row's sums must not depend on it
+def test_ulv_factors_whatever_shares_the_launch(P):
+    import workloads as W
+    A = W.random_hss(1400, 350, 300, seed=9)[0]
+    At = torch.tensor(A, device=DEV)
+    hs = [P.hss_compress(At, leaf_size=350, rtol=1e-13, d0=320, d_step=32, seed=5) for _ in range(17)]
+    b = torch.randn(1400, 3, dtype=torch.float64, device=DEV,
+                    generator=torch.Generator(device=DEV).manual_seed(1))
+    P.hss_factor(hs[0])
+    x = P.hss_solve(hs[0], b)
+    for count in (2, 3, 5, 17):
+        P.hss_factor_batched(hs[:count])
+        for h in hs[:count]:
+            assert torch.equal(P.hss_solve(h, b), x)
+
+
 # one column to more than a launch's 64 (two slabs), in place, on handles with
 # 8-row tasks (nodes above 160 rows), partial blocks, rank-zero nodes and a
 # single-node tree; several handles of different widths together
