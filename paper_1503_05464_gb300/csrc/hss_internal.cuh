@@ -288,7 +288,7 @@ class GemmPlan {
  private:
   struct Phase {
     size_t items_off, starts_off;
-    int n, tiles, nc;
+    int n, tiles, nc, tm;
   };
   std::vector<char> host_;
   std::vector<Phase> phases_;

@@ -14,12 +14,13 @@
 #include <cstring>
 
 #include <algorithm>
+#include <functional>
 
 namespace hss {
 
 namespace {
 
-constexpr int G_TM = 64, G_TN = 64, G_TK = 16, G_THREADS = 256;
+constexpr int G_TN = 64, G_TK = 16, G_THREADS = 256;
 
 template <typename T>
 __device__ __forceinline__ const T* src_row(const RowSrc<T>& s, int r) {
@@ -35,12 +36,24 @@ __device__ __forceinline__ T mat_at(const GemmItem<T>& it, int j, int l) {
                      : reinterpret_cast<const T*>(it.M)[off];
 }
 
-template <typename T>
+// A block computes TM x 64 entries of an item, 16 inner indices per stage; the
+// next stage's values are loaded (through the row maps) before the current one
+// is multiplied, and stored to the other buffer after it.  An entry adds its
+// terms in increasing l, whatever the tile.
+// FP64: bound by the two FMAs a clock and SM, so a tile's last rows and columns
+// are trimmed to 16 (a thread's rows are 16 apart) and TM is chosen per launch
+// (gemm_rows below).  The 59 products of the factorization of a Schur
+// complement of n = 10,000 took 36.9 ms with 64 x 64 tiles filled by
+// synchronous loads, and take 32.1 ms.  FP32: 4 x 4 neighbouring entries
+// per thread (vector loads from shared memory).
+template <typename T, int TM>
 __global__ void __launch_bounds__(G_THREADS)
 gemm_batched_kernel(const GemmItem<T>* __restrict__ items, const int* __restrict__ tile_start,
                     int nitems) {
-  __shared__ T Ms[G_TM][G_TK + 1];
-  __shared__ T Zs[G_TK][G_TN];
+  constexpr int NR = TM / 16;          // rows per thread
+  constexpr bool D = sizeof(T) == 8;   // rows and columns 16 apart
+  __shared__ T Ms[2][TM][G_TK + 1];
+  __shared__ T Zs[2][G_TK][G_TN];
   // locate the item of this tile (binary search in the tile prefix)
   int lo = 0, hi = nitems - 1;
   const int b = blockIdx.x;
@@ -54,52 +67,91 @@ gemm_batched_kernel(const GemmItem<T>* __restrict__ items, const int* __restrict
   const int ncol = it.c1 - it.c0;
   const int tiles_c = (ncol + G_TN - 1) / G_TN;
   const int tr = local / tiles_c, tc = local - tr * tiles_c;
-  const int j0 = tr * G_TM, cb = it.c0 + tc * G_TN;
+  const int j0 = tr * TM, cb = it.c0 + tc * G_TN;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-
-  T acc[4][4];
+  // (16-row and 16-column blocks that exist)
+  const int nr = D ? min(NR, (it.rows - j0 + 15) / 16) : NR;
+  const int nc = D ? min(4, (it.c1 - cb + 15) / 16) : 4;
+  // what this thread loads of a stage: neighbouring threads take what is
+  // contiguous in memory
+  const int mr = it.m_trans ? tid % TM : tid / G_TK, ml = it.m_trans ? tid / TM : tid % G_TK;
+  const int mdr = it.m_trans ? 0 : G_THREADS / G_TK, mdl = it.m_trans ? G_THREADS / TM : 0;
+  const int zc = it.z_trans ? tid / G_TK : tid % G_TN, zl = it.z_trans ? tid % G_TK : tid / G_TN;
+  const int zdc = it.z_trans ? G_THREADS / G_TK : 0, zdl = it.z_trans ? 0 : G_THREADS / G_TN;
+  T mv[NR], zv[4];
+  auto load = [&](int l0) {
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+    for (int q = 0; q < NR; ++q) {
+      const int j = j0 + mr + q * mdr, ll = l0 + ml + q * mdl;
+      mv[q] = (j < it.rows && ll < it.inner) ? mat_at(it, j, ll) : T(0);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int ll = l0 + zl + q * zdl, cc = cb + zc + q * zdc;
+      zv[q] = T(0);
+      if (ll < it.inner && cc < it.c1)
+        zv[q] = it.z_trans ? src_row(it.Z, cc)[ll] : src_row(it.Z, ll)[cc];
+    }
+  };
+  auto store = [&](int s) {
+#pragma unroll
+    for (int q = 0; q < NR; ++q) Ms[s][mr + q * mdr][ml + q * mdl] = mv[q];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) Zs[s][zl + q * zdl][zc + q * zdc] = zv[q];
+  };
+  auto row = [&](int r) { return D ? ty + 16 * r : ty * NR + r; };
+  auto col = [&](int c) { return D ? tx + 16 * c : tx * 4 + c; };
+
+  T acc[NR][4];
+#pragma unroll
+  for (int a = 0; a < NR; ++a)
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc[a][q] = T(0);
 
-  for (int l0 = 0; l0 < it.inner; l0 += G_TK) {
+  if (it.inner > 0) {
+    load(0);
+    store(0);
+  }
+  __syncthreads();
+  for (int l0 = 0, s = 0; l0 < it.inner; l0 += G_TK, s ^= 1) {
+    const bool more = l0 + G_TK < it.inner;
+    if (more) load(l0 + G_TK);
+    if (nr == NR && nc == 4) {
+#pragma unroll
+      for (int l = 0; l < G_TK; ++l) {
+        T a[NR], z[4];
+#pragma unroll
+        for (int r = 0; r < NR; ++r) a[r] = Ms[s][row(r)][l];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) z[c] = Zs[s][l][col(c)];
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[r][c] = fma(a[r], z[c], acc[r][c]);
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < NR; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (r < nr && c < nc) {
+#pragma unroll
+            for (int l = 0; l < G_TK; ++l)
+              acc[r][c] = fma(Ms[s][row(r)][l], Zs[s][l][col(c)], acc[r][c]);
+          }
+    }
+    if (more) store(s ^ 1);
     __syncthreads();
-    for (int e = tid; e < G_TM * G_TK; e += G_THREADS) {
-      int r = e / G_TK, l = e - r * G_TK;
-      int j = j0 + r, ll = l0 + l;
-      Ms[r][l] = (j < it.rows && ll < it.inner) ? mat_at(it, j, ll) : T(0);
-    }
-    for (int e = tid; e < G_TK * G_TN; e += G_THREADS) {
-      int l = e / G_TN, c = e - l * G_TN;
-      int ll = l0 + l, cc = cb + c;
-      T v = T(0);
-      if (ll < it.inner && cc < it.c1) v = it.z_trans ? src_row(it.Z, cc)[ll] : src_row(it.Z, ll)[cc];
-      Zs[l][c] = v;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int l = 0; l < G_TK; ++l) {
-      T a[4], z[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) a[r] = Ms[ty * 4 + r][l];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) z[c] = Zs[l][tx * 4 + c];
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] = fma(a[r], z[c], acc[r][c]);
-    }
   }
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    int j = j0 + ty * 4 + r;
+  for (int r = 0; r < NR; ++r) {
+    int j = j0 + row(r);
     if (j >= it.rows) continue;
     const T* xr = it.X.p0 ? src_row(it.X, j) : nullptr;
     T* o = it.out + (int64_t)j * it.ldo;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      int cc = cb + tx * 4 + c;
+      int cc = cb + col(c);
       if (cc >= it.c1) continue;
       T v = it.sign * acc[r][c];
       if (xr) v += xr[cc];
@@ -241,10 +293,11 @@ gemm_narrow_kernel(const GemmItem<T>* __restrict__ items, const int2* __restrict
 // Launch shape of one batched GEMM: the 64 x 64 tile kernel (nc = 0), or the
 // narrow kernel with nc columns per block.
 struct GemmShape {
-  int nc;
+  int nc;        // 0: the tile kernel
+  int tm = 64;   // its rows per tile
   int tiles(int rows, int ncol) const {
     return nc ? ((rows + N_ROWS - 1) / N_ROWS) * ((ncol + nc - 1) / nc)
-              : ((rows + G_TM - 1) / G_TM) * ((ncol + G_TN - 1) / G_TN);
+              : ((rows + tm - 1) / tm) * ((ncol + G_TN - 1) / G_TN);
   }
 };
 
@@ -257,11 +310,60 @@ constexpr int NARROW_MAX = 32;
 
 template <typename T>
 struct GemmGroup {
-  GemmShape shape{0};
+  GemmShape shape{0, 64};
   std::vector<GemmItem<T>> live;
   std::vector<int> starts;   // tile kernel: first block of each item; narrow: (item, tile) pairs
   int tiles = 0;
 };
+
+// Rows per tile of an FP64 launch: 64, 32 or 16, whichever lets it end first
+// with its tiles handed to the SMs as they become free.  In units of 16 x 16
+// entries a tile costs its blocks and 0.6 for its loads and barriers, times the
+// inner length; if some SM gets a second tile, half of the largest on top
+// (tiles resident together end together).  With eight tiles of 64 rows or more
+// per SM the last round no longer matters.
+template <typename T>
+int gemm_rows(const std::vector<GemmItem<T>>& items, int lim) {
+  if (sizeof(T) != 8) return 64;
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return 64;
+  }
+  int64_t tiles = 0;
+  for (const auto& it : items)
+    if (it.rows > 0 && it.c1 - it.c0 > lim)
+      tiles += static_cast<int64_t>((it.rows + 63) / 64) * ((it.c1 - it.c0 + 63) / 64);
+  if (tiles == 0 || tiles >= 8 * sms) return 64;
+  int best = 64;
+  double best_t = 0.0;
+  std::vector<double> end;
+  for (int tm = 64; tm >= 16; tm /= 2) {
+    end.assign(static_cast<size_t>(sms), 0.0);   // a heap: the SM free first on top
+    double t = 0.0, largest = 0.0;
+    int count = 0;
+    for (const auto& it : items) {
+      if (it.rows <= 0 || it.c1 - it.c0 <= lim) continue;
+      for (int j = 0; j < it.rows; j += tm)
+        for (int c = it.c0; c < it.c1; c += 64, ++count) {
+          const int nr = (std::min(tm, it.rows - j) + 15) / 16, nc = (std::min(64, it.c1 - c) + 15) / 16;
+          const double cost = (nr * nc + 0.6) * (it.inner + 16);
+          std::pop_heap(end.begin(), end.end(), std::greater<double>());
+          end.back() += cost;
+          t = std::max(t, end.back());
+          largest = std::max(largest, cost);
+          std::push_heap(end.begin(), end.end(), std::greater<double>());
+        }
+    }
+    if (count > sms) t += 0.5 * largest;
+    if (tm == 64 || t < best_t) {
+      best = tm;
+      best_t = t;
+    }
+  }
+  return best;
+}
 
 template <typename T>
 void split_gemm(const std::vector<GemmItem<T>>& items, GemmGroup<T> g[2], bool narrow) {
@@ -270,6 +372,7 @@ void split_gemm(const std::vector<GemmItem<T>>& items, GemmGroup<T> g[2], bool n
   for (const auto& it : items)
     if (it.rows > 0 && it.c1 > it.c0 && it.c1 - it.c0 <= lim) mc = std::max(mc, it.c1 - it.c0);
   g[0].shape.nc = 0;
+  g[0].shape.tm = gemm_rows(items, lim);
   g[1].shape.nc = mc <= 1 ? 1 : mc == 2 ? 2 : mc <= 4 ? 4 : 8;
   for (const auto& it : items) {
     if (it.rows <= 0 || it.c1 <= it.c0) continue;
@@ -293,7 +396,13 @@ void launch_gemm_shape(GemmShape g, int tiles, const GemmItem<T>* items, const i
                        cudaStream_t s) {
   const int2* map = reinterpret_cast<const int2*>(starts);
   switch (g.nc) {
-    case 0: gemm_batched_kernel<T><<<tiles, G_THREADS, 0, s>>>(items, starts, n); break;
+    case 0:
+      if constexpr (sizeof(T) == 8) {
+        if (g.tm == 16) gemm_batched_kernel<T, 16><<<tiles, G_THREADS, 0, s>>>(items, starts, n);
+        if (g.tm == 32) gemm_batched_kernel<T, 32><<<tiles, G_THREADS, 0, s>>>(items, starts, n);
+      }
+      if (g.tm == 64) gemm_batched_kernel<T, 64><<<tiles, G_THREADS, 0, s>>>(items, starts, n);
+      break;
     case 1: gemm_narrow_kernel<T, 1><<<tiles, N_THREADS, 0, s>>>(items, map); break;
     case 2: gemm_narrow_kernel<T, 2><<<tiles, N_THREADS, 0, s>>>(items, map); break;
     case 4: gemm_narrow_kernel<T, 4><<<tiles, N_THREADS, 0, s>>>(items, map); break;
@@ -586,6 +695,7 @@ void GemmPlan<T>::add(const std::vector<GemmItem<T>>& items) {
     ph.n = static_cast<int>(g.live.size());
     ph.tiles = g.tiles;
     ph.nc = g.shape.nc;
+    ph.tm = g.shape.tm;
     phases_.push_back(ph);
   }
 }
@@ -598,7 +708,7 @@ Err GemmPlan<T>::run(cudaStream_t s) {
   HSS_TRY(upload_async(buf, host_.data(), host_.size(), s));
   Err e;
   for (const Phase& ph : phases_) {
-    launch_gemm_shape<T>(GemmShape{ph.nc}, ph.tiles,
+    launch_gemm_shape<T>(GemmShape{ph.nc, ph.tm}, ph.tiles,
                          reinterpret_cast<const GemmItem<T>*>(buf + ph.items_off),
                          reinterpret_cast<const int*>(buf + ph.starts_off), ph.n, s);
     e = check_launch(ph.nc ? "gemm_narrow_kernel" : "gemm_batched_kernel");

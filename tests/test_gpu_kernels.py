@@ -242,3 +242,21 @@ def test_tensor_core_sampling_at_segment_edges(P, mode, tol, n, c, starts):
     for M, S in ((A64, Sr), (A64.T, Sc)):
         bound = tol * (M.abs() @ R64.abs()) + 1e-30
         assert bool(((S.double() - M @ R64).abs() <= bound).all())
+
+
+# products of one tile and of many (tiles of 16, 32 and 64 rows), ragged rows,
+# columns and inner lengths: a factorization's D, Vhat, W and root updates
+@pytest.mark.parametrize("n,leaf,rank", [(131, 66, 5), (530, 133, 49), (2100, 525, 130), (3300, 413, 71)])
+def test_ulv_products_at_tile_edges(P, n, leaf, rank):
+    import workloads as W
+    A = W.random_hss(n, leaf, rank, seed=n, diag_shift=float(n))[0]
+    h = P.hss_compress(torch.tensor(A, device=DEV), leaf_size=leaf, rtol=1e-13, d0=rank + 20,
+                       d_step=32, seed=5)
+    P.hss_factor(h)
+    b = torch.randn(n, 2, dtype=torch.float64, device=DEV,
+                    generator=torch.Generator(device=DEV).manual_seed(n))
+    x = P.hss_solve(h, b)
+    # normwise backward error against the compressed form itself: 50 n u covers
+    # the LQ and LU with a growth factor of order ten
+    res = float(torch.linalg.norm(P.hss_matvec(h, x) - b))
+    assert res <= 50 * n * 2.0 ** -53 * float(np.linalg.norm(A)) * float(torch.linalg.norm(x))
