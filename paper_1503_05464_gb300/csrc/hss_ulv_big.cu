@@ -22,6 +22,7 @@
 // The factors have the per-node kernel's layout.
 // Every launch shape that a node's sums depend on follows from the node's own
 // order, so factors do not depend on what shares the launch.
+#include "hss_fp.cuh"
 #include "hss_internal.cuh"
 #include "hss_tree.h"
 
@@ -150,14 +151,16 @@ __device__ __forceinline__ double reduce_scatter4(double (&p)[4]) {
 // sends the partial sums a_i . a_j of all rows j >= i (and rank 0 the pivot
 // column) to its peers, and after one cluster barrier each has sigma, tau,
 // the scale of v and, as v is a multiple of a_i, every row's product with it.
-// Warp w owns rows w, w + 8, w + 16, w + 24.  The square root and divisions
-// run in one warp: any FP64 instruction holds its scheduler's pipe 64 cycles.
+// Warp w owns rows w, w + 8, w + 16, w + 24.  The square root and the quotients
+// run in one warp, on the integer pipes (hss_fp.cuh: the same bits; a lane's
+// FP64 root and divisions, one after the other, took 2100 of a step's 11,600
+// cycles; 56 panels 10.5 -> 9.9 ms).
 // T = D (I + U D)^{-1} with U the strict upper triangle of V V^T and D =
 // diag(tau) (the inverse of a unit triangle: no division, tau may be 0).
 //
 // Bound: FP64 latency (about 3 us a step).  One CTA per panel, which took the
 // sums from global memory and was bound by its SM's two FMAs a clock, needed
-// 530 us a panel at m = 1200 against 190.
+// 530 us a panel at m = 1200 against 180.
 template <int C>
 __global__ void __launch_bounds__(B_THREADS) lq_panel_kernel(const LqPanel* items, int in_smem) {
   extern __shared__ double lsm[];
@@ -223,19 +226,20 @@ __global__ void __launch_bounds__(B_THREADS) lq_panel_kernel(const LqPanel* item
       for (int o = C / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     }
     s = __shfl_sync(0xffffffffu, s, lane & 24);
-    if (w == (i & 7) && lane == 8 * (i >> 3)) {   // the owner of row i
-      const double sigma = sqrt(fma(al, al, s));
-      double tau = 0.0, beta = al, scal = 0.0;
-      if (s != 0.0) {
-        beta = -copysign(sigma, al);
-        tau = (beta - al) / beta;
-        scal = 1.0 / (al - beta);
+    if (w == (i & 7)) {   // the warp of row i: lanes 0 and 1 the two quotients
+      const double si = __shfl_sync(0xffffffffu, s, 8 * (i >> 3));
+      const double ali = __shfl_sync(0xffffffffu, al, 8 * (i >> 3));
+      double q = 0.0, beta = ali;
+      if (si != 0.0) {
+        beta = -copysign(fp_sqrt(fma(ali, ali, si)), ali);
+        q = fp_div(lane == 0 ? beta - ali : 1.0, lane == 0 ? beta : ali - beta);
       }
-      sh[0] = tau;
-      sh[1] = scal;
-      tq[i] = tau;
-      sc[i] = scal;
-      if (rank == 0) A[i * ld + i] = beta;
+      if (lane < 2) {
+        sh[lane] = q;
+        if (lane == 0) tq[i] = q;
+        else sc[i] = q;
+      }
+      if (rank == 0 && lane == 0) A[i * ld + i] = beta;
     }
     __syncthreads();
     const double tau = sh[0], scal = sh[1];
