@@ -1274,7 +1274,17 @@ Err launch_sample_tc(const float* A, int64_t n, int64_t lda, const float* R, int
   for (int64_t w = 0; w < nsw; ++w) {
     const int c = static_cast<int>((ncols - done) / (nsw - w));
     const int cpad = (c + 63) / 64 * 64;
+    // what does not depend on the sweep's width comes first: the leaf ranges are
+    // formed once, and widths may differ by one (131 columns: 65, 66)
     uint8_t* base = static_cast<uint8_t*>(scratch->part);
+    int* err = reinterpret_cast<int*>(base);
+    base += 256;
+    int32_t* leaf_lo = reinterpret_cast<int32_t*>(base);
+    base += align256(static_cast<size_t>(n) * 4);
+    int32_t* leaf_hi = reinterpret_cast<int32_t*>(base);
+    base += align256(static_cast<size_t>(n) * 4);
+    uint8_t* side1 = base;
+    base += align256(static_cast<size_t>(pl.ngp) * pl.ngroups);
     __nv_bfloat16* R16 = reinterpret_cast<__nv_bfloat16*>(base);
     float* Rt = reinterpret_cast<float*>(base);
     const int ldrt = 2 * pl.ngp * BM;
@@ -1282,14 +1292,6 @@ Err launch_sample_tc(const float* A, int64_t n, int64_t lda, const float* R, int
     float* scp = reinterpret_cast<float*>(base);
     base += align256(static_cast<size_t>(pl.ngp) * c * pl.ntc * BN * 4);
     float* srp = reinterpret_cast<float*>(base);
-    base += align256(static_cast<size_t>(pl.npanel) * pl.ngroups * 2 * c * BM * 4);
-    int32_t* leaf_lo = reinterpret_cast<int32_t*>(base);
-    base += align256(static_cast<size_t>(n) * 4);
-    int32_t* leaf_hi = reinterpret_cast<int32_t*>(base);
-    base += align256(static_cast<size_t>(n) * 4);
-    uint8_t* side1 = base;
-    base += align256(static_cast<size_t>(pl.ngp) * pl.ngroups);
-    int* err = reinterpret_cast<int*>(base);
     if (leaf_of != nullptr && w == 0) {
       leaf_bounds_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, s>>>(
           leaf_of, static_cast<int>(n), leaf_lo, leaf_hi);

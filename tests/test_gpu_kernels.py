@@ -260,3 +260,25 @@ def test_ulv_products_at_tile_edges(P, n, leaf, rank):
     # the LQ and LU with a growth factor of order ten
     res = float(torch.linalg.norm(P.hss_matvec(h, x) - b))
     assert res <= 50 * n * 2.0 ** -53 * float(np.linalg.norm(A)) * float(torch.linalg.norm(x))
+
+
+# sweeps of one call that differ in width (65 + 66 columns, 86 + 87 + 87, 106 +
+# 107 + 107) share the leaf mask; the last is as wide as a 128-column sweep gets
+@pytest.mark.parametrize("mode,tol", [("bf16x3", 1e-5), ("bf16x2", 3e-5), ("tf32", 5.2e-4)])
+@pytest.mark.parametrize("c", [131, 260, 320, 383])
+def test_tensor_core_sampling_masks_every_sweep(P, mode, tol, c):
+    n, starts = 1100, [0, 300, 301, 700, 1100]
+    rng = np.random.default_rng(c)
+    A = torch.tensor(rng.standard_normal((n, n)), dtype=torch.float32, device=DEV)
+    R = torch.zeros((n, c), device=DEV)
+    P.hss_random_gaussian(3, n, 0, c, R)
+    M = A.double()
+    for lo, hi in zip(starts[:-1], starts[1:]):
+        M[lo:hi, lo:hi] = 0
+    Sr, Sc, only = (torch.empty((n, c), device=DEV) for _ in range(3))
+    P.hss_sample(A, R, 0, c, Sr, Sc, leaf_starts=starts, mode=mode)
+    P.hss_sample(A, R, 0, c, only, None, leaf_starts=starts, mode=mode)
+    assert torch.equal(only, Sr)
+    R64 = R.double()
+    for W, S in ((M, Sr), (M.T, Sc)):   # the bound of the test above
+        assert bool(((S.double() - W @ R64).abs() <= tol * (W.abs() @ R64.abs()) + 1e-30).all())
