@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(U_THREADS) ulv_factor_kernel(const FacItem* it
           bv = redv[q];
           bi = redi[q];
         }
-      if (bv == 0.0) {
+      if (!(bv > 0.0)) {   // zeros and NaN only (then no row was chosen)
         if (tid == 0) *it.status = HSS_ERR_SINGULAR;
         return;
       }

@@ -634,7 +634,9 @@ __global__ void __launch_bounds__(B_THREADS) lu_panel_kernel(const LuPanel* item
       if (cv[slot][r] > cv[slot][win] ||
           (cv[slot][r] == cv[slot][win] && ci[slot][r] < ci[slot][win]))
         win = r;
-    if (cv[slot][win] <= 0) {   // a zero column (the same decision on every CTA)
+    // a zero column, or a NaN in it, whose bits are above every number's (the same
+    // decision on every CTA)
+    if (cv[slot][win] <= 0 || cv[slot][win] > __double_as_longlong(INFINITY)) {
       if (rank == 0 && tid == 0) *it.status = HSS_ERR_SINGULAR;
       sync_all();   // no CTA leaves while a peer may still write to it
       return;

@@ -282,3 +282,27 @@ def test_tensor_core_sampling_masks_every_sweep(P, mode, tol, c):
     R64 = R.double()
     for W, S in ((M, Sr), (M.T, Sc)):   # the bound of the test above
         assert bool(((S.double() - W @ R64).abs() <= tol * (W.abs() @ R64.abs()) + 1e-30).all())
+
+
+# a NaN leaves no pivot in some column of the root's LU: in one CTA (50 rows),
+# blocked over 1 to 8 CTAs, and from a leaf block below the root
+@pytest.mark.parametrize("n,leaf", [(50, 64), (63, 64), (64, 64), (100, 128), (300, 512), (700, 1024),
+                                    (100, 50), (400, 100)])
+@pytest.mark.parametrize("at", [(0, 0), (-1, -1), (3, 20)])
+def test_factor_of_nan_is_singular(P, n, leaf, at):
+    import workloads as W
+    A = torch.as_tensor(W.toeplitz_inv_distance(n), device=DEV).clone()
+    good = P.hss_compress(A, leaf_size=leaf)
+    A[at] = float("nan")          # (the sampling masks the leaf blocks: ranks as without it)
+    h = P.hss_compress(A, leaf_size=leaf)
+    with pytest.raises(P.HssError) as e:
+        P.hss_factor(h)
+    assert e.value.status == P.hss.HSS_ERR_SINGULAR
+    with pytest.raises(P.HssError) as e:
+        P.hss_solve(h, torch.ones(n, dtype=torch.float64, device=DEV))
+    assert e.value.status == P.hss.HSS_ERR_STATE
+    assert P.hss_factor_batched([h, good]) == [P.hss.HSS_ERR_SINGULAR, 0]
+    # the other handle's solution: |A - H| <= 100 rtol |A|, condition below 3
+    b = torch.ones(n, dtype=torch.float64, device=DEV)
+    A = torch.as_tensor(W.toeplitz_inv_distance(n), device=DEV)
+    assert float((A @ P.hss_solve(good, b) - b).norm()) <= 3e-4 * float(b.norm())
