@@ -948,8 +948,10 @@ std::array<IdKernel, 6> kernels2() {
 // Measuring tuner of the team size (threads per column) of the ID launches.
 // The results do not depend on the team size (fixed summation tree), so the
 // tuner may try several on real launches: launches are grouped into classes
-// (spread-out or cluster mode, columns in shared or global memory, and the
-// powers of two of the largest side, the sample count and the item count);
+// (spread-out or cluster mode, columns in shared or global memory, the powers
+// of two of the largest side, the sample count and the item count, and whether
+// the launch may change its group or cluster size: a class's choice is made for
+// every launch of the class, so it has to be one that each of them can run);
 // the first launches of a class try the instruction-count model's choice and
 // its two neighbours, twice each, timed with CUDA events and normalised by
 // the launch's sum of m d min(m, d); later launches of the class take the
@@ -959,9 +961,10 @@ class TeamTuner {
  public:
   struct Key {
     int dev, group, smem, lg_m, lg_d, lg_n;
+    bool alt;   // the launch may also halve its group or double its clusters
     bool operator<(const Key& o) const {
-      return std::tie(dev, group, smem, lg_m, lg_d, lg_n) <
-             std::tie(o.dev, o.group, o.smem, o.lg_m, o.lg_d, o.lg_n);
+      return std::tie(dev, group, smem, lg_m, lg_d, lg_n, alt) <
+             std::tie(o.dev, o.group, o.smem, o.lg_m, o.lg_d, o.lg_n, o.alt);
     }
   };
   struct Trial {
@@ -1298,7 +1301,7 @@ Err launch_id_batched(const IdItem* items_dev, const std::vector<IdItem>& h, boo
     const bool half_ok = (max_m + gsz - 1) / gsz < 32 && gsz >= 4 &&
                          need(gsz / 2) <= 227 * 1024 - 2048;
     const int choice = TeamTuner::get().choose(
-        TeamTuner::Key{dev_ordinal, two_per_sm ? 2 : 1, 0, ilog2(max_m), ilog2(d), ilog2(count)},
+        TeamTuner::Key{dev_ordinal, two_per_sm ? 2 : 1, 0, ilog2(max_m), ilog2(d), ilog2(count), half_ok},
         team_index(gsz, true), 2, units, &trial, half_ok);
     const int ti = choice & 7;
     if (choice >> 3) gsz /= 2;
@@ -1398,7 +1401,7 @@ Err launch_id_batched(const IdItem* items_dev, const std::vector<IdItem>& h, boo
     }
     TeamTuner::Trial* trial = nullptr;
     const int choice = TeamTuner::get().choose(
-        TeamTuner::Key{dev_ordinal, two ? 3 : 0, w_in_smem, ilog2(max_m), ilog2(d), ilog2(count)},
+        TeamTuner::Key{dev_ordinal, two ? 3 : 0, w_in_smem, ilog2(max_m), ilog2(d), ilog2(count), dbl_ok},
         team_index(C, w_in_smem == 0), w_in_smem ? 0 : 2, units, &trial, false, dbl_ok);
     const int ti = choice & 7;
     if (choice & 16) {   // clusters of C2: the columns stay in global memory
@@ -1418,6 +1421,7 @@ Err launch_id_batched(const IdItem* items_dev, const std::vector<IdItem>& h, boo
       if (e == cudaSuccess) cudaEventRecord(trial->e1, s);
       TeamTuner::get().launched(trial, e == cudaSuccess);
     }
+    if (e != cudaSuccess) cudaGetLastError();   // (reported here, not to the caller's next call)
     res = e == cudaSuccess ? check_launch("id_cpqr_cluster_kernel")
                            : fail(HSS_ERR_CUDA, std::string("id_cpqr_cluster_kernel launch: ") +
                                                     cudaGetErrorString(e));

@@ -306,3 +306,19 @@ def test_factor_of_nan_is_singular(P, n, leaf, at):
     b = torch.ones(n, dtype=torch.float64, device=DEV)
     A = torch.as_tensor(W.toeplitz_inv_distance(n), device=DEV)
     assert float((A @ P.hss_solve(good, b) - b).norm()) <= 3e-4 * float(b.norm())
+
+
+def test_id_launch_choice_fits_every_shape_of_a_class(P):
+    """Two batches of one tuner class (powers of two of their sizes), in
+    clusters of 8, which may double, and of 16, which may not; both through
+    the whole of the class's trials."""
+    def batch(count, m, d, seed):
+        g = torch.Generator(device=DEV).manual_seed(seed)
+        B = torch.randn(20, d, generator=g, device=DEV, dtype=torch.float64)
+        return [torch.randn(m, 20, generator=g, device=DEV, dtype=torch.float64) @ B for _ in range(count)]
+    pair = batch(10, 517, 384, 1), batch(8, 755, 496, 2)
+    first = [P.hss_id_batched(Y, 1e-9) for Y in pair]
+    for _ in range(8):
+        for Y, ref in zip(pair, first):
+            for x, y in zip(P.hss_id_batched(Y, 1e-9), ref):
+                assert x[0] == y[0] == 20 and torch.equal(x[1], y[1]) and torch.equal(x[2], y[2])
