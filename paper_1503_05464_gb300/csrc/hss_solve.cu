@@ -899,9 +899,11 @@ extern "C" hss_status hss_solve_batched(int32_t count, hss_t* hs, const void* co
     return HSS_ERR_INVALID;
   std::vector<hss_status> st(std::max(count, 1), HSS_OK);
   std::vector<SolveJob> jobs;
+  const hss_s* one = nullptr;   // the first handle there is: one launch, one dtype
   for (int32_t q = 0; q < count; ++q) {
     st[q] = check_solve(hs[q], B[q], ldb[q], nrhs[q], X[q], ldx[q]);
-    if (st[q] == HSS_OK && hs[0] && hs[q]->dtype != hs[0]->dtype) {
+    if (!one) one = hs[q];
+    if (st[q] == HSS_OK && hs[q]->dtype != one->dtype) {
       hs[q]->err = "hss_solve_batched: handles of different dtypes";
       st[q] = HSS_ERR_INVALID;
     }

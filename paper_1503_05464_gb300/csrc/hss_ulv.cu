@@ -705,11 +705,14 @@ extern "C" hss_status hss_factor(hss_t h, void* stream) {
 extern "C" hss_status hss_factor_batched(int32_t count, hss_t* hs, void* stream,
                                          hss_status* status) {
   if (count < 0 || (count > 0 && !hs)) return HSS_ERR_INVALID;
-  for (int32_t q = 1; q < count; ++q)
-    if (hs[q] && hs[0] && hs[q]->dtype != hs[0]->dtype) {
+  const hss_s* one = nullptr;   // the first handle there is: one launch, one dtype
+  for (int32_t q = 0; q < count; ++q) {
+    if (!one) one = hs[q];
+    if (hs[q] && hs[q]->dtype != one->dtype) {
       set_thread_error("hss_factor_batched: handles of different dtypes");
       return HSS_ERR_INVALID;
     }
+  }
   std::vector<hss_status> st(std::max(count, 1), HSS_OK);
   factor_many(count, hs, (cudaStream_t)stream, st.data());
   hss_status first = HSS_OK;

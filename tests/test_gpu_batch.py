@@ -174,3 +174,35 @@ def test_batched_factor_reports_each_handle(P):
     P.hss_factor_batched([h1])
     X, sts = P.hss_solve_batched([h1, h2], [torch.ones(600, dtype=torch.float64, device=DEV)] * 2)
     assert sts[0] == 0 and sts[1] == P.hss.HSS_ERR_STATE
+
+
+@pytest.mark.parametrize("order", [(None, "f64", "f32"), (None, None, "f32", "f64"), ("f32", None, "f64")])
+def test_batch_of_mixed_dtypes_behind_a_missing_handle(P, order):
+    """A missing handle is reported and does not stand for a dtype: the first
+    handle there is sets it, the other dtype is refused before any launch."""
+    import ctypes
+    L, H = P.hss.load(), P.hss
+    dt = {"f32": torch.float32, "f64": torch.float64}
+    hs, Bs = {}, {}
+    for k, t in dt.items():
+        A = W.toeplitz_inv_distance(300, dtype=np.float64, device=DEV).to(t).contiguous()
+        hs[k] = P.hss_compress(A, leaf_size=64)
+        P.hss_factor(hs[k])
+        Bs[k] = torch.randn(300, 3, dtype=t, device=DEV)
+    ref = {k: P.hss_solve(hs[k], Bs[k]) for k in dt}
+    cnt = len(order)
+    B = [Bs[k or "f64"] for k in order]
+    X = [torch.full_like(b, 7.0) for b in B]
+    vp, i64 = ctypes.c_void_p * cnt, ctypes.c_int64 * cnt
+    handles = vp(*[hs[k].handle.value if k else None for k in order])
+    sts = (ctypes.c_int * cnt)()
+    live = next(k for k in order if k)
+    assert L.hss_solve_batched(cnt, handles, vp(*[b.data_ptr() for b in B]), i64(*[3] * cnt), i64(*[3] * cnt),
+                               vp(*[x.data_ptr() for x in X]), i64(*[3] * cnt), None, sts) == H.HSS_ERR_INVALID
+    torch.cuda.synchronize()
+    assert list(sts) == [H.HSS_OK if k == live else H.HSS_ERR_INVALID for k in order]
+    for k, x in zip(order, X):
+        assert torch.equal(x, ref[k] if k == live else torch.full_like(x, 7.0))
+    assert L.hss_factor_batched(cnt, handles, None, sts) == H.HSS_ERR_INVALID
+    for k in dt:   # refused before anything was released
+        assert torch.equal(P.hss_solve(hs[k], Bs[k]), ref[k])
