@@ -322,3 +322,27 @@ def test_id_launch_choice_fits_every_shape_of_a_class(P):
         for Y, ref in zip(pair, first):
             for x, y in zip(P.hss_id_batched(Y, 1e-9), ref):
                 assert x[0] == y[0] == 20 and torch.equal(x[1], y[1]) and torch.equal(x[2], y[2])
+
+
+# panel partials (128 rows each) whose running sum leaves FP32's range and comes
+# back: 3e38 + 3e38 - 3e38 - 2e38; an odd pitch with bf16x3 takes the mma.sync
+# kernel
+@pytest.mark.parametrize("mode,pad", [("native", 0), ("native", 1), ("bf16x3", 1)])
+def test_column_sample_whose_partials_pass_the_fp32_range(P, mode, pad):
+    n, c = 600, 5
+    A = torch.zeros((n, n + pad), device=DEV)[:, :n]
+    for i, v in ((3, 3e38), (130, 3e38), (257, -3e38), (400, -2e38)):
+        A[i] = v
+    A[:, 7] = 0.0
+    A[500, 7] = float("inf")
+    A[501, 8] = float("nan")
+    R = torch.ones((n, c), device=DEV)
+    Sr, Sc = torch.empty((n, c), device=DEV), torch.empty((n, c), device=DEV)
+    P.hss_sample(A, R, 0, c, Sr, Sc, mode=mode)
+    want = A.double().T @ R.double()
+    plain = [j for j in range(n) if j not in (7, 8)]
+    # one rounding of each term (bf16x3: its three planes hold 24 bits) and of the sum
+    assert bool(((Sc.double() - want)[plain].abs() <= 5 * 2.0 ** -23 * 3e38).all())
+    assert bool(torch.isnan(Sc[8]).all())
+    if mode == "native":
+        assert bool((Sc[7] == float("inf")).all())
