@@ -346,3 +346,18 @@ def test_column_sample_whose_partials_pass_the_fp32_range(P, mode, pad):
     assert bool(torch.isnan(Sc[8]).all())
     if mode == "native":
         assert bool((Sc[7] == float("inf")).all())
+
+
+def test_row_sample_keeps_the_remainders_at_cuts(P):
+    """FP32, rows of A against ones: 2^23, then 124 times 0.75 (one in each
+    tile), so that every sum rounds and the remainders carry the rest.  The
+    CTAs' ranges cut a row's panel two or three times, each panel elsewhere;
+    the total, 2^23 + 93, is a number of FP32."""
+    n = 8000          # 63 panels of 125 tiles on 152 SMs
+    A = torch.zeros((n, n), device=DEV)
+    A[:, ::64] = 0.75
+    A[:, 0] = 2.0 ** 23
+    R = torch.ones((n, 3), device=DEV)
+    S = torch.empty((n, 3), device=DEV)
+    P.hss_sample(A, R, 0, 3, S, None)
+    assert bool((S == 2.0 ** 23 + 93).all())
