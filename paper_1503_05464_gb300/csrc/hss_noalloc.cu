@@ -25,13 +25,19 @@ constexpr int NOALLOC_MAX_LEAVES = 2048;    // leaves of the mask
 constexpr int NOALLOC_MAX_DEVICES = 64;
 
 // Partial sums of both products.  Within the limits above the CUDA-core
-// kernels need at most 16 MiB (16 panels x 2048 x 64 FP64 values) and the
+// kernels need at most 32.8 MiB on a GPU of 252 SMs (FP64: the column slab of
+// 16 panels x 2048 x 64 values, 16 MiB, and the row slab of 128 x 64 values for
+// each SM and panel, 16.8 MiB; FP32 8 MiB, and 16.8 for rows and remainders) and the
 // tensor-core kernel at most 35.2 MiB (its bfloat16 copy of R plus column and
 // row slabs; largest at n = 1984 with 125 clusters of two CTAs; 35.9 MiB in
 // TF32, whose copy of R is a transposed FP32 one), so 36 MiB holds every
 // call on a GPU of up to 252 SMs.  The need of each call is still checked before any
 // work is queued.
 constexpr size_t NOALLOC_PART_BYTES = (size_t)36 << 20;
+static_assert(8 * (16 * NOALLOC_MAX_N + (252 + 16) * 128) * NOALLOC_MAX_COLS <= NOALLOC_PART_BYTES &&
+                  4 * (16 * NOALLOC_MAX_N + 2 * (252 + 16) * 128) * NOALLOC_MAX_COLS <=
+                      NOALLOC_PART_BYTES,
+              "the CUDA-core kernels' slabs exceed the fixed scratch");
 
 static __device__ __align__(256) unsigned char g_noalloc_part[NOALLOC_PART_BYTES];
 static __device__ __align__(256) int32_t g_noalloc_leaf_of[NOALLOC_MAX_N];
