@@ -81,13 +81,14 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Doubles of a reflector buffer (it also holds 128 partial sums) and of the
-// candidate's column (later a block of the back substitution: 16 x 17 entries
-// of R1 and 4 x 32 of T)
-constexpr int ID_BS = 16;
-__host__ __device__ inline int id_vec(int d) { return d < 128 ? 128 : d; }
-__host__ __device__ inline int id_cbuf(int d) {
-  return d < ID_BS * (ID_BS + 1) + 128 ? ID_BS * (ID_BS + 1) + 128 : d;
+// Doubles of a block of the back substitution (16 x 17 entries of R1 and 4 x 32
+// of T), which takes the place of the candidate's column, or where that is
+// shorter of the columns' limits and downdates (3 mloc doubles), and gets
+// doubles of its own only where both are short: with few samples the number of
+// columns a CTA can hold must not fall for it
+constexpr int ID_BS = 16, ID_BLK = ID_BS * (ID_BS + 1) + 128;
+__host__ __device__ inline int id_cbuf(int d, int mloc) {
+  return d < ID_BLK && 3 * mloc < ID_BLK ? ID_BLK : d;
 }
 
 // Residual norms are >= 0 and inactive columns carry -1: as 64-bit integers
@@ -363,16 +364,15 @@ id_cpqr_cluster_kernel(const IdItem* __restrict__ items, int f64in,
   }
   const int mloc = (m - crank + C - 1) / C;       // columns crank, crank+C, ...
   const int mloc_max = (m + C - 1) / C;
-  // reflectors of steps i (vbuf + (i & 1) dv) and i - 1: the update of a step
+  // reflectors of steps i (vbuf + (i & 1) d) and i - 1: the update of a step
   // is applied in the same pass as the next step's dot product; then the
-  // candidate's column (cbuf).  The buffer of u_{i-1} also takes the partial
-  // sums of a candidate's residual, at the end of step i.  After the
+  // candidate's column (cbuf).  The buffer of u_{i-1} also takes the (at most
+  // 128) partial sums of a candidate's residual, at the end of step i.  After the
   // elimination: R1's diagonal, its reciprocals, and a block of the back
   // substitution
-  const int dv = id_vec(d);
-  double* vbuf = smem;                            // 2 dv
-  double* cbuf = vbuf + 2 * dv;                   // id_cbuf(d)
-  double* nrm = cbuf + id_cbuf(d);                // mloc_max
+  double* vbuf = smem;                            // 2 d
+  double* cbuf = vbuf + 2 * d;                    // id_cbuf(d, mloc_max)
+  double* nrm = cbuf + id_cbuf(d, mloc_max);      // mloc_max
   double* lim = nrm + mloc_max;                   // mloc_max: tol3z * (norm at last recompute)^2
   double* rdiag = lim + mloc_max;                 // mloc_max: R_ii of the pivot columns
   double* dprev = rdiag + mloc_max;               // mloc_max: tau (u_i . w), update pending
@@ -486,10 +486,13 @@ id_cpqr_cluster_kernel(const IdItem* __restrict__ items, int f64in,
         const double x = (c >= r + 1 && c < d) ? cbuf[c] : 0.0;
         pa = fma(x, x, pa);
       }
-    psum[32 * warp + lane] = pa;
+    if (32 * warp + lane < d) psum[32 * warp + lane] = pa;   // (the others are zero)
     asm volatile("bar.sync 1, 128;" ::: "memory");
     if (warp != 0) return;
-    double st = (psum[lane] + psum[32 + lane]) + (psum[64 + lane] + psum[96 + lane]);
+    double ps[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) ps[q] = 32 * q + lane < d ? psum[32 * q + lane] : 0.0;
+    double st = (ps[0] + ps[1]) + (ps[2] + ps[3]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) st = st + __shfl_xor_sync(0xffffffffu, st, o);
     const double alpha = have && r < d ? cbuf[r] : 0.0;
@@ -537,7 +540,7 @@ id_cpqr_cluster_kernel(const IdItem* __restrict__ items, int f64in,
       }
     }
     __syncthreads();
-    push_candidate(0, redb[0], redi[0], 0, vbuf, vbuf + dv);
+    push_candidate(0, redb[0], redi[0], 0, vbuf, vbuf + d);
   }
 
   const int kmax = min(m, d);
@@ -549,8 +552,8 @@ id_cpqr_cluster_kernel(const IdItem* __restrict__ items, int f64in,
   for (int i = 0; i < kmax; ++i) {
     if (!sync_all()) return;   // candidates of step i pushed, dot products of step i-1 done
     const int slot = i & 1;
-    double* vloc = vbuf + (i & 1) * dv;         // reflector u_i
-    const double* vprev = vbuf + ((i + 1) & 1) * dv;  // u_{i-1}
+    double* vloc = vbuf + (i & 1) * d;         // reflector u_i
+    const double* vprev = vbuf + ((i + 1) & 1) * d;  // u_{i-1}
     // every warp reduces the C candidates (lane r <- CTA r): all threads agree
     // on the pivot without a block barrier
     long long bv = LLONG_MIN;
@@ -727,7 +730,7 @@ id_cpqr_cluster_kernel(const IdItem* __restrict__ items, int f64in,
           cv = redb[w];
           cj = redi[w];
         }
-      push_candidate(slot ^ 1, cv, cj, i + 1, vloc, vbuf + ((i + 1) & 1) * dv);
+      push_candidate(slot ^ 1, cv, cj, i + 1, vloc, vbuf + ((i + 1) & 1) * d);
     }
   }
 
@@ -741,7 +744,7 @@ id_cpqr_cluster_kernel(const IdItem* __restrict__ items, int f64in,
   }
   // the update of step k - 1 is still pending on the remaining columns
   if (k > 0) {
-    const double* ul = vbuf + ((k - 1) & 1) * dv;
+    const double* ul = vbuf + ((k - 1) & 1) * d;
     const int na = nact;
     for (int q = warp; q < na; q += ID_WARPS) {
       const int jl = alist[q];
@@ -816,9 +819,10 @@ id_cpqr_cluster_kernel(const IdItem* __restrict__ items, int f64in,
   // division's 680 cycles of latency per row: 0.38 ms at m = 342, k = 241;
   // by blocks 0.24 ms.)
   double* diag = vbuf;        // k <= d entries
-  double* rinv = vbuf + dv;   // their reciprocals
-  double(*Rb)[ID_BS + 1] = reinterpret_cast<double(*)[ID_BS + 1]>(cbuf);
-  double(*xs)[2][32] = reinterpret_cast<double(*)[2][32]>(cbuf + ID_BS * (ID_BS + 1));
+  double* rinv = vbuf + d;    // their reciprocals
+  double* blk = d < ID_BLK && 3 * mloc_max >= ID_BLK ? lim : cbuf;
+  double(*Rb)[ID_BS + 1] = reinterpret_cast<double(*)[ID_BS + 1]>(blk);
+  double(*xs)[2][32] = reinterpret_cast<double(*)[2][32]>(blk + ID_BS * (ID_BS + 1));
   for (int a = tid; a < k; a += ID_THREADS) {
     const double x = __ldcg(R1 + (size_t)a * k + a);
     diag[a] = x;
@@ -1126,9 +1130,13 @@ Err launch_id_batched(const IdItem* items_dev, const std::vector<IdItem>& h, boo
   while (C < 16 && (long)count * C * 2 <= sms && max_m / (C * 2) >= 16) C *= 2;
   const int d = std::max(max_d, 1);
   auto need = [&](int c) {
-    int mloc = (max_m + c - 1) / c;
-    return sizeof(double) * (2 * (size_t)id_vec(d) + (size_t)id_cbuf(d) + 4 * (size_t)mloc) +
-           4 * sizeof(int) * (size_t)((mloc + 1) & ~1);
+    auto bytes = [](int d, int mloc) {
+      return sizeof(double) * (2 * (size_t)d + (size_t)id_cbuf(d, mloc) + 4 * (size_t)mloc) +
+             4 * sizeof(int) * (size_t)((mloc + 1) & ~1);
+    };
+    // (an item smaller than the largest may need the block's own doubles)
+    const int mloc = (max_m + c - 1) / c;
+    return std::max(bytes(d, mloc), bytes(std::min(d, ID_BLK - 1), std::min(mloc, (ID_BLK - 1) / 3)));
   };
   // a large side among many items: more CTAs per item until its share of the
   // per-column arrays fits in shared memory

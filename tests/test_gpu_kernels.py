@@ -361,3 +361,26 @@ def test_row_sample_keeps_the_remainders_at_cuts(P):
     S = torch.empty((n, 3), device=DEV)
     P.hss_sample(A, R, 0, 3, S, None)
     assert bool((S == 2.0 ** 23 + 93).all())
+
+
+# the most columns 16 CTAs hold beside few samples (their shared memory is full);
+# many columns and few samples, so that the back substitution's block takes the
+# columns' own arrays; and beside smaller items, whose block has doubles of its own
+@pytest.mark.parametrize("shapes", [[(76400, 32)], [(75700, 128)], [(3000, 40)], [(2200, 399), (60, 33), (130, 140)]])
+def test_id_of_many_columns_and_few_samples(P, shapes):
+    g = torch.Generator(device=DEV).manual_seed(len(shapes))
+    k, Ys = 19, []
+    for m, d in shapes:
+        B = torch.randn(k, d, generator=g, device=DEV, dtype=torch.float64)
+        Ys.append(torch.randn(m, k, generator=g, device=DEV, dtype=torch.float64) @ B)
+    out = P.hss_id_batched(Ys, 1e-9)
+    for Y, (kk, perm, E) in zip(Ys, out):
+        m = Y.shape[0]
+        assert kk == k
+        assert torch.equal(torch.sort(perm).values, torch.arange(m, device=DEV, dtype=torch.int32))
+        perm = perm.long()
+        # Y's other rows from the skeleton rows: E's entries are a few units, k
+        # roundings of each product, and the triangle's condition below 1e5
+        assert float((Y[perm[k:]] - E @ Y[perm[:k]]).abs().max()) <= 1e-9 * float(Y.abs().max())
+        kk1, perm1, E1 = P.hss_id_batched([Y], 1e-9)[0]
+        assert kk1 == k and torch.equal(perm1.long(), perm) and torch.equal(E1, E)
