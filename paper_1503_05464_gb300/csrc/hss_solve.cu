@@ -16,7 +16,8 @@
 // all-ones NaNs; a poll is bounded, and on a timeout the NaN reaches the
 // solution).  Triangular systems go by blocks of 32 rows: a task subtracts
 // the rows of L it needs and multiplies by the inverse of its diagonal block
-// (hss_factor leaves these, hss_ulv.cu), so the chain is one task per 32 rows.
+// (hss_factor leaves these, hss_ulv.cu; an ill-conditioned block is left as it
+// is, and the task substitutes), so the chain is one task per 32 rows.
 // One launch per tree level and operation (23 to 112 a solve), a warp per
 // right-hand side on its triangular chain, spent 5 FP64 instructions for
 // every useful one on narrow reductions: an FP64 instruction holds its pipe
@@ -37,6 +38,7 @@
 #include "hss_tree.h"
 
 #include <algorithm>
+#include <cfloat>
 #include <cmath>
 #include <climits>
 
@@ -187,6 +189,42 @@ __device__ __forceinline__ void sv_fma(double (&a)[2][NC], const S* ms, const do
 #pragma unroll
     for (int c = 0; c < NC; ++c) a[0][c] = fma(m0, zs[l * NC + c], a[0][c]);
   }
+}
+
+// v <- B^-1 v for the columns of v ([row][NC]) by substitution, a warp per
+// column, lane = row.  divided: B's rows are divided by its diagonal, where the
+// reciprocals stand; else B itself.
+template <int NC>
+__device__ __forceinline__ void sv_substitute(double* v, const double* B, int rows, bool upper,
+                                              bool divided) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (w >= NC) return;
+  const double* row = B + lane * (SV_ROWS + 1);
+  double x = lane < rows ? v[lane * NC + w] : 0.0;
+  if (divided) {
+    x *= row[lane];
+    if (upper) {
+#pragma unroll 8
+      for (int t = SV_ROWS - 1; t > 0; --t) {
+        const double xt = __shfl_sync(0xffffffffu, x, t);
+        if (lane < t && t < rows) x = fma(-row[t], xt, x);
+      }
+    } else {
+#pragma unroll 8
+      for (int t = 0; t < SV_ROWS - 1; ++t) {
+        const double xt = __shfl_sync(0xffffffffu, x, t);
+        if (lane > t) x = fma(-row[t], xt, x);
+      }
+    }
+  } else {
+    for (int q = 0; q < rows; ++q) {
+      const int t = upper ? rows - 1 - q : q;
+      if (lane == t) x /= row[t];
+      const double xt = __shfl_sync(0xffffffffu, x, t);
+      if (upper ? lane < t : lane > t) x = fma(-row[t], xt, x);
+    }
+  }
+  if (lane < rows) v[lane * NC + w] = x;
 }
 
 constexpr int SV_MS = SV_ENT + SV_ROWS;   // a stage's matrix with its odd pitch
@@ -401,10 +439,21 @@ __global__ void __launch_bounds__(SV_THREADS, NC == 4 ? 5 : 6) ulv_solve_kernel(
         if (e < rows * NC) ms[e] = val[o];
       }
       __syncthreads();
+      const bool up = (tk.flags & SD_POST_UPPER) != 0;
+      const double kind = ps[up ? (SV_ROWS - 1) * (SV_ROWS + 1) : SV_ROWS - 1];
+      const bool subst = kind != 0.0;   // the block, not its inverse
+      if (subst) {
+        sv_substitute<NC>(ms, ps, rows, up, kind == 1.0);
+        __syncthreads();
+      }
 #pragma unroll
       for (int o = 0; o < EO; ++o) {
         const int e = tid + o * SV_THREADS, r = e / NC, c = e - r * NC;
         if (r >= rows) continue;
+        if (subst) {
+          val[o] = ms[e];
+          continue;
+        }
         double s[4] = {0.0, 0.0, 0.0, 0.0};
         const double* p = ps + r * (SV_ROWS + 1);
         // (the zeros of a triangular block are left out four at a time)

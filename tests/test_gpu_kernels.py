@@ -384,3 +384,54 @@ def test_id_of_many_columns_and_few_samples(P, shapes):
         assert float((Y[perm[k:]] - E @ Y[perm[:k]]).abs().max()) <= 1e-9 * float(Y.abs().max())
         kk1, perm1, E1 = P.hss_id_batched([Y], 1e-9)[0]
         assert kk1 == k and torch.equal(perm1.long(), perm) and torch.equal(E1, E)
+
+
+def _ill_triangles(kind, n, seed):
+    """A = L U with |B||B^-1| to 1e11 in its diagonal blocks, and |L||U|: unit
+    lower triangles of -0.9 (partial pivoting keeps the rows), or U alone, or U
+    with two diagonal entries 2^120 below their rows."""
+    rng = np.random.default_rng(seed)
+    low = np.tril(-0.9 * np.ones((n, n)), -1) + np.eye(n)
+    up = np.triu(rng.standard_normal((n, n)), 1) + 6 * np.eye(n)
+    if kind != "lower":
+        low, up = np.eye(n), np.triu(-np.ones((n, n)), 1) + np.eye(n)
+    if kind == "wide":
+        up[3, 3] = up[n - 2, n - 2] = 2.0 ** -120
+    return low @ up, np.abs(low) @ np.abs(up)
+
+
+def _solves_as_substitution(P, A, bound, leaf):
+    """|A x - b| within `bound` |x| and a column's bits the same in every
+    width (1, 2 and 4 columns a task) and in a batch."""
+    n = A.shape[0]
+    h = P.hss_compress(torch.tensor(A, device=DEV), leaf_size=leaf)
+    P.hss_factor(h)
+    b = A @ np.random.default_rng(n).standard_normal((n, 33))
+    B = torch.tensor(b, device=DEV)
+    x = P.hss_solve(h, B)
+    xn = x.cpu().numpy()
+    assert np.all(np.abs(A @ xn - b) <= bound(xn))
+    for k in (1, 9):
+        assert torch.equal(P.hss_solve(h, B[:, :k].contiguous()), x[:, :k])
+    X, st = P.hss_solve_batched([h, h], [B[:, :3].contiguous(), B])
+    assert st == [0, 0] and torch.equal(X[0], x[:, :3]) and torch.equal(X[1], x)
+
+
+@pytest.mark.parametrize("kind", ["lower", "upper", "wide"])
+@pytest.mark.parametrize("n", [20, 33, 45, 60])
+def test_solve_with_ill_conditioned_root_blocks(P, kind, n):
+    A, LU = _ill_triangles(kind, n, n)
+    # Higham, Accuracy and Stability, theorem 9.4: 3 n u |L||U||x|
+    _solves_as_substitution(P, A, lambda x: 3 * n * 2.0 ** -53 * (LU @ np.abs(x)), 128)
+
+
+@pytest.mark.parametrize("n", [20, 45, 64, 150])
+def test_solve_with_ill_conditioned_node_blocks(P, n):
+    """Two nodes of rank zero, each A_i = L Q: the LQ's L is ill conditioned.
+    Householder LQ and substitution: 10 n u |A||x| in norms."""
+    import scipy.linalg as sla
+    rng = np.random.default_rng(n)
+    low = np.tril(-0.9 * np.ones((n, n)), -1) + np.eye(n)
+    A = sla.block_diag(*[low @ np.linalg.qr(rng.standard_normal((n, n)))[0] for _ in range(2)])
+    _solves_as_substitution(
+        P, A, lambda x: 10 * n * 2.0 ** -53 * np.linalg.norm(A) * np.linalg.norm(x, axis=0), n)
