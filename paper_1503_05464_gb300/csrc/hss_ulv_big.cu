@@ -18,7 +18,7 @@
 //           to 32 rows (lq_update_kernel);
 //   root    right-looking blocked LU with partial pivoting: the panel by a
 //           cluster that splits its rows (lu_panel_kernel), the block row by
-//           the inverse of the panel's unit triangle, GEMM update of the rest.
+//           substitution, 16 columns a CTA, GEMM update of the rest.
 // The factors have the per-node kernel's layout.
 // Every launch shape that a node's sums depend on follows from the node's own
 // order, so factors do not depend on what shares the launch.
@@ -509,7 +509,6 @@ struct LuPanel {
   double* A;        // m x m
   int32_t* piv;
   int32_t* status;
-  double* Linv;     // NB x NB: the inverse of the panel's unit lower triangle
   int m, j0, nbb;
 };
 
@@ -538,7 +537,6 @@ __global__ void __launch_bounds__(B_THREADS) lu_panel_kernel(const LuPanel* item
   __shared__ int wi[B_WARPS];
   __shared__ int pivs[NB];
   __shared__ int src[2 * NB], dst[2 * NB], nmove;
-  __shared__ double xl[NB][NB + 1];
   const LuPanel it = items[blockIdx.x / C];
   const int m = it.m, j0 = it.j0, nbb = it.nbb;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -714,56 +712,43 @@ __global__ void __launch_bounds__(B_THREADS) lu_panel_kernel(const LuPanel* item
     for (int q = 0; q < 2 * NB; ++q)
       if (q < n) col[static_cast<int64_t>(dst[q]) * m] = v[q];
   }
-  if (rank == 0) {
-    // inverse of the unit lower triangle: lane = column, warp w keeps rows w + 8 t
-    double x[4];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) x[t] = (w + 8 * t == lane) ? 1.0 : 0.0;
-    for (int l = 0; l < nbb; ++l) {
-      if (w == (l & 7)) {
-#pragma unroll
-        for (int t = 0; t < 4; ++t)
-          if (t == (l >> 3)) xl[l][lane] = x[t];
-      }
-      __syncthreads();
-      const double xv = xl[l][lane];
-#pragma unroll
-      for (int t = 0; t < 4; ++t)
-        if (w + 8 * t > l && w + 8 * t < nbb) x[t] = fma(-A[(w + 8 * t) * ld + l], xv, x[t]);
-    }
-#pragma unroll
-    for (int t = 0; t < 4; ++t) it.Linv[(w + 8 * t) * NB + lane] = x[t];
-  }
 }
 
-// U12 = L11^{-1} A12 of a batch of panels (one per blockIdx.y): 16 columns a
-// CTA, thread = (column, rows t and t + 16).  With the inverse the 32 rows
-// are independent sums; substitution is a chain of 32 dependent FMAs on one
-// thread per column.
+// U12 = L11^{-1} A12 of a batch of panels (one per blockIdx.y) by substitution:
+// 16 columns a CTA, thread = (column, rows t and t + 16); row b goes through
+// shared memory to the rows below it.  (A thread per column has a chain of 496
+// FMAs; with the inverse of L11 the rows are independent, but the error grows
+// with L11's condition.)
 __global__ void __launch_bounds__(B_THREADS) lu_u12_kernel(const LuPanel* items) {
-  __shared__ double Li[NB][NB + 1];
+  __shared__ double L[NB][NB + 1];
   __shared__ double x[NB][17];
   const LuPanel it = items[blockIdx.y];
   const int c0 = it.j0 + it.nbb + blockIdx.x * 16;
   if (c0 >= it.m) return;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, c = c0 + tx;
   double* A = it.A + static_cast<int64_t>(it.j0) * it.m;
-  for (int e = tid; e < NB * NB; e += B_THREADS) Li[e / NB][e % NB] = it.Linv[e];
+  for (int e = tid; e < it.nbb * NB; e += B_THREADS)
+    if (e % NB < it.nbb) L[e / NB][e % NB] = A[static_cast<int64_t>(e / NB) * it.m + it.j0 + e % NB];
+  double v[2];
 #pragma unroll
   for (int a = 0; a < 2; ++a) {
     const int r = ty + 16 * a;
-    x[r][tx] = (r < it.nbb && c < it.m) ? A[static_cast<int64_t>(r) * it.m + c] : 0.0;
+    v[a] = (r < it.nbb && c < it.m) ? A[static_cast<int64_t>(r) * it.m + c] : 0.0;
   }
-  __syncthreads();
-  double s0 = 0.0, s1 = 0.0;
-#pragma unroll 8
-  for (int l = 0; l < NB; ++l) {
-    s0 = fma(Li[ty][l], x[l][tx], s0);
-    s1 = fma(Li[ty + 16][l], x[l][tx], s1);
+  for (int b = 0; b < it.nbb; ++b) {
+    if (ty == (b & 15)) x[b][tx] = b < 16 ? v[0] : v[1];
+    __syncthreads();
+    const double xb = x[b][tx];
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      const int r = ty + 16 * a;
+      if (r > b && r < it.nbb) v[a] = fma(-L[r][b], xb, v[a]);
+    }
   }
-  if (c < it.m) {
-    if (ty < it.nbb) A[static_cast<int64_t>(ty) * it.m + c] = s0;
-    if (ty + 16 < it.nbb) A[static_cast<int64_t>(ty + 16) * it.m + c] = s1;
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    const int r = ty + 16 * a;
+    if (r < it.nbb && c < it.m) A[static_cast<int64_t>(r) * it.m + c] = v[a];
   }
 }
 
@@ -978,7 +963,7 @@ Err ulv_factor_big_multi(const std::vector<std::pair<hss_s*, int>>& items,
     hss_s* h;
     int id, m, k, r, kc, mc, leaf, root, f64in;
     int32_t* status;
-    double *Dw, *W, *VhT, *Vd, *Tall, *Linv;
+    double *Dw, *W, *VhT, *Vd, *Tall;
   };
   std::vector<Node> N;
   for (size_t q = 0; q < items.size(); ++q) {
@@ -1003,7 +988,6 @@ Err ulv_factor_big_multi(const std::vector<std::pair<hss_s*, int>>& items,
     const size_t mm = static_cast<size_t>(x.m) * x.m;
     if (x.root) {
       x.Dw = F.root_lu;
-      HSS_TRY(ar.alloc_t(&x.Linv, NB * NB, s));
     } else {
       HSS_TRY(ar.alloc_t(&x.Dw, mm, s));
       HSS_TRY(ar.alloc_t(&x.W, mm, s));
@@ -1061,7 +1045,7 @@ Err ulv_factor_big_multi(const std::vector<std::pair<hss_s*, int>>& items,
       for (Node& x : N) {
         if (!x.root || j0 >= x.m) continue;
         const int m = x.m, nbb = std::min(NB, m - j0), rest = m - j0 - nbb;
-        lp.push_back({x.Dw, x.h->ulv.root_piv, x.status, x.Linv, m, j0, nbb});
+        lp.push_back({x.Dw, x.h->ulv.root_piv, x.status, m, j0, nbb});
         if (rest <= 0) continue;
         lt.push_back(lp.back());
         maxrest = std::max(maxrest, rest);

@@ -435,3 +435,14 @@ def test_solve_with_ill_conditioned_node_blocks(P, n):
     A = sla.block_diag(*[low @ np.linalg.qr(rng.standard_normal((n, n)))[0] for _ in range(2)])
     _solves_as_substitution(
         P, A, lambda x: 10 * n * 2.0 ** -53 * np.linalg.norm(A) * np.linalg.norm(x, axis=0), n)
+
+
+@pytest.mark.parametrize("kind", ["lower", "upper"])
+@pytest.mark.parametrize("n", [64, 100, 150, 333])
+def test_factor_with_ill_conditioned_panels(P, kind, n):
+    """The same triangles down the diagonal of a blocked root: the panels' unit
+    triangles are ill conditioned too."""
+    import scipy.linalg as sla
+    As, LUs = zip(*[_ill_triangles(kind, min(60, n - i), i) for i in range(0, n, 60)])
+    A, LU = sla.block_diag(*As), sla.block_diag(*LUs)
+    _solves_as_substitution(P, A, lambda x: 3 * n * 2.0 ** -53 * (LU @ np.abs(x)), 512)
