@@ -493,6 +493,26 @@ Err matvec_tasks(hss_s* h, const T* X, int64_t ldx, int nrhs, T* B, int64_t ldb,
       e = fail(HSS_ERR_CUDA, "hss_matvec: device query");
     } else {
       const int64_t total = (int64_t)g.ntasks * g.nch;
+      if (h->tree.nodes.size() == 1) {
+        // H = D: half of the tasks are D x and all of the work, and none waits
+        // for long.  A CTA claims a task ahead, so the CTAs per SM are those
+        // whose rounds over the D x tasks are the fewest tasks per SM in all
+        // (three or more if there are several rounds).  FP64, n = 1000, 3000,
+        // 8000: 1 column 35, 103, 313 -> 34, 90, 286 us, 8 columns 66, 348, 1619 ->
+        // 66, 258, 1111, 16 columns 95, 523, 2910 -> 68, 348, 2280 with eight
+        // (six) CTAs per SM before.
+        const int64_t dx = total / 2;
+        int best = per_sm;
+        int64_t least = INT64_MAX;
+        for (int p = per_sm; p >= 1; --p) {
+          const int64_t rounds = (dx + (int64_t)sms * p - 1) / ((int64_t)sms * p);
+          if (rounds * p < least && (p >= 3 || rounds == 1)) {
+            least = rounds * p;
+            best = p;
+          }
+        }
+        per_sm = best;
+      }
       const int grid = (int)std::min<int64_t>(total, (int64_t)sms * std::max(per_sm, 1));
       fn<<<grid, MV_THREADS, 0, s>>>(g);
       e = check_launch("matvec_kernel");

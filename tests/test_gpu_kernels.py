@@ -446,3 +446,22 @@ def test_factor_with_ill_conditioned_panels(P, kind, n):
     As, LUs = zip(*[_ill_triangles(kind, min(60, n - i), i) for i in range(0, n, 60)])
     A, LU = sla.block_diag(*As), sla.block_diag(*LUs)
     _solves_as_substitution(P, A, lambda x: 3 * n * 2.0 ** -53 * (LU @ np.abs(x)), 512)
+
+
+# a single node: fewer CTAs per SM than fit, one and several rounds of tasks
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("n", [90, 1000, 2600, 5200])
+def test_matvec_of_one_dense_node(P, dtype, n):
+    g = torch.Generator(device=DEV).manual_seed(n)
+    A = torch.randn(n, n, generator=g, device=DEV, dtype=torch.float64).to(dtype)
+    X = torch.randn(n, 32, generator=g, device=DEV, dtype=torch.float64).to(dtype)
+    h = P.hss_compress(A, leaf_size=n)
+    full = P.hss_matvec(h, X)
+    # a sum of n products
+    u = 2.0 ** -24 if dtype == torch.float32 else 2.0 ** -53
+    A64, X64 = A.double(), X.double()
+    assert bool(((full.double() - A64 @ X64).abs() <= 2 * n * u * (A64.abs() @ X64.abs())).all())
+    for k in (1, 3, 9):
+        x = X[:, :k].contiguous()
+        y = P.hss_matvec(h, x)
+        assert torch.equal(y, full[:, :k]) and torch.equal(P.hss_matvec(h, x), y)
