@@ -41,8 +41,8 @@ constexpr int S_THREADS = 256;
 // in shared memory for both products: a thread takes rows ty, ty + NTY, ...
 // of the row product, four inner indices per 16-byte load (the odd multiple
 // of 16 bytes in the pitch keeps the rows of a warp on different banks), and
-// CJ adjacent columns of the column product.  Chunks of 32 columns where 64
-// would add padding (FP64: the pipe's time is the padded columns').
+// CJ adjacent columns of the column product.  Chunks are 64 or 32 columns wide
+// (simt_plan).
 // What is left above the FMA floor is shared-memory bandwidth: a read of 16
 // bytes a lane takes about three of the SM's shared-memory cycles even where
 // lanes share addresses, and the 8 x 4 and 4 x 4 register blocks need 12 and
@@ -73,8 +73,15 @@ struct SimtPlan {
 template <typename T>
 SimtPlan simt_plan(int64_t n, int64_t ncols, int sms) {
   SimtPlan pl;
-  // 64-column chunks unless 32-column ones have less padding
-  pl.dc = (ncols + 63) / 64 * 64 == (ncols + 31) / 32 * 32 ? 64 : 32;
+  // FP64: 32-column chunks where they pad less, as the pipe's time is the padded
+  // columns' (n = 8000, in chunks of 64 / 32: 32 columns 13.8 / 7.0 ms, 64 13.8 /
+  // 14.0, 96 27.5 / 21.1, 128 27.5 / 27.8).  FP32 is bound by shared memory, where
+  // the smaller register blocks of 32 columns cost more than the padding unless
+  // one chunk holds all (n = 10000: 32 columns 0.75 / 0.54 ms, 48 0.75 / 1.05, 65
+  // 1.55 / 1.64, 96 1.47 / 1.59, 160 2.23 / 2.62).
+  const bool narrow = sizeof(T) == 4 ? ncols <= 32
+                                     : (ncols + 63) / 64 * 64 != (ncols + 31) / 32 * 32;
+  pl.dc = narrow ? 32 : 64;
   const int bk = sizeof(T) == 4 ? 64 : 32;
   pl.npanel = (int)((n + S_BM - 1) / S_BM);
   pl.ntile = (int)((n + bk - 1) / bk);
