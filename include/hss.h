@@ -198,7 +198,8 @@ hss_status hss_factor(hss_t h, void* stream);
  * Errors: STATE (no hss_factor yet), INVALID, OOM, CUDA.  Stream-ordered:
  * the call returns without waiting for the device.  (The first solve after
  * hss_factor builds a task table, which stays with the handle and serves any
- * number of columns.)
+ * number of columns.)  Columns go 64 at a time, or as many as the work
+ * buffer's memory is there for; OOM if it is not there for one.
  */
 hss_status hss_solve(hss_t h, const void* B, int64_t ldb, int64_t nrhs,
                      void* X, int64_t ldx, void* stream);

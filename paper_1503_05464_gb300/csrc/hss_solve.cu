@@ -56,7 +56,7 @@ constexpr int SV_ENT = 1024;
 constexpr int SV_LMAX = SV_ENT / 8;
 constexpr int SV_FINE_M = 160;
 constexpr int64_t SV_MANY_ROWS = 200000;
-constexpr int SV_COLS = 64;   // right-hand sides per launch (bounds the work buffer)
+constexpr int SV_COLS = 64;   // right-hand sides per launch, fewer where memory is short
 constexpr long long SV_WAIT_LIMIT = 1ll << 33;   // clock cycles (about 4 s)
 
 enum {   // SvTerm::flags
@@ -772,16 +772,16 @@ Err sv_plan(hss_s* h) {
   return ok();
 }
 
-// columns [c0, c0 + SV_COLS) of every job (those that have them)
+// columns [c0, c0 + width) of every job (those that have them)
 template <typename T>
-Err solve_slab(const std::vector<SolveJob*>& jobs, int c0, cudaStream_t s) {
+Err solve_slab(const std::vector<SolveJob*>& jobs, int c0, int width, cudaStream_t s) {
   std::vector<SvJob> js;
   std::vector<const UlvFactors*> fs;
   size_t rows = 0;
   int maxnr = 1;
   std::vector<size_t> off;
   for (SolveJob* j : jobs) {
-    const int nr = std::min(SV_COLS, j->nr - c0);
+    const int nr = std::min(width, j->nr - c0);
     if (nr <= 0) continue;
     const UlvFactors& F = j->h->ulv;
     SvJob q{};
@@ -894,10 +894,23 @@ void solve_many(std::vector<SolveJob>& jobs, cudaStream_t s) {
     live.push_back(&j);
     maxnr = std::max(maxnr, j.nr);
   }
-  for (int c0 = 0; c0 < maxnr; c0 += SV_COLS) {
-    const Err e = live[0]->h->dtype == HSS_F64 ? solve_slab<double>(live, c0, s)
-                                               : solve_slab<float>(live, c0, s);
-    if (e.st == HSS_OK) continue;
+  // The work buffer holds a value only once (its values are their own flags), so
+  // each panel of Q has rows of its own: about r (m - r / 2) / 32 rows for r
+  // reflectors of a node of order m.  Where that does not fit, half as many
+  // columns at a time (a column's bits do not depend on it).
+  int width = SV_COLS;
+  for (int c0 = 0; c0 < maxnr;) {
+    width = std::min(width, maxnr - c0);
+    const Err e = live[0]->h->dtype == HSS_F64 ? solve_slab<double>(live, c0, width, s)
+                                               : solve_slab<float>(live, c0, width, s);
+    if (e.st == HSS_OK) {
+      c0 += width;
+      continue;
+    }
+    if (e.st == HSS_ERR_OOM && width > 1) {
+      width /= 2;
+      continue;
+    }
     for (SolveJob* j : live) {
       j->h->err = e.msg;
       *j->st = e.st;

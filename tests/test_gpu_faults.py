@@ -90,3 +90,38 @@ def test_injected_oom_fails_cleanly_and_leaks_nothing(P, mode):
     b = torch.ones(n, dtype=torch.float32, device=DEV)
     x = P.hss_solve(h, b)
     assert float(torch.linalg.norm(A @ x - b) / torch.linalg.norm(b)) < 1e-4
+
+
+def test_solve_takes_fewer_columns_where_memory_is_short(P):
+    """The work buffer's allocation fails: half the columns at a time, with
+    the same bits; a single column has nothing to halve."""
+    H = P.hss
+    import workloads as W
+    A = W.toeplitz_inv_distance(900, dtype=np.float64, device=DEV)
+    h, g = (P.hss_compress(A, leaf_size=100) for _ in range(2))
+    P.hss_factor(h)
+    P.hss_factor(g)
+    B = torch.randn(900, 70, dtype=torch.float64, device=DEV)
+    ref = P.hss_solve(h, B)
+    both, _ = P.hss_solve_batched([h, g], [B, B[:, :9].contiguous()])
+    torch.cuda.synchronize()
+    used, _ = H.hss_pool_bytes()
+    for after in (1, 2):      # the first launch's buffer, then the second's
+        H.hss_set_fault(H.HSS_FAULT_OOM, after)
+        try:
+            assert torch.equal(P.hss_solve(h, B), ref)
+            H.hss_set_fault(H.HSS_FAULT_OOM, after)
+            X, st = P.hss_solve_batched([h, g], [B, B[:, :9].contiguous()])
+            assert st == [0, 0] and torch.equal(X[0], both[0]) and torch.equal(X[1], both[1])
+        finally:
+            H.hss_set_fault(H.HSS_FAULT_NONE)
+    H.hss_set_fault(H.HSS_FAULT_OOM, 1)
+    try:
+        with pytest.raises(P.HssError) as e:
+            P.hss_solve(h, B[:, 0].contiguous())
+        assert e.value.status == H.HSS_ERR_OOM
+    finally:
+        H.hss_set_fault(H.HSS_FAULT_NONE)
+    torch.cuda.synchronize()
+    assert H.hss_pool_bytes()[0] == used
+    assert torch.equal(P.hss_solve(h, B), ref)
