@@ -175,7 +175,10 @@ hss_status hss_compress_matfree(int64_t n, hss_dtype dtype, const hss_matfree* o
  * hss_matvec -- B = H X with the compressed form (Algorithm 2).
  *   X  device, n x nrhs row-major, ldx >= nrhs, the handle's dtype.
  *   B  device, n x nrhs row-major, ldb >= nrhs; must not overlap X.
- * Errors: INVALID, OOM, CUDA.  Stream-ordered: the call returns without
+ * Errors: INVALID, OOM, CUDA, TIMEOUT (a bounded wait inside an EARLIER product
+ * or solve with this handle gave up, and its result holds NaN: reported once,
+ * by the first call after that work has run, which does nothing else; a call
+ * with nrhs = 0 asks for it).  Stream-ordered: the call returns without
  * waiting for the device.  (The first product of up to 32 columns builds
  * a task table that stays with the handle; wider products send small tables
  * through pinned blocks of the calling thread, eight of which may be in
@@ -195,7 +198,8 @@ hss_status hss_factor(hss_t h, void* stream);
  * hss_solve -- X = H^{-1} B with the ULV factors (Algorithm 4).
  *   B  device, n x nrhs row-major, ldb >= nrhs, the handle's dtype.
  *   X  device, n x nrhs row-major, ldx >= nrhs (may equal B when ldx == ldb).
- * Errors: STATE (no hss_factor yet), INVALID, OOM, CUDA.  Stream-ordered:
+ * Errors: STATE (no hss_factor yet), INVALID, OOM, CUDA, TIMEOUT (of an
+ * earlier call, as hss_matvec).  Stream-ordered:
  * the call returns without waiting for the device.  (The first solve after
  * hss_factor builds a task table, which stays with the handle and serves any
  * number of columns.)  Columns go 64 at a time, or as many as the work
@@ -440,7 +444,8 @@ typedef enum {
   HSS_FAULT_OOM = 1,         /* the value-th device allocation from now (1 = the
                                 next) fails with HSS_ERR_OOM, once                  */
   HSS_FAULT_WAIT_LIMIT = 2   /* the bounded barrier wait of the ID's spread-out
-                                (group) mode gives up after `value` clock cycles
+                                (group) mode and the bounded polls of the product
+                                and the solve give up after `value` clock cycles
                                 instead of about 2^33; 0 restores the default       */
 } hss_fault;
 

@@ -197,6 +197,40 @@ Err upload_kept(void** dst, const std::vector<std::pair<const void*, size_t>>& p
   return e;
 }
 
+namespace {
+std::mutex g_words_mu;
+std::vector<unsigned*> g_words;   // the words not in use; pages stay until the process ends
+}  // namespace
+
+Err host_word_get(unsigned** w) {
+  std::lock_guard<std::mutex> lock(g_words_mu);
+  if (g_words.empty()) {
+    // (a capture of the caller's does not cover this)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    HSS_CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode));
+    constexpr size_t page = 4096;
+    unsigned* p = nullptr;
+    const cudaError_t e = cudaHostAlloc(reinterpret_cast<void**>(&p), page,
+                                        cudaHostAllocPortable | cudaHostAllocMapped);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return fail(HSS_ERR_OOM, std::string("cudaHostAlloc: ") + cudaGetErrorString(e));
+    }
+    for (size_t q = 0; q < page / sizeof(unsigned); ++q) g_words.push_back(p + q);
+  }
+  *w = g_words.back();
+  g_words.pop_back();
+  **w = 0;
+  return ok();
+}
+
+void host_word_put(unsigned* w) {
+  if (!w) return;
+  std::lock_guard<std::mutex> lock(g_words_mu);
+  g_words.push_back(w);
+}
+
 }  // namespace hss
 
 using namespace hss;

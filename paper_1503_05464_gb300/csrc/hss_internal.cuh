@@ -43,8 +43,9 @@ int64_t launches_so_far();
 // Message returned by hss_last_error(NULL) on the calling thread.
 void set_thread_error(const std::string& msg);
 
-// Injected faults (hss_set_fault): the group-mode barrier's wait limit in
-// clock cycles (0 = the kernel's default).
+// Injected faults (hss_set_fault): the limit of the group-mode barrier's wait
+// and of the product's and the solve's polls in clock cycles (0 = the kernel's
+// default).
 int64_t fault_wait_limit();
 
 // Stream-ordered device allocation (cudaMallocAsync); null for 0 bytes.
@@ -60,6 +61,11 @@ Err upload_async(void* dst, const void* src, size_t bytes, cudaStream_t s);
 // complete when the function returns (it uses a stream of its own, so the
 // caller's stream is neither waited for nor captured into).  Freed with dfree.
 Err upload_kept(void** dst, const std::vector<std::pair<const void*, size_t>>& parts);
+
+// A zeroed word of pinned host memory that a kernel may set and the host read
+// without waiting, from a pool kept for the process; host_word_put gives it back.
+Err host_word_get(unsigned** w);
+void host_word_put(unsigned* w);
 
 template <typename T>
 inline Err dalloc_t(T** p, size_t count, cudaStream_t s) {

@@ -17,7 +17,8 @@
 // counter, and whatever a task reads is written by tasks of lower tickets, so
 // its CTA is running or has finished: the polls end whatever number of CTAs is
 // resident and whatever else is on the device.  Each poll is bounded all the
-// same: on a timeout the value stays NaN and reaches the product.
+// same: on a timeout the value stays NaN and reaches the product, and the next
+// call with the handle reports it (hss_s::timeout).
 //
 // A task's matrix rows never depend on a wait: they are on their way to shared
 // memory (cp.async, 16 rows by 64 inner indices a stage) while the task
@@ -77,6 +78,8 @@ struct MvArgs {
   const int2* tasks;   // (description, r0)
   const MvDesc* descs;
   unsigned* ctl;       // [0] ticket, [1] a poll has timed out
+  unsigned* timeout;   // the handle's word for that
+  long long limit;     // of a poll, in clock cycles
   void* buf;
   const void* X;
   void* B;
@@ -106,16 +109,17 @@ __device__ __forceinline__ bool mv_unset(float v) { return __float_as_int(v) == 
 
 // *p once it has been written (bounded; the flag ends the other polls early)
 template <typename T>
-__device__ __forceinline__ T mv_poll(const T* p, unsigned* stop) {
+__device__ __forceinline__ T mv_poll(const T* p, const MvArgs& g) {
   T v = mv_ld(p);
   if (!mv_unset(v)) return v;
   const long long t0 = clock64();
   unsigned polls = 0;
   while (mv_unset(v = mv_ld(p))) {
     if ((++polls & 31u) != 0u) continue;
-    if (*reinterpret_cast<volatile unsigned*>(stop)) break;
-    if (clock64() - t0 > MV_WAIT_LIMIT) {
-      atomicExch(stop, 1u);
+    if (*reinterpret_cast<volatile unsigned*>(g.ctl + 1)) break;
+    if (clock64() - t0 > g.limit) {
+      atomicExch(g.ctl + 1, 1u);
+      *reinterpret_cast<volatile unsigned*>(g.timeout) = 1u;
       break;
     }
   }
@@ -192,7 +196,6 @@ __global__ void __launch_bounds__(MV_THREADS, NC == 8 ? 6 : 8) matvec_kernel(con
   __shared__ MvDesc tk;
   __shared__ unsigned snext;
   const int tid = threadIdx.x, lane = tid & 31;
-  unsigned* stop = g.ctl + 1;
   const unsigned total = (unsigned)g.ntasks * (unsigned)g.nch;
   T* buf = reinterpret_cast<T*>(g.buf);
   const int64_t nr = g.nrhs;
@@ -277,13 +280,13 @@ __global__ void __launch_bounds__(MV_THREADS, NC == 8 ? 6 : 8) matvec_kernel(con
         }
         // one lane of each warp polls until its value is there, so that a
         // wait costs one load a warp; then every value is read
-        if (lane == 0 && p[0]) mv_poll(p[0], stop);
+        if (lane == 0 && p[0]) mv_poll(p[0], g);
         __syncwarp();
 #pragma unroll
         for (int u = 0; u < U; ++u) v[u] = p[u] ? mv_ld(p[u]) : T(0);
 #pragma unroll
         for (int u = 0; u < U; ++u)
-          if (p[u] && mv_unset(v[u])) v[u] = mv_poll(p[u], stop);
+          if (p[u] && mv_unset(v[u])) v[u] = mv_poll(p[u], g);
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
@@ -305,9 +308,9 @@ __global__ void __launch_bounds__(MV_THREADS, NC == 8 ? 6 : 8) matvec_kernel(con
     T xv = T(0), xb = T(0);
     if (xi >= 0) {
       if (up && tk.from_x) xv = Xb[(int64_t)xi * g.ldx + oc];
-      else xv = mv_poll(zrow(up, xi) + oc, stop);
+      else xv = mv_poll(zrow(up, xi) + oc, g);
     }
-    if (has_out && tk.kind == MV_LEAF) xb = mv_poll(buf + (tk.dx + r0 + orow) * nr + cb + oc, stop);
+    if (has_out && tk.kind == MV_LEAF) xb = mv_poll(buf + (tk.dx + r0 + orow) * nr + cb + oc, g);
     __syncthreads();   // every warp is done with zs
     if (part < parts) {
 #pragma unroll
@@ -451,6 +454,7 @@ template <typename T>
 Err matvec_tasks(hss_s* h, const T* X, int64_t ldx, int nrhs, T* B, int64_t ldb, cudaStream_t s) {
   {
     std::lock_guard<std::mutex> lock(h->plan_mu);
+    HSS_TRY(h->take_timeout_word());
     if (!h->mv_tasks) {
       std::vector<MvDesc> descs;
       std::vector<int2> tasks;
@@ -468,6 +472,8 @@ Err matvec_tasks(hss_s* h, const T* X, int64_t ldx, int nrhs, T* B, int64_t ldb,
   g.ntasks = h->mv_ntasks;
   g.nch = (nrhs + nc - 1) / nc;
   g.nrhs = nrhs;
+  g.timeout = h->timeout;
+  g.limit = fault_wait_limit() > 0 ? fault_wait_limit() : MV_WAIT_LIMIT;
   g.X = X;
   g.B = B;
   g.ldx = ldx;

@@ -321,6 +321,7 @@ extern "C" hss_status hss_matvec(hss_t h, const void* X, int64_t ldx, int64_t nr
     h->err = "hss_matvec: the handle holds no complete compressed form";
     return HSS_ERR_STATE;
   }
+  if (h->timed_out("hss_matvec")) return HSS_ERR_TIMEOUT;
   if (nrhs == 0) return HSS_OK;
   cudaStream_t s = (cudaStream_t)stream;
   Err e = h->dtype == HSS_F64

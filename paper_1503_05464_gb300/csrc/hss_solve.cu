@@ -14,7 +14,7 @@
 // result for NC right-hand sides, claimed in dependence order from a ticket
 // counter, each polling the values it needs (the work buffer starts as
 // all-ones NaNs; a poll is bounded, and on a timeout the NaN reaches the
-// solution).  Triangular systems go by blocks of 32 rows: a task subtracts
+// solution and the handle's next call reports it).  Triangular systems go by blocks of 32 rows: a task subtracts
 // the rows of L it needs and multiplies by the inverse of its diagonal block
 // (hss_factor leaves these, hss_ulv.cu; an ill-conditioned block is left as it
 // is, and the task substitutes), so the chain is one task per 32 rows.
@@ -104,6 +104,7 @@ struct SvJob {
   double* buf;
   const void* B;
   void* X;
+  unsigned* timeout;   // the handle's word for a poll that has run out
   int64_t ldb, ldx;
   int32_t nrhs, pad;
 };
@@ -114,6 +115,7 @@ struct SvArgs {
   const SvJob* jobs;   // several jobs
   const int4* list;    // ... (job, description, r0, column chunk)
   unsigned* ctl;       // [0] ticket, [1] a poll has timed out
+  long long limit;     // of a poll, in clock cycles
   unsigned total;
   int nch;
 };
@@ -126,16 +128,20 @@ __device__ __forceinline__ double sv_ld(const double* p) {
 __device__ __forceinline__ bool sv_unset(double v) { return __double_as_longlong(v) == -1ll; }
 
 // *p once it has been written (bounded; the flag ends the other polls early)
-__device__ __forceinline__ double sv_poll(const double* p, unsigned* stop) {
+__device__ __forceinline__ double sv_poll(const double* p, const SvArgs& g, const SvJob& jb) {
   double v = sv_ld(p);
   if (!sv_unset(v)) return v;
   const long long t0 = clock64();
   unsigned polls = 0;
   while (sv_unset(v = sv_ld(p))) {
     if ((++polls & 31u) != 0u) continue;
-    if (*reinterpret_cast<volatile unsigned*>(stop)) break;
-    if (clock64() - t0 > SV_WAIT_LIMIT) {
-      atomicExch(stop, 1u);
+    bool out = *reinterpret_cast<volatile unsigned*>(g.ctl + 1) != 0;
+    if (!out && clock64() - t0 > g.limit) {
+      atomicExch(g.ctl + 1, 1u);
+      out = true;
+    }
+    if (out) {   // (the other jobs' polls end early as well: each marks its own)
+      *reinterpret_cast<volatile unsigned*>(jb.timeout) = 1u;
       break;
     }
   }
@@ -248,7 +254,6 @@ __global__ void __launch_bounds__(SV_THREADS, NC == 4 ? 5 : 6) ulv_solve_kernel(
   __shared__ unsigned snext;
   constexpr int EO = SV_ROWS * NC > SV_THREADS ? SV_ROWS * NC / SV_THREADS : 1;   // outputs per thread
   const int tid = threadIdx.x, lane = tid & 31;
-  unsigned* stop = g.ctl + 1;
   unsigned claim = 0;
   if (tid == 0) snext = atomicAdd(g.ctl, 1u);
   if (!BATCH && tid == 0) jb = g.job;
@@ -361,18 +366,18 @@ __global__ void __launch_bounds__(SV_THREADS, NC == 4 ? 5 : 6) ulv_solve_kernel(
         if (!ahead) {
           // one lane of each warp polls until its value is there, then every
           // value is read
-          if (lane == 0 && p[0]) sv_poll(p[0], stop);
+          if (lane == 0 && p[0]) sv_poll(p[0], g, jb);
           __syncwarp();
 #pragma unroll
           for (int u = 0; u < U; ++u) v[u] = p[u] ? sv_ld(p[u]) : 0.0;
         }
         if (__any_sync(0xffffffffu, p[0] && sv_unset(v[0]))) {
-          if (lane == 0 && p[0]) sv_poll(p[0], stop);
+          if (lane == 0 && p[0]) sv_poll(p[0], g, jb);
           __syncwarp();
         }
 #pragma unroll
         for (int u = 0; u < U; ++u)
-          if (p[u] && sv_unset(v[u])) v[u] = sv_poll(p[u], stop);
+          if (p[u] && sv_unset(v[u])) v[u] = sv_poll(p[u], g, jb);
       }
       double* z = zs + (k & 1) * SV_LMAX * NC;
 #pragma unroll
@@ -413,7 +418,7 @@ __global__ void __launch_bounds__(SV_THREADS, NC == 4 ? 5 : 6) ulv_solve_kernel(
       if (tk.flags & SD_XINPUT) xv[o] = (double)Bin[(tk.x0 + xr[o]) * jb.ldb + c];
       else
         xv[o] = sv_poll(buf + (xr[o] < tk.xsplit ? tk.x0 + xr[o] : tk.x1 + (xr[o] - tk.xsplit)) * nrow_b +
-                            cb + c, stop);
+                            cb + c, g, jb);
     }
     __syncthreads();   // every warp is done with zs
     {
@@ -760,6 +765,7 @@ struct SolveJob {
 Err sv_plan(hss_s* h) {
   std::lock_guard<std::mutex> lock(h->plan_mu);
   UlvFactors& F = h->ulv;
+  HSS_TRY(h->take_timeout_word());
   if (F.plan) return ok();
   SvPlan pl;
   sv_build(h, pl);
@@ -791,6 +797,7 @@ Err solve_slab(const std::vector<SolveJob*>& jobs, int c0, int width, cudaStream
     q.ldb = j->ldb;
     q.ldx = j->ldx;
     q.nrhs = nr;
+    q.timeout = j->h->timeout;
     js.push_back(q);
     fs.push_back(&F);
     off.push_back(rows);
@@ -843,6 +850,7 @@ Err solve_slab(const std::vector<SolveJob*>& jobs, int c0, int width, cudaStream
   SvArgs g{};
   g.ctl = reinterpret_cast<unsigned*>(mem);
   g.total = (unsigned)total;
+  g.limit = fault_wait_limit() > 0 ? fault_wait_limit() : SV_WAIT_LIMIT;
   if (cudaMemsetAsync(mem, 0, 256, s) != cudaSuccess ||
       cudaMemsetAsync(buf, 0xff, rows * sizeof(double), s) != cudaSuccess) {
     cudaGetLastError();
@@ -931,6 +939,7 @@ hss_status check_solve(hss_s* h, const void* B, int64_t ldb, int64_t nrhs, const
     h->err = "hss_solve: bad B, X, nrhs or leading dimension";
     return HSS_ERR_INVALID;
   }
+  if (h->timed_out("hss_solve")) return HSS_ERR_TIMEOUT;
   return HSS_OK;
 }
 

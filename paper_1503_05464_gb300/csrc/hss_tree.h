@@ -151,6 +151,19 @@ struct hss_s {
   size_t mv_off = 0;
   int mv_ntasks = 0;
   int64_t mv_rows = 0;
+  // set by a product or solve one of whose polls has run out (its result then
+  // holds NaN); taken with the first table, reported by the next call
+  unsigned* timeout = nullptr;
+  hss::Err take_timeout_word() { return timeout ? hss::ok() : hss::host_word_get(&timeout); }
+  // true once after such a call has finished
+  bool timed_out(const char* what) {
+    volatile unsigned* w = timeout;
+    if (!w || !*w) return false;
+    *w = 0;
+    err = std::string(what) + ": a wait of an earlier product or solve with this handle gave up; "
+                              "its result holds NaN";
+    return true;
+  }
   // The caller's stream may be gone by now: drain the device, then free on
   // the legacy stream.
   ~hss_s() {
@@ -160,5 +173,6 @@ struct hss_s {
     hss::dfree(mv_tasks, nullptr);
     store.release(nullptr);
     cudaDeviceSynchronize();
+    hss::host_word_put(timeout);
   }
 };

@@ -369,8 +369,8 @@ def hss_kernel_launches() -> int:
 
 def hss_set_fault(kind: int, value: int = 0) -> None:
     """Arm an injected fault (HSS_FAULT_OOM: the value-th allocation from now
-    fails; HSS_FAULT_WAIT_LIMIT: the ID's group barrier gives up after value
-    cycles) or clear them (HSS_FAULT_NONE)."""
+    fails; HSS_FAULT_WAIT_LIMIT: the ID's group barrier and the polls of the
+    product and the solve give up after value cycles) or clear them (HSS_FAULT_NONE)."""
     _check(load().hss_set_fault(kind, value))
 
 

@@ -125,3 +125,47 @@ def test_solve_takes_fewer_columns_where_memory_is_short(P):
     torch.cuda.synchronize()
     assert H.hss_pool_bytes()[0] == used
     assert torch.equal(P.hss_solve(h, B), ref)
+
+
+def test_product_and_solve_report_a_wait_that_gave_up(P):
+    """The polls' limit forced down: the kernels finish, the result holds NaN,
+    the next call with the handle says so, once, and the handle goes on."""
+    H = P.hss
+    import workloads as W
+    n = 4000          # a tree of eight levels: the last tasks wait for the whole chain
+    A = W.toeplitz_inv_distance(n, dtype=np.float64, device=DEV)
+    h, g = (P.hss_compress(A, leaf_size=16) for _ in range(2))
+    for x in (h, g):
+        P.hss_factor(x)
+    B = torch.randn(n, 3, dtype=torch.float64, device=DEV)
+    Y, X = P.hss_matvec(h, B), P.hss_solve(h, B)
+    P.hss_solve(g, B)
+
+    def reported(call):
+        with pytest.raises(P.HssError) as e:
+            call()
+        assert e.value.status == H.HSS_ERR_TIMEOUT
+
+    def short(call):
+        H.hss_set_fault(H.HSS_FAULT_WAIT_LIMIT, 16)
+        try:
+            out = call()
+            torch.cuda.synchronize()
+            return out
+        finally:
+            H.hss_set_fault(H.HSS_FAULT_NONE)
+
+    assert bool(torch.isnan(short(lambda: P.hss_matvec(h, B))).any())
+    ptr = H.ctypes.c_void_p(B.data_ptr())          # no columns: asks only
+    ask = [H.load().hss_matvec(h.handle, ptr, 3, 0, ptr, 3, None) for _ in range(2)]
+    assert ask == [H.HSS_ERR_TIMEOUT, H.HSS_OK]
+    assert torch.equal(P.hss_matvec(h, B), Y)
+    assert bool(torch.isnan(short(lambda: P.hss_solve(h, B))).any())
+    reported(lambda: P.hss_solve(h, B))
+    assert torch.equal(P.hss_solve(h, B), X)
+    out, st = short(lambda: P.hss_solve_batched([h, g], [B, B]))
+    assert st == [0, 0] and bool(torch.isnan(torch.cat(out)).any())
+    _, st = P.hss_solve_batched([h, g], [B, B])
+    assert H.HSS_ERR_TIMEOUT in st and set(st) <= {0, H.HSS_ERR_TIMEOUT}
+    out, st = P.hss_solve_batched([h, g], [B, B])
+    assert st == [0, 0] and torch.equal(out[0], X) and torch.equal(out[1], X)
