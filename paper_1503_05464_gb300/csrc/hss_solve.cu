@@ -446,31 +446,32 @@ __global__ void __launch_bounds__(SV_THREADS, NC == 4 ? 5 : 6) ulv_solve_kernel(
       __syncthreads();
       const bool up = (tk.flags & SD_POST_UPPER) != 0;
       const double kind = ps[up ? (SV_ROWS - 1) * (SV_ROWS + 1) : SV_ROWS - 1];
-      const bool subst = kind != 0.0;   // the block, not its inverse
-      if (subst) {
+      if (kind == 0.0) {
+#pragma unroll
+        for (int o = 0; o < EO; ++o) {
+          const int e = tid + o * SV_THREADS, r = e / NC, c = e - r * NC;
+          if (r >= rows) continue;
+          double s[4] = {0.0, 0.0, 0.0, 0.0};
+          const double* p = ps + r * (SV_ROWS + 1);
+          // (the zeros of a triangular block are left out four at a time)
+          int l = up ? r & ~3 : 0;
+          const int end = tk.flags & SD_POST_LOWER ? min(rows, (r & ~3) + 4) : rows;
+          for (; l + 3 < end; l += 4)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) s[q] = fma(p[l + q], ms[(l + q) * NC + c], s[q]);
+#pragma unroll
+          for (int q = 0; q < 3; ++q)
+            if (l + q < end) s[q] = fma(p[l + q], ms[(l + q) * NC + c], s[q]);
+          val[o] = (s[0] + s[1]) + (s[2] + s[3]);
+        }
+      } else {   // the block, not its inverse
         sv_substitute<NC>(ms, ps, rows, up, kind == 1.0);
         __syncthreads();
-      }
 #pragma unroll
-      for (int o = 0; o < EO; ++o) {
-        const int e = tid + o * SV_THREADS, r = e / NC, c = e - r * NC;
-        if (r >= rows) continue;
-        if (subst) {
-          val[o] = ms[e];
-          continue;
+        for (int o = 0; o < EO; ++o) {
+          const int e = tid + o * SV_THREADS;
+          if (e < rows * NC) val[o] = ms[e];
         }
-        double s[4] = {0.0, 0.0, 0.0, 0.0};
-        const double* p = ps + r * (SV_ROWS + 1);
-        // (the zeros of a triangular block are left out four at a time)
-        int l = tk.flags & SD_POST_UPPER ? r & ~3 : 0;
-        const int end = tk.flags & SD_POST_LOWER ? min(rows, (r & ~3) + 4) : rows;
-        for (; l + 3 < end; l += 4)
-#pragma unroll
-          for (int q = 0; q < 4; ++q) s[q] = fma(p[l + q], ms[(l + q) * NC + c], s[q]);
-#pragma unroll
-        for (int q = 0; q < 3; ++q)
-          if (l + q < end) s[q] = fma(p[l + q], ms[(l + q) * NC + c], s[q]);
-        val[o] = (s[0] + s[1]) + (s[2] + s[3]);
       }
     }
 #pragma unroll
