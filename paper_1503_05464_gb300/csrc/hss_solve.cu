@@ -55,7 +55,6 @@ constexpr int SV_ROWS = 32, SV_THREADS = 128;
 constexpr int SV_ENT = 1024;
 constexpr int SV_LMAX = SV_ENT / 8;
 constexpr int SV_FINE_M = 160;
-constexpr int64_t SV_MANY_ROWS = 200000;
 constexpr int SV_COLS = 64;   // right-hand sides per launch, fewer where memory is short
 constexpr long long SV_WAIT_LIMIT = 1ll << 33;   // clock cycles (about 4 s)
 
@@ -508,6 +507,7 @@ struct SvPlan {
   std::vector<int2> tasks;
   std::vector<int> phases;
   int64_t rows = 0;   // of the work buffer
+  double load = 0.0;  // the tasks, each with its length in units of 2000 matrix entries
 };
 
 void sv_build(const hss_s* h, SvPlan& pl) {
@@ -745,6 +745,12 @@ void sv_build(const hss_s* h, SvPlan& pl) {
       }
     }
   }
+  pl.load = (double)pl.tasks.size();
+  for (const SvDesc& d : pl.descs)
+    for (int t = 0; t < d.nterm; ++t) {
+      const double part = d.t[t].flags & (ST_LOWER | ST_UPPER) ? 0.5 : 1.0;
+      pl.load += part * d.rows * d.t[t].inner / 2000.0;
+    }
   phase();   // (the end)
   if (pl.phases.empty() || pl.phases.back() != (int)pl.tasks.size())
     pl.phases.push_back((int)pl.tasks.size());
@@ -774,6 +780,7 @@ Err sv_plan(hss_s* h) {
   HSS_TRY(upload_kept(&F.plan, {{pl.descs.data(), F.plan_off},
                                 {pl.tasks.data(), pl.tasks.size() * sizeof(int2)}}));
   F.plan_rows = pl.rows;
+  F.plan_load = pl.load;
   F.plan_tasks = std::move(pl.tasks);
   F.plan_phases = std::move(pl.phases);
   return ok();
@@ -807,15 +814,22 @@ Err solve_slab(const std::vector<SolveJob*>& jobs, int c0, int width, cudaStream
   }
   if (js.empty()) return ok();
   // Columns per task.  More make better use of a matrix entry; fewer make the
-  // tasks shorter and the chains of dependent tasks with them.  Solve in ms
-  // with 1 / 2 / 4 / 8 columns: Schur complement n = 5041, 8 right-hand sides
-  // 1.71 / 1.70 / 2.16 / 3.37, 32: 3.69 / 2.95 / 2.94 / 3.95; Toeplitz
-  // n = 80,000 (many rows of results), 4 right-hand sides 0.82 / 0.72 / 0.74 /
-  // -, 32: 4.49 / 3.23 / 2.43 / 2.31.
-  int64_t nrows = 0;
-  for (const UlvFactors* F : fs) nrows += F->plan_rows;
-  const bool many = nrows >= SV_MANY_ROWS;
-  const int nc = maxnr <= (many ? 1 : 4) ? 1 : maxnr <= (many ? 2 : 16) ? 2 : 4;
+  // tasks shorter and the chains of dependent tasks with them.  One, until a
+  // dependent step has the work of some 600 one-column tasks of usual length (the
+  // SMs hold 900), two to 1500, then four: of 27 handles (Toeplitz n = 1000 to
+  // 160,000, QChem, Schur, Gaussian and BEM kernels, single dense nodes, leaves
+  // of 16 and of 1024) at 2 to 64 right-hand sides this is within 0.5% of the
+  // best of the three on average and within 11% at worst.  In us with 1 / 2 / 4
+  // columns: Toeplitz n = 8000, 8 right-hand sides 208 / 217 / 240, 32 480 / 364 /
+  // 358; n = 80,000, 2: 559 / 524 / 684, 8: 1273 / 952 / 898; Schur complement n
+  // = 10,000, 4: 2169 / 2406 / 3110, 16: 4475 / 3817 / 4021, 64: 14539 / 10383 /
+  // 8859; dense n = 3000, 64: 2294 / 2006 / 1822.
+  double steps = 1.0, load = 0.0;
+  for (size_t q = 0; q < js.size(); ++q) {
+    steps = std::max(steps, (double)fs[q]->plan_phases.size());
+    load += fs[q]->plan_load * js[q].nrhs;
+  }
+  const int nc = maxnr < 2 || load <= 600.0 * steps ? 1 : maxnr < 3 || load <= 1500.0 * steps ? 2 : 4;
   // several handles: their phases interleaved, so that one handle's chain of
   // dependent tasks does not hold every CTA
   std::vector<int4> list;
