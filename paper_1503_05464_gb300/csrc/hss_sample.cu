@@ -1,18 +1,17 @@
 // Fused sampling S^r = (A - D) R, S^c = (A - D)^T R (Section 2.2, step 2 of
 // the compression; Algorithm 1's leaf samples S^r(I,:) - D R(I,:)).
 //
-// One pass over A serves both products: a CTA owns a panel of BM rows and a
-// chunk of DC sample columns and walks every column tile of A once.  The row
-// sample of its panel is complete when the walk ends (accumulated on chip);
-// the column sample of each tile is a partial sum over the panel's rows and is
-// written to a slab of partial sums, which a second kernel reduces over the
-// panels in a fixed order (deterministic: no floating-point atomics).
-// Entries with leaf(i) == leaf(j) are masked to zero while A is staged, which
-// subtracts the leaf diagonal blocks D exactly (no cancellation).  In FP32 the
-// row sample is summed per column tile and the tile sums are added with Kahan
-// compensation; the panel partials of the column sample are summed with
-// compensation too: the sample error stays near one rounding instead of
-// growing like sqrt(n).
+// One pass over A serves both products: the (128-row panel, column tile) pairs
+// of a chunk of DC sample columns are dealt evenly over the CTAs, and a CTA walks
+// its range.  Its part of a panel's row sample (accumulated on chip) and the
+// column sample of each tile, a partial sum over the panel's rows, go to two
+// slabs, which a second kernel reduces in a fixed order (deterministic: no
+// floating-point atomics).  Entries with leaf(i) == leaf(j) are masked to zero
+// while A is staged, which subtracts the leaf diagonal blocks D exactly (no
+// cancellation).  In FP32 the row sample is summed per 32 columns and these sums
+// are added with Kahan compensation, whose remainder goes to the slab as well;
+// the partials of both samples are summed with compensation: the sample error
+// stays near one rounding instead of growing like sqrt(n).
 #include "hss_internal.cuh"
 
 #include <algorithm>

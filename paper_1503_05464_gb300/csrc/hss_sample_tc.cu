@@ -37,7 +37,8 @@
 //                the bfloat16 planes or round to TF32 (double-buffered,
 //                swizzled operand layout); two warps per scheduler keep the
 //                ALUs fed;
-//   warp 1       MMA issuer (one thread): tcgen05.mma into TMEM;
+//   warp 1       MMA issuer (an elected lane of a warp that walks the tiles with
+//                uniform values): tcgen05.mma into TMEM;
 //   warps 10-13  column drain: the column product of each tile (TMEM, three
 //                buffers) is summed over the panel pair through distributed
 //                shared memory: each CTA sends its partner the half of the 64
@@ -57,9 +58,10 @@
 // What bounds it: the hand-offs.  At n = 20000 and 128 columns a tile takes
 // 3800 cycles, of which the tensor pipe is busy 1540, shared memory about 2400
 // (operands, planes, stages, exchange) and HBM 2300 (A, and 1 GB of slabs).
-// The call took 1.33 ms and takes 0.88: an issuing warp with uniform operands
-// (1.24 -> 1.00), places stepped instead of divided out (1.30 -> 1.19), the
-// slab and the exchange by bulk copies, the reduction's rows (0.96 -> 0.88).
+// The call (without a leaf mask) took 1.33 ms and takes 0.87: an issuing warp
+// with uniform operands (1.24 -> 1.00), places stepped instead of divided out
+// (1.30 -> 1.19), the slab and the exchange by bulk copies, the reduction's rows
+// (0.96 -> 0.88).  With the mask of 256-row leaves 0.90.
 // TMEM columns: [0,128) the row accumulator, [128,256) the running row sum,
 // [256,448) three column accumulators, [448,512) R_p^T, the column
 // product's A operand (TF32: two column accumulators in [256,384) and R_p^T,

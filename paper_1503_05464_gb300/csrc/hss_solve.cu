@@ -31,9 +31,9 @@
 // What bounds it: at one column the chain of dependent tasks (about 4 us per
 // 32-row block of a triangular system, 10 us per panel of Q at m = 600), at
 // many columns FP64 work at about half its rate.  Measured (GB300, whole call,
-// before -> after): Toeplitz n = 80,000, FP64, 1 / 16 columns 1.80 -> 0.43,
-// 4.6 -> 1.3 ms; Schur complement n = 5041, FP32, 1 / 32 columns 4.8 -> 0.87,
-// 9.9 -> 2.2 ms; n = 10,000, 64 columns 82 -> 8.8 ms.
+// against one launch per tree level and operation): Toeplitz n = 80,000, FP64, 1
+// / 16 columns 1.80 -> 0.45, 4.6 -> 1.34 ms; Schur complement n = 5041, FP32, 1 /
+// 32 columns 4.8 -> 0.90, 9.9 -> 2.26 ms; n = 10,000, 64 columns 82 -> 8.9 ms.
 #include "hss_internal.cuh"
 #include "hss_tree.h"
 
