@@ -3,6 +3,7 @@
 
 #include "hss_internal.cuh"
 
+#include <atomic>
 #include <mutex>
 
 struct hss_s;
@@ -154,8 +155,14 @@ struct hss_s {
   int64_t mv_rows = 0;
   // set by a product or solve one of whose polls has run out (its result then
   // holds NaN); taken with the first table, reported by the next call
-  unsigned* timeout = nullptr;
-  hss::Err take_timeout_word() { return timeout ? hss::ok() : hss::host_word_get(&timeout); }
+  std::atomic<unsigned*> timeout{nullptr};
+  hss::Err take_timeout_word() {   // (under plan_mu)
+    unsigned* w = timeout;
+    if (w) return hss::ok();
+    const hss::Err e = hss::host_word_get(&w);
+    if (e.st == HSS_OK) timeout = w;
+    return e;
+  }
   // true once after such a call has finished
   bool timed_out(const char* what) {
     volatile unsigned* w = timeout;
