@@ -465,3 +465,16 @@ def test_matvec_of_one_dense_node(P, dtype, n):
         x = X[:, :k].contiguous()
         y = P.hss_matvec(h, x)
         assert torch.equal(y, full[:, :k]) and torch.equal(P.hss_matvec(h, x), y)
+
+
+# the root's interchanges fit shared memory up to 2112 rows
+@pytest.mark.parametrize("n", [2112, 2113])
+def test_root_interchanges_on_both_sides_of_shared_memory(P, n):
+    g = torch.Generator(device=DEV).manual_seed(n)
+    A = torch.randn(n, n, generator=g, device=DEV, dtype=torch.float64)
+    h = P.hss_compress(A, leaf_size=n)
+    P.hss_factor(h)
+    b = torch.randn(n, 2, generator=g, device=DEV, dtype=torch.float64)
+    x = P.hss_solve(h, b)
+    # partial pivoting: growth below 50 on random matrices, n u each
+    assert float((A @ x - b).norm()) <= 50 * n * 2.0 ** -53 * float(A.norm()) * float(x.norm())
