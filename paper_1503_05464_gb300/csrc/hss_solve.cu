@@ -507,7 +507,7 @@ struct SvPlan {
   std::vector<int2> tasks;
   std::vector<int> phases;
   int64_t rows = 0;   // of the work buffer
-  double load = 0.0;  // the tasks, each with its length in units of 2000 matrix entries
+  double entries = 0.0;   // matrix entries that the tasks multiply by
 };
 
 void sv_build(const hss_s* h, SvPlan& pl) {
@@ -745,11 +745,10 @@ void sv_build(const hss_s* h, SvPlan& pl) {
       }
     }
   }
-  pl.load = (double)pl.tasks.size();
   for (const SvDesc& d : pl.descs)
     for (int t = 0; t < d.nterm; ++t) {
       const double part = d.t[t].flags & (ST_LOWER | ST_UPPER) ? 0.5 : 1.0;
-      pl.load += part * d.rows * d.t[t].inner / 2000.0;
+      pl.entries += part * d.rows * d.t[t].inner;
     }
   phase();   // (the end)
   if (pl.phases.empty() || pl.phases.back() != (int)pl.tasks.size())
@@ -780,7 +779,7 @@ Err sv_plan(hss_s* h) {
   HSS_TRY(upload_kept(&F.plan, {{pl.descs.data(), F.plan_off},
                                 {pl.tasks.data(), pl.tasks.size() * sizeof(int2)}}));
   F.plan_rows = pl.rows;
-  F.plan_load = pl.load;
+  F.plan_entries = pl.entries;
   F.plan_tasks = std::move(pl.tasks);
   F.plan_phases = std::move(pl.phases);
   return ok();
@@ -814,22 +813,33 @@ Err solve_slab(const std::vector<SolveJob*>& jobs, int c0, int width, cudaStream
   }
   if (js.empty()) return ok();
   // Columns per task.  More make better use of a matrix entry; fewer make the
-  // tasks shorter and the chains of dependent tasks with them.  One, until a
-  // dependent step has the work of some 600 one-column tasks of usual length (the
-  // SMs hold 900), two to 1500, then four: of 27 handles (Toeplitz n = 1000 to
-  // 160,000, QChem, Schur, Gaussian and BEM kernels, single dense nodes, leaves
-  // of 16 and of 1024) at 2 to 64 right-hand sides this is within 0.5% of the
-  // best of the three on average and within 11% at worst.  In us with 1 / 2 / 4
-  // columns: Toeplitz n = 8000, 8 right-hand sides 208 / 217 / 240, 32 480 / 364 /
-  // 358; n = 80,000, 2: 559 / 524 / 684, 8: 1273 / 952 / 898; Schur complement n
-  // = 10,000, 4: 2169 / 2406 / 3110, 16: 4475 / 3817 / 4021, 64: 14539 / 10383 /
-  // 8859; dense n = 3000, 64: 2294 / 2006 / 1822.
-  double steps = 1.0, load = 0.0;
+  // tasks shorter and the chains of dependent tasks with them.  So it follows
+  // from the tasks that stand side by side: one column until a phase has 250 to
+  // 550 one-column tasks on average (the SMs hold 900; the longer the tasks, the
+  // more), two until 700 to 1900, then four.  Deep trees and single nodes, with
+  // few tasks a phase, go by the columns alone.  Measured on 113 handles
+  // (Toeplitz n = 315 to 160,000, QChem, Schur, Gaussian, BEM and random ones,
+  // combs, dense nodes, leaves of 16 to 1000, both dtypes) at 2 to 64 right-hand
+  // sides: 1.6% above the best of the three on average (a line at a size of the
+  // work buffer, 4.4%).  In us with 1 / 2 / 4 columns: Toeplitz n = 8000, 8
+  // right-hand sides 208 / 217 / 240, 32 480 / 364 / 358; n = 80,000, 2: 559 / 524 /
+  // 684, 8: 1273 / 952 / 898; Schur complement n = 10,000, 4: 2169 / 2406 / 3110, 16:
+  // 4475 / 3817 / 4021, 64: 14539 / 10383 / 8859; dense n = 3000, 64: 2294 / 2006 /
+  // 1822; leaves of 16, n = 1376, 32: 258 / 185 / 164.
+  double phases = 1.0, tasks = 0.0, entries = 0.0, side = 0.0;
   for (size_t q = 0; q < js.size(); ++q) {
-    steps = std::max(steps, (double)fs[q]->plan_phases.size());
-    load += fs[q]->plan_load * js[q].nrhs;
+    phases = std::max(phases, (double)fs[q]->plan_phases.size() - 1.0);
+    tasks += (double)fs[q]->plan_tasks.size();
+    side += (double)fs[q]->plan_tasks.size() * js[q].nrhs;
+    entries += fs[q]->plan_entries;
   }
-  const int nc = maxnr < 2 || load <= 600.0 * steps ? 1 : maxnr < 3 || load <= 1500.0 * steps ? 2 : 4;
+  side /= phases;
+  const double len = std::min(entries / std::max(tasks, 1.0), 2000.0);   // entries per task
+  int nc = 4;
+  if (maxnr < 2) nc = 1;
+  else if (tasks < 6.0 * phases) nc = maxnr <= 4 ? 1 : maxnr <= 16 ? 2 : 4;
+  else if (side <= 250.0 + 0.15 * len) nc = 1;
+  else if (maxnr < 3 || side <= 700.0 + 0.6 * len) nc = 2;
   // several handles: their phases interleaved, so that one handle's chain of
   // dependent tasks does not hold every CTA
   std::vector<int4> list;

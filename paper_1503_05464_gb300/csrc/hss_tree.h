@@ -100,13 +100,14 @@ struct UlvFactors {
   size_t bytes = 0;
   // the solve's task table (hss_solve.cu), built at the first solve: the
   // descriptions and (at plan_off) the tasks on the device; the tasks and
-  // the phases they fall into; rows of a solve's work buffer; the tasks' work
+  // the phases they fall into; rows of a solve's work buffer; the matrix
+  // entries that the tasks multiply by
   void* plan = nullptr;
   size_t plan_off = 0;
   std::vector<int2> plan_tasks;
   std::vector<int> plan_phases;
   int64_t plan_rows = 0;
-  double plan_load = 0.0;
+  double plan_entries = 0.0;
   void release(cudaStream_t s) {
     dfree(block, s);
     block = nullptr;
