@@ -42,7 +42,7 @@ typedef enum {
   HSS_ERR_OOM = 2,       /* device allocation failed */
   HSS_ERR_CUDA = 3,      /* a CUDA call or kernel launch failed */
   HSS_ERR_RANK_CAP = 4,  /* adaptive sampling reached d_max before every node compressed */
-  HSS_ERR_SINGULAR = 5,  /* zero pivot in the root LU of the ULV factorization */
+  HSS_ERR_SINGULAR = 5,  /* no pivot (zeros or NaN) in a column of the ULV factorization's root LU */
   HSS_ERR_TIMEOUT = 6,   /* a device-side wait gave up after its iteration limit */
   HSS_ERR_STATE = 7      /* call out of order (e.g. hss_solve before hss_factor) */
 } hss_status;
@@ -189,8 +189,8 @@ hss_status hss_matvec(hss_t h, const void* X, int64_t ldx, int64_t nrhs,
 
 /*
  * hss_factor -- ULV-like factorization of the compressed form (Algorithm 3),
- * in FP64 whatever the handle's dtype.  Errors: SINGULAR (zero pivot in the
- * root LU), OOM, CUDA.  Synchronizes `stream`.
+ * in FP64 whatever the handle's dtype.  Errors: SINGULAR (a column of the
+ * root LU holds no pivot: zeros, or a NaN of the matrix), OOM, CUDA.  Synchronizes `stream`.
  */
 hss_status hss_factor(hss_t h, void* stream);
 

@@ -748,7 +748,7 @@ void factor_many(int count, hss_t* hs, cudaStream_t s, hss_status* st) {
   for (int q : live) {
     hss_s* h = hs[q];
     if (st[q] == HSS_OK && hst[q] != 0) {
-      h->err = "hss_factor: zero pivot in the root LU";
+      h->err = "hss_factor: no pivot (zeros or NaN) in a column of the root LU";
       st[q] = HSS_ERR_SINGULAR;
     }
     if (st[q] != HSS_OK) {
