@@ -464,7 +464,7 @@ __global__ void reduce_simt_kernel(const T* __restrict__ P, const T* __restrict_
     reduce_row_entry(PR, n, pl, c0, ncols, Sr, lds, t - nc);
 }
 
-// The SIMT path: scratch of simt_bytes
+// The SIMT path: scratch of sample_scratch_bytes
 template <typename T, int DC>
 Err launch_simt(const T* A, int64_t n, int64_t lda, const T* R, int64_t ldr, int64_t c0,
                 int64_t ncols, T* Sr, T* Sc, int64_t lds, const int32_t* leaf_of,
